@@ -158,7 +158,7 @@ def workload(name: str, scale: int):
 # sources the kernel compiles from; a figure is used only while they match
 PROFILES = {
     "small": ("bcreach_small_articulation.json", ("bcreach.cu", "bc_math.cuh")),
-    "wide": ("bcreach_wide_twins.json", ("wide.cu", "bc_math.cuh", "coop.cuh")),
+    "wide": ("bcreach_wide_twins.json", ("pull.cu", "bc_math.cuh", "coop.cuh")),
 }
 
 
@@ -268,7 +268,7 @@ def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
         rec = measured_traffic("wide")
         traffic = rec["dram_bytes_per_batch"] * st["n_wide_batches"] if rec and st["n_wide_batches"] else None
         return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": f"k_bcreach_wide (whole GPU on one {S}-source batch)",
+                "traffic": traffic, "kernel": "k_bcreach_pull (whole GPU on one BFS level of many sources)",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
                 "work": {"bytes": by, "f_dag": f_dag, "sources_x_entries": wse, "sources_x_vertices": wsv,
                          "batches": int(st["n_wide_batches"]), "ms": ms,

@@ -41,13 +41,12 @@
  *
  * Environment: BCS_TRACE (any value) prints per-stage timings to stderr;
  * BCS_LARGE_PATH=wide|batched|per_source|mid forces the kernel used for
- * pieces too large for shared memory (the whole GPU on one batch of 64
- * sources, 32 sources per CTA, one source per CTA, or one 64-source batch
- * per CTA for pieces of at most 65,536 vertices), which is otherwise chosen
- * from the pieces' sizes and count, their BFS depth, the number of sources
- * and the memory each kernel needs (or by the autotuner);
- * BCS_LARGE_PATH=wide_all|mid_all (for tests) sends every piece through the
- * whole-GPU kernel, or the one-batch-per-CTA kernel, where its depth allows.
+ * pieces too large for shared memory (the whole GPU on one BFS level of many
+ * sources, 32 sources per CTA, one source per CTA, or the first one on
+ * connected pieces of at most 65,536 vertices only), which is otherwise chosen
+ * from the pieces' BFS depth, the number of sources and the memory each kernel
+ * needs (or by the autotuner); BCS_LARGE_PATH=wide_all|mid_all (for tests)
+ * sends every piece through the first kernel where its depth allows.
  */
 #ifndef BCSHATTER_H
 #define BCSHATTER_H
@@ -153,9 +152,9 @@ typedef struct bcs_stats {
   int64_t small_ng_cap;    /* most sources one small-path CTA ran at once */
   int64_t small_smem_budget; /* shared-memory budget per small-path CTA (bytes) */
   int64_t n_side;          /* side vertices taken out of the pieces (BCS_STEP_S) */
-  int64_t n_wide_batches;  /* source batches (64, or 32) run with the whole GPU on
-                              one batch (large pieces of small BFS depth), or one
-                              per CTA on mid-size pieces (BCS_LARGE_PATH=mid) */
+  int64_t n_wide_batches;  /* batches of 64 sources run with the whole GPU on one
+                              BFS level of many of them (pieces of small BFS depth
+                              that do not fit shared memory) */
   int64_t n_rounds;        /* split-and-merge rounds of the preprocessing loop
                               (BCS_STEP_L) */
   int64_t small_limit;     /* shared memory (bytes) a piece may need for one source

@@ -51,18 +51,16 @@ constexpr int DISC_CH = 4;  // row entries per step of the shared-memory discove
 constexpr int LARGE_THREADS = 512;
 // BFS depth above which large pieces run one source per CTA rather than 32
 constexpr int MS_DEPTH_LIMIT = 64;
-// Large pieces with at least this many vertices and a BFS eccentricity (from
-// their first vertex) of at most WIDE_MAX_ECC run on the whole-GPU path
-constexpr int WIDE_MIN_N = 32768;
-constexpr int WIDE_MAX_ECC = 40;
-// Pieces of at most MID_MAX_N vertices that do not fit shared memory can run
-// one 64-source batch per CTA (BCS_LARGE_PATH=mid), by default only if
-// MID_BY_DEFAULT and they give at least MID_MIN_UNITS_PER_SM batches per SM.
-// Off: on the uneven batch of pieces up to 4,096 vertices it measured 3 %
-// slower than 32 sources per CTA (4.14 s against 4.04 s per call).
+// Large pieces whose BFS eccentricity (from their first vertex) is at most
+// PULL_MAX_ECC run on the pull kernel (pull.cu)
+constexpr int PULL_MAX_ECC = 40;
+// pieces of at most this many vertices are ordered one per CTA, larger ones
+// one after the other by the whole GPU
+constexpr int PIECE_BFS_MAX_N = 32768;
+// BCS_LARGE_PATH=mid: the pull kernel on connected pieces of at most this
+// many vertices and MID_MAX_ECC levels
 constexpr int MID_MAX_N = 65536;
-constexpr int64_t MID_MIN_UNITS_PER_SM = 8;
-constexpr bool MID_BY_DEFAULT = false;
+constexpr int MID_MAX_ECC = 30;
 
 struct SmallItem {
   int32_t comp;
@@ -107,7 +105,6 @@ struct CoefT<true> {
 
 // Reciprocals 1/k of the integers k < RECIP_TABLE (entry 0 unused), filled
 // once per device by IEEE division (correctly rounded).
-constexpr int RECIP_TABLE = 1024;
 static __device__ double g_recip_table[RECIP_TABLE];
 
 __global__ void k_fill_recip_table() {
@@ -695,6 +692,14 @@ static int recip_table_ready(int device) {
   return BCS_OK;
 }
 
+int recip_table(Ctx &ctx, const double **out) {
+  BCS_TRY(recip_table_ready(ctx.device));
+  void *p = nullptr;
+  BCS_CUDA(cudaGetSymbolAddress(&p, g_recip_table));
+  *out = (const double *)p;
+  return BCS_OK;
+}
+
 // CTAs of the shared-memory kernel that fit on one SM with `smem` bytes each
 template <bool R, bool I, bool F>
 static int small_ctas_per_sm(int device, size_t smem, int *out) {
@@ -837,7 +842,8 @@ static int tune_large_piece(Ctx &ctx, const CompDesc &c, const BcInput &in, cons
   };
   const int64_t ns = nsrc_of(c), sms = ctx.num_sms;
   std::vector<Cand> cands;
-  if (wide_ok) cands.push_back({LARGE_PATH_WIDE, 512});
+  // the pull kernel on about a wave of rows
+  if (wide_ok) cands.push_back({LARGE_PATH_WIDE, std::max<int64_t>(512, 64 * (((int64_t)1 << 21) / c.n))});
   if (depth <= 4 * MS_DEPTH_LIMIT) cands.push_back({LARGE_PATH_BATCHED, 32 * sms});
   cands.push_back({LARGE_PATH_PER_SOURCE, 6 * sms});
   *choice = cands[0].path;
@@ -1023,80 +1029,75 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     grid = (int)std::min<int64_t>(grid, (int64_t)out.size());
     return BCS_OK;
   };
-  // Large pieces of small BFS depth: the whole GPU on one 32-source batch at
-  // a time (wide.cu), the sources taken in the BFS order of the piece from
-  // its first vertex (neighbouring sources share most of their levels).  The
-  // BFS from that vertex also bounds the depth: no source reaches deeper than
-  // twice its eccentricity.  BCS_LARGE_PATH=wide takes every large piece
-  // whose depth allows it; batched|per_source take none.
-  struct WidePiece {
-    int32_t ci;
-    std::shared_ptr<DBuf<int32_t>> order;
-    int32_t nsrc;
-    int depth_bound;
-  };
-  std::vector<WidePiece> wide;
+  // Large pieces of small BFS depth: the pull kernel, the sources of a piece
+  // taken in the order of its BFS from its first vertex (neighbouring sources
+  // share most of their levels).  That search also bounds the depth: no source
+  // reaches deeper than twice its eccentricity.  BCS_LARGE_PATH=wide takes
+  // every large piece whose depth allows it, mid the connected ones of at most
+  // MID_MAX_N vertices; batched|per_source take none.
+  DBuf<CompDesc> d_comps;
+  if (!small.empty() || !large.empty()) {
+    BCS_TRY(d_comps.alloc(C, ctx.stream));
+    BCS_CUDA(cudaMemcpyAsync(d_comps.p, comps.data(), C * sizeof(CompDesc), cudaMemcpyHostToDevice, ctx.stream));
+  }
+  std::vector<PullJob> pull;
+  DBuf<int32_t> pull_order;
   // large pieces the autotuner gave to 32-source batches, or to one source per CTA
   std::vector<int32_t> ms_tuned, ps_tuned;
-  // Mid-size pieces (at most MID_MAX_N vertices, every vertex a source or
-  // one piece with a source list): one 64-source batch per CTA (wide.cu),
-  // when forced, or when they are many enough to keep every CTA busy.
-  std::vector<int32_t> mid;
-  if (!dbg && !po.per_source_large && !po.srcmap &&
-      (lp_mode == LARGE_PATH_MID || (lp_mode == LARGE_PATH_AUTO && MID_BY_DEFAULT))) {
-    std::vector<int32_t> rest;
-    int64_t units = 0;
-    for (int32_t ci : large) {
-      const CompDesc &c = comps[ci];
-      if (c.n <= MID_MAX_N && (c.src_off < 0 || po.sources)) {
-        mid.push_back(ci);
-        units += (nsrc_of(c) + 63) / 64;
-      } else {
-        rest.push_back(ci);
-      }
-    }
-    if (lp_mode == LARGE_PATH_MID || units >= MID_MIN_UNITS_PER_SM * (int64_t)ctx.num_sms) {
-      large.swap(rest);
-    } else {
-      mid.clear();
-    }
-  }
   {
-    const bool force_wide = lp_mode == LARGE_PATH_WIDE;
-    const bool no_wide = lp_mode == LARGE_PATH_BATCHED || lp_mode == LARGE_PATH_PER_SOURCE;
-    std::vector<int32_t> rest;
+    const bool force_wide = lp_mode == LARGE_PATH_WIDE, force_mid = lp_mode == LARGE_PATH_MID;
+    const bool none = lp_mode == LARGE_PATH_BATCHED || lp_mode == LARGE_PATH_PER_SOURCE || dbg || po.per_source_large;
+    std::vector<int32_t> rest, cand, by_cta;
+    std::vector<int64_t> off, cta_off;
+    int64_t total = 0;
     for (int32_t ci : large) {
       const CompDesc &c = comps[ci];
-      // tuning pays only over many sources
-      const bool tune_this = tune && c.src_off < 0 && nsrc_of(c) >= 24LL * ctx.num_sms;
-      const bool cand = !no_wide && !dbg && !po.per_source_large && (c.src_off < 0 || po.sources) &&
-                        (force_wide || tune_this || c.n >= WIDE_MIN_N);
-      if (!cand) {
+      if (none || (c.src_off >= 0 && !po.sources) || (force_mid && c.n > MID_MAX_N)) {
         rest.push_back(ci);
         continue;
       }
-      auto ord = std::make_shared<DBuf<int32_t>>();
-      BCS_TRY(ord->alloc(c.n, ctx.stream));
+      cand.push_back(ci);
+      off.push_back(total);
+      if (c.n <= PIECE_BFS_MAX_N) {
+        by_cta.push_back(ci);
+        cta_off.push_back(total);
+      }
+      total += std::max<int64_t>(c.n, nsrc_of(c));
+    }
+    if (!cand.empty()) BCS_TRY(pull_order.alloc(total, ctx.stream));
+    std::vector<int32_t> cta_depth, cta_reached;
+    BCS_TRY(piece_bfs(ctx, comps, d_comps.p, by_cta, in, cta_off, pull_order.p, &cta_depth, &cta_reached));
+    for (size_t k = 0, kc = 0; k < cand.size(); k++) {
+      const int32_t ci = cand[k];
+      const CompDesc &c = comps[ci];
+      int32_t *const ord = pull_order.p + off[k];
       int depth = 0;
       int64_t reached = 0;
-      BCS_TRY(bfs_queue(ctx, in.row + c.row_off, in.col, c.n, 0, ord->p, &depth, &reached));
-      if (reached != c.n && c.row_off == 0) {
+      if (c.n <= PIECE_BFS_MAX_N) {
+        depth = cta_depth[kc];
+        reached = cta_reached[kc++];
+      } else {
+        BCS_TRY(bfs_queue(ctx, in.row + c.row_off, in.col, c.n, 0, ord, &depth, &reached));
+      }
+      if (reached != c.n && c.row_off == 0 && !force_mid) {
         // a whole graph of several components (the plain calls; pieces are
         // connected): every component searched from its smallest vertex
         DevGraph g{c.n, c.nnz, in.row, in.col};
-        BCS_TRY(bfs_queue_components(ctx, g, ord->p, &depth));
+        BCS_TRY(bfs_queue_components(ctx, g, ord, &depth));
         reached = c.n;
       }
       // every source's BFS depth is at most twice its component's root's
       const int bound = 2 * depth + 2;
-      const bool wide_ok = bound <= wide_depth_limit() && reached == c.n;
+      const bool ok = bound <= pull_depth_limit() && reached == c.n && (!force_mid || depth <= MID_MAX_ECC);
+      // tuning pays only over many sources
+      const bool tune_this = tune && c.src_off < 0 && nsrc_of(c) >= 24LL * ctx.num_sms;
       int choice = LARGE_PATH_AUTO;
       if (tune_this) {
         const long long key = ((long long)(R * 2 + I) << 40) | (bits_of(c.n) << 24) |
                               (bits_of((double)c.nnz / c.n) << 16) | bits_of(depth);
         choice = tuned_in(g_tune_large, key);
         if (!choice) {
-          BCS_TRY(tune_large_piece(ctx, c, in, po, wide_ok, depth, ord->p, &choice));
+          BCS_TRY(tune_large_piece(ctx, c, in, po, ok, depth, ord, &choice));
           remember_in(g_tune_large, key, choice);
         }
         ctx.stats.tuned |= 1ll << choice;
@@ -1104,24 +1105,34 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         if (choice == LARGE_PATH_PER_SOURCE) ps_tuned.push_back(ci);
         if (choice != LARGE_PATH_WIDE) continue;
       }
-      const bool heuristic = !force_wide && choice == LARGE_PATH_AUTO;
-      if (!wide_ok || (heuristic && (depth > WIDE_MAX_ECC || c.n < WIDE_MIN_N))) {
+      bool take = ok;
+      if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) {
+        take = take && depth <= PULL_MAX_ECC;
+      }
+      const size_t state = pull_piece_bytes(c.n, c.nnz, bound);
+      if (take && state > ((size_t)1 << 30)) {  // its state has to fit
+        size_t free_b = 0, total_b = 0;
+        BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        take = state <= free_b / 4 * 3;
+      }
+      if (!take) {
         rest.push_back(ci);
         continue;
       }
-      int32_t ns = (int32_t)nsrc_of(c);
       if (po.sources) {  // the caller's sources, in the caller's order
         std::vector<int32_t> h(po.nsources);
         for (int64_t i = 0; i < po.nsources; i++) h[i] = (int32_t)po.sources[i];
-        BCS_TRY(ord->alloc(std::max<int64_t>(po.nsources, 1), ctx.stream));
-        BCS_CUDA(cudaMemcpyAsync(ord->p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
+        BCS_CUDA(cudaMemcpyAsync(ord, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
         BCS_CUDA(cudaStreamSynchronize(ctx.stream));
-        ns = (int32_t)po.nsources;
       }
-      wide.push_back(WidePiece{ci, ord, ns, bound});
+      pull.push_back(PullJob{ci, (int32_t)nsrc_of(c), bound, off[k]});
     }
     large.swap(rest);
   }
+  nmax_large = 0;  // of what is left for the kernels below
+  for (int32_t ci : large) nmax_large = std::max<int64_t>(nmax_large, comps[ci].n);
+  for (int32_t ci : ms_tuned) nmax_large = std::max<int64_t>(nmax_large, comps[ci].n);
+  for (int32_t ci : ps_tuned) nmax_large = std::max<int64_t>(nmax_large, comps[ci].n);
   // Large pieces: 32 sources per CTA when there are enough batches to give
   // every SM two of them and their scratch fits at least one CTA per SM,
   // else one source per CTA (more CTAs in flight).
@@ -1198,21 +1209,16 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   for (int32_t ci : large) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
   for (int32_t ci : ms_tuned) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
   for (int32_t ci : ps_tuned) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
-  for (int32_t ci : mid) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
-  for (const WidePiece &wp : wide) ctx.stats.n_large_sources += wp.nsrc;
+  for (const PullJob &j : pull) ctx.stats.n_large_sources += j.nsrc;
   ctx.stats.work_sources_entries = work_se;
   ctx.stats.work_sources_vertices = work_sv;
-  if (small.empty() && large.empty() && wide.empty() && ms_tuned.empty() && ps_tuned.empty() && mid.empty())
-    return BCS_OK;
+  if (small.empty() && large.empty() && pull.empty() && ms_tuned.empty() && ps_tuned.empty()) return BCS_OK;
 
-  DBuf<CompDesc> d_comps;
   DBuf<int> d_err;
   DBuf<unsigned long long> d_dag;
-  BCS_TRY(d_comps.alloc(C, ctx.stream));
   BCS_TRY(d_err.alloc(4, ctx.stream));
   BCS_TRY(d_dag.alloc(1, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(d_dag.p, 0, sizeof(unsigned long long), ctx.stream));
-  BCS_CUDA(cudaMemcpyAsync(d_comps.p, comps.data(), C * sizeof(CompDesc), cudaMemcpyHostToDevice, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), ctx.stream));
   DBuf<int64_t> d_srcs;
   if (po.sources && !items.empty()) {
@@ -1284,30 +1290,15 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     tm.stop_into(ctx, &ctx.stats.ms_bcreach_small);
     tr.mark("small");
   }
-  for (const WidePiece &wp : wide) {
+  if (!pull.empty()) {
     StageTimer tm(ctx.stream);
     tm.start();
-    BCS_TRY(run_wide(ctx, comps[wp.ci], in, F, wp.order->p, wp.nsrc, wp.depth_bound, d_err.p, d_dag.p));
+    int per_batch = 64;
+    if (const char *e = std::getenv("BCS_WIDE_SOURCES"))
+      if (lp_mode != LARGE_PATH_MID) per_batch = std::atoi(e) <= 32 ? 32 : 64;
+    BCS_TRY(run_pull(ctx, comps, pull, in, F, pull_order.p, d_comps.p, per_batch, d_err.p, d_dag.p));
     tm.stop_into(ctx, &ctx.stats.ms_bcreach_large);
-    tr.mark("wide");
-  }
-  if (!mid.empty()) {
-    StageTimer tm(ctx.stream);
-    tm.start();
-    DBuf<int32_t> d_ord;
-    if (po.sources) {  // one piece: its sources, as local ids
-      std::vector<int32_t> h(po.nsources);
-      for (int64_t i = 0; i < po.nsources; i++) h[i] = (int32_t)po.sources[i];
-      BCS_TRY(d_ord.alloc(std::max<int64_t>(po.nsources, 1), ctx.stream));
-      BCS_CUDA(cudaMemcpyAsync(d_ord.p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
-      BCS_CUDA(cudaStreamSynchronize(ctx.stream));
-    }
-    std::vector<int32_t> too_deep;
-    BCS_TRY(run_mid(ctx, comps, mid, in, F, po.sources ? d_ord.p : nullptr, d_comps.p, d_err.p, d_dag.p, &too_deep));
-    // pieces too deep for its levels (or not connected): one source per CTA
-    ps_tuned.insert(ps_tuned.end(), too_deep.begin(), too_deep.end());
-    tm.stop_into(ctx, &ctx.stats.ms_bcreach_large);
-    tr.mark("mid");
+    tr.mark("pull");
   }
   // one source per CTA over the given list; *d_lmax (optional) receives the
   // deepest BFS level any of them reached

@@ -273,6 +273,7 @@ struct BcInput {
   double *bcp = nullptr;          // accumulation target, indexed by vertex
 };
 
+// WIDE: the pull kernel; MID: the pull kernel on connected pieces of at most 65,536 vertices
 enum { LARGE_PATH_AUTO = 0, LARGE_PATH_WIDE = 1, LARGE_PATH_BATCHED = 2, LARGE_PATH_PER_SOURCE = 3, LARGE_PATH_MID = 4 };
 
 struct BcPlanOpts {
@@ -312,22 +313,31 @@ int run_ms(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<int32
 // descriptors; their vertex ranges index BcInput's arrays.
 int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps, const BcInput &in, const BcPlanOpts &po);
 
-// Bc-Reach over one large piece of small BFS depth with the whole GPU on one
-// 32-source batch at a time (wide.cu).  d_order: the piece's sources (local
-// ids, device), taken 32 at a time in this order.
-// depth_bound: no source of the piece reaches deeper (at most
-// wide_depth_limit()).
-int run_wide(Ctx &ctx, const CompDesc &c, const BcInput &in, bool fp32, const int32_t *d_order, int32_t nsrc,
-             int depth_bound, int *d_err, unsigned long long *d_dag);
-// deepest BFS level run_wide can index
-int wide_depth_limit();
-// Bc-Reach over the listed mid-size pieces (every vertex a source, or with
-// d_order the one piece's sources), one 64-source batch per CTA at a time
-// (wide.cu).  d_comps: the device copy of comps.  Pieces found too deep for
-// its level cap, or not connected, are left undone and listed in too_deep.
-int run_mid(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<int32_t> &pieces, const BcInput &in,
-            bool fp32, const int32_t *d_order, const CompDesc *d_comps, int *d_err, unsigned long long *d_dag,
-            std::vector<int32_t> *too_deep);
+// Bc-Reach on pieces of small BFS depth, the whole GPU on one level of many
+// sources at a time (pull.cu).  A job: a piece, its sources (local ids at
+// d_order[ord_off ..)) and a bound on their BFS depth (at most
+// pull_depth_limit()).  per_batch: 64 (or 32) sources, four of these to a slab.
+struct PullJob {
+  int32_t ci, nsrc;
+  int depth_bound;
+  int64_t ord_off;
+};
+int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<PullJob> &jobs, const BcInput &in,
+             bool fp32, const int32_t *d_order, const CompDesc *d_comps, int per_batch, int *d_err,
+             unsigned long long *d_dag);
+// device address of the reciprocals of the integers below RECIP_TABLE
+constexpr int RECIP_TABLE = 1024;
+int recip_table(Ctx &ctx, const double **out);
+// deepest BFS level run_pull can index
+int pull_depth_limit();
+// bytes of device state one slab of a piece takes, at most
+size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound);
+// BFS of each listed piece from its first vertex, one piece per CTA: the
+// vertices in the order reached at order[ord_off[i] ..), the deepest level and
+// the number reached (host results; synchronises)
+int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_comps, const std::vector<int32_t> &list,
+              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, std::vector<int32_t> *depth,
+              std::vector<int32_t> *reached);
 // BFS of a connected graph from `root` (rows at rp[v]..rp[v+1] of col):
 // queue_out[0..*reached) the vertices in the order the search reaches them,
 // *depth the deepest level (order.cu)
