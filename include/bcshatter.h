@@ -40,13 +40,14 @@
  * launch and a device-wide synchronisation).
  *
  * Environment: BCS_TRACE (any value) prints per-stage timings to stderr;
- * BCS_LARGE_PATH=wide|batched|per_source|mid forces the kernel used for
+ * BCS_LARGE_PATH=wide|batched|per_source|mid|deep forces the kernel used for
  * pieces too large for shared memory (the whole GPU on one BFS level of many
- * sources, 32 sources per CTA, one source per CTA, or the first one on
- * connected pieces of at most 65,536 vertices only), which is otherwise chosen
- * from the pieces' BFS depth, the number of sources and the memory each kernel
- * needs (or by the autotuner); BCS_LARGE_PATH=wide_all|mid_all (for tests)
- * sends every piece through the first kernel where its depth allows.
+ * sources, 32 sources per CTA, one source per CTA, the first one on connected
+ * pieces of at most 65,536 vertices only, or a thread per (source, vertex)
+ * pair), which is otherwise chosen from the pieces' BFS depth and degree, the
+ * number of sources and the memory each kernel needs (or by the autotuner);
+ * BCS_LARGE_PATH=wide_all|mid_all|deep_all (for tests) sends every piece
+ * through that kernel where its depth or degree allows.
  */
 #ifndef BCSHATTER_H
 #define BCSHATTER_H
@@ -162,7 +163,7 @@ typedef struct bcs_stats {
   int64_t tuned;           /* the autotuner's choices this call, as bits: 1 the
                               small/large threshold; 1 << k a large piece on
                               kernel k (1 whole-GPU, 2 32-source batches, 3 one
-                              source per CTA) */
+                              source per CTA, 5 a thread per pair) */
   double work_nm;          /* sum over pieces of n_c * m_c (m_c undirected) */
   double work_sources_entries; /* sum over processed sources of the piece's CSR entries */
   double work_sources_vertices; /* sum over processed sources of the piece's vertices */

@@ -54,9 +54,8 @@ constexpr int MS_DEPTH_LIMIT = 64;
 // Large pieces whose BFS eccentricity (from their first vertex) is at most
 // PULL_MAX_ECC run on the pull kernel (pull.cu)
 constexpr int PULL_MAX_ECC = 40;
-// pieces of at most this many vertices are ordered one per CTA, larger ones
-// one after the other by the whole GPU
-constexpr int PIECE_BFS_MAX_N = 32768;
+// and deeper ones than this, of small degree, on the deep kernel (deep.cu)
+constexpr int DEEP_MIN_ECC = 40;
 // BCS_LARGE_PATH=mid: the pull kernel on connected pieces of at most this
 // many vertices and MID_MAX_ECC levels
 constexpr int MID_MAX_N = 65536;
@@ -835,7 +834,7 @@ static int time_candidate(Ctx &ctx, const std::vector<CompDesc> &comps, const Bc
 // order from the piece's first vertex (d_ord) for the whole-GPU kernel,
 // consecutive ids for the others.
 static int tune_large_piece(Ctx &ctx, const CompDesc &c, const BcInput &in, const BcPlanOpts &po, bool wide_ok,
-                            int depth, const int32_t *d_ord, int *choice) {
+                            bool deep_ok, int depth, const int32_t *d_ord, int *choice) {
   struct Cand {
     int path;
     int64_t m;
@@ -845,6 +844,7 @@ static int tune_large_piece(Ctx &ctx, const CompDesc &c, const BcInput &in, cons
   // the pull kernel on about a wave of rows
   if (wide_ok) cands.push_back({LARGE_PATH_WIDE, std::max<int64_t>(512, 64 * (((int64_t)1 << 21) / c.n))});
   if (depth <= 4 * MS_DEPTH_LIMIT) cands.push_back({LARGE_PATH_BATCHED, 32 * sms});
+  if (deep_ok) cands.push_back({LARGE_PATH_DEEP, 24 * sms});
   cands.push_back({LARGE_PATH_PER_SOURCE, 6 * sms});
   *choice = cands[0].path;
   if (cands.size() == 1) return BCS_OK;
@@ -903,7 +903,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   int lp_mode = po.large_path;
   bool all_large = false;
   if (const char *e = std::getenv("BCS_LARGE_PATH")) {
-    if (!std::strcmp(e, "wide_all") || !std::strcmp(e, "mid_all")) all_large = true;
+    if (!std::strcmp(e, "wide_all") || !std::strcmp(e, "mid_all") || !std::strcmp(e, "deep_all")) all_large = true;
+    if (!std::strcmp(e, "deep") || !std::strcmp(e, "deep_all")) lp_mode = LARGE_PATH_DEEP;
     if (!std::strcmp(e, "mid_all")) lp_mode = LARGE_PATH_MID;
     if (!std::strcmp(e, "wide") || !std::strcmp(e, "wide_all")) lp_mode = LARGE_PATH_WIDE;
     if (!std::strcmp(e, "batched")) lp_mode = LARGE_PATH_BATCHED;
@@ -1041,14 +1042,21 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     BCS_CUDA(cudaMemcpyAsync(d_comps.p, comps.data(), C * sizeof(CompDesc), cudaMemcpyHostToDevice, ctx.stream));
   }
   std::vector<PullJob> pull;
-  DBuf<int32_t> pull_order;
+  // deep pieces of small degree: deep.cu (src_off: the caller's sources in pull_order, < 0: every vertex)
+  struct DeepJob {
+    int32_t ci, nsrc;
+    int depth_bound;
+    int64_t ord_off, src_off;
+  };
+  std::vector<DeepJob> deep;
+  DBuf<int32_t> pull_order, pull_parent;  // BFS orders and tree parents, a piece after the other
   // large pieces the autotuner gave to 32-source batches, or to one source per CTA
   std::vector<int32_t> ms_tuned, ps_tuned;
   {
     const bool force_wide = lp_mode == LARGE_PATH_WIDE, force_mid = lp_mode == LARGE_PATH_MID;
     const bool none = lp_mode == LARGE_PATH_BATCHED || lp_mode == LARGE_PATH_PER_SOURCE || dbg || po.per_source_large;
-    std::vector<int32_t> rest, cand, by_cta;
-    std::vector<int64_t> off, cta_off;
+    std::vector<int32_t> rest, cand;
+    std::vector<int64_t> off;
     int64_t total = 0;
     for (int32_t ci : large) {
       const CompDesc &c = comps[ci];
@@ -1058,37 +1066,38 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       }
       cand.push_back(ci);
       off.push_back(total);
-      if (c.n <= PIECE_BFS_MAX_N) {
-        by_cta.push_back(ci);
-        cta_off.push_back(total);
-      }
-      total += std::max<int64_t>(c.n, nsrc_of(c));
+      total += c.n + (po.sources ? po.nsources : 0);
     }
-    if (!cand.empty()) BCS_TRY(pull_order.alloc(total, ctx.stream));
+    if (!cand.empty()) {
+      BCS_TRY(pull_order.alloc(total, ctx.stream));
+      BCS_TRY(pull_parent.alloc(total, ctx.stream));
+    }
     std::vector<int32_t> cta_depth, cta_reached;
-    BCS_TRY(piece_bfs(ctx, comps, d_comps.p, by_cta, in, cta_off, pull_order.p, &cta_depth, &cta_reached));
-    for (size_t k = 0, kc = 0; k < cand.size(); k++) {
+    BCS_TRY(piece_bfs(ctx, comps, d_comps.p, cand, in, off, pull_order.p, pull_parent.p, &cta_depth, &cta_reached));
+    for (size_t k = 0; k < cand.size(); k++) {
       const int32_t ci = cand[k];
       const CompDesc &c = comps[ci];
       int32_t *const ord = pull_order.p + off[k];
-      int depth = 0;
-      int64_t reached = 0;
-      if (c.n <= PIECE_BFS_MAX_N) {
-        depth = cta_depth[kc];
-        reached = cta_reached[kc++];
-      } else {
-        BCS_TRY(bfs_queue(ctx, in.row + c.row_off, in.col, c.n, 0, ord, &depth, &reached));
-      }
+      int depth = cta_depth[k];
+      int64_t reached = cta_reached[k];
+      if (reached < 0)  // large and wide: the whole GPU
+        BCS_TRY(bfs_queue(ctx, in.row + c.row_off, in.col, c.n, 0, ord, pull_parent.p + off[k], &depth, &reached));
       if (reached != c.n && c.row_off == 0 && !force_mid) {
         // a whole graph of several components (the plain calls; pieces are
         // connected): every component searched from its smallest vertex
         DevGraph g{c.n, c.nnz, in.row, in.col};
-        BCS_TRY(bfs_queue_components(ctx, g, ord, &depth));
+        BCS_TRY(bfs_queue_components(ctx, g, ord, pull_parent.p + off[k], &depth));
         reached = c.n;
       }
       // every source's BFS depth is at most twice its component's root's
       const int bound = 2 * depth + 2;
       const bool ok = bound <= pull_depth_limit() && reached == c.n && (!force_mid || depth <= MID_MAX_ECC);
+      bool deep_ok = false;
+      if (reached == c.n && (lp_mode == LARGE_PATH_DEEP || (depth > DEEP_MIN_ECC && !force_wide && !force_mid))) {
+        size_t free_b = 0, total_b = 0;
+        BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        deep_ok = deep_takes(c, bound, free_b);
+      }
       // tuning pays only over many sources
       const bool tune_this = tune && c.src_off < 0 && nsrc_of(c) >= 24LL * ctx.num_sms;
       int choice = LARGE_PATH_AUTO;
@@ -1097,35 +1106,35 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
                               (bits_of((double)c.nnz / c.n) << 16) | bits_of(depth);
         choice = tuned_in(g_tune_large, key);
         if (!choice) {
-          BCS_TRY(tune_large_piece(ctx, c, in, po, ok, depth, ord, &choice));
+          BCS_TRY(tune_large_piece(ctx, c, in, po, ok, deep_ok, depth, ord, &choice));
           remember_in(g_tune_large, key, choice);
         }
         ctx.stats.tuned |= 1ll << choice;
         if (choice == LARGE_PATH_BATCHED) ms_tuned.push_back(ci);
         if (choice == LARGE_PATH_PER_SOURCE) ps_tuned.push_back(ci);
-        if (choice != LARGE_PATH_WIDE) continue;
+        if (choice != LARGE_PATH_WIDE && choice != LARGE_PATH_DEEP) continue;
       }
-      bool take = ok;
-      if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) {
-        take = take && depth <= PULL_MAX_ECC;
-      }
+      bool take = ok && lp_mode != LARGE_PATH_DEEP && choice != LARGE_PATH_DEEP;
+      if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) take = take && depth <= PULL_MAX_ECC;
       const size_t state = pull_piece_bytes(c.n, c.nnz, bound);
       if (take && state > ((size_t)1 << 30)) {  // its state has to fit
         size_t free_b = 0, total_b = 0;
         BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
         take = state <= free_b / 4 * 3;
       }
-      if (!take) {
+      if (!take && !deep_ok) {
         rest.push_back(ci);
         continue;
       }
       if (po.sources) {  // the caller's sources, in the caller's order
         std::vector<int32_t> h(po.nsources);
         for (int64_t i = 0; i < po.nsources; i++) h[i] = (int32_t)po.sources[i];
-        BCS_CUDA(cudaMemcpyAsync(ord, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
+        BCS_CUDA(cudaMemcpyAsync(ord + c.n, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
         BCS_CUDA(cudaStreamSynchronize(ctx.stream));
       }
-      pull.push_back(PullJob{ci, (int32_t)nsrc_of(c), bound, off[k]});
+      const int64_t src_off = po.sources ? off[k] + c.n : -1;
+      if (take) pull.push_back(PullJob{ci, (int32_t)nsrc_of(c), bound, po.sources ? src_off : off[k]});
+      else deep.push_back(DeepJob{ci, (int32_t)nsrc_of(c), bound, off[k], src_off});
     }
     large.swap(rest);
   }
@@ -1210,9 +1219,10 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   for (int32_t ci : ms_tuned) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
   for (int32_t ci : ps_tuned) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
   for (const PullJob &j : pull) ctx.stats.n_large_sources += j.nsrc;
+  for (const DeepJob &j : deep) ctx.stats.n_large_sources += j.nsrc;
   ctx.stats.work_sources_entries = work_se;
   ctx.stats.work_sources_vertices = work_sv;
-  if (small.empty() && large.empty() && pull.empty() && ms_tuned.empty() && ps_tuned.empty()) return BCS_OK;
+  if (small.empty() && large.empty() && pull.empty() && deep.empty() && ms_tuned.empty() && ps_tuned.empty()) return BCS_OK;
 
   DBuf<int> d_err;
   DBuf<unsigned long long> d_dag;
@@ -1299,6 +1309,14 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     BCS_TRY(run_pull(ctx, comps, pull, in, F, pull_order.p, d_comps.p, per_batch, d_err.p, d_dag.p));
     tm.stop_into(ctx, &ctx.stats.ms_bcreach_large);
     tr.mark("pull");
+  }
+  for (const DeepJob &j : deep) {
+    StageTimer tm(ctx.stream);
+    tm.start();
+    BCS_TRY(run_deep(ctx, comps[j.ci], in, F, pull_order.p + j.ord_off, pull_parent.p + j.ord_off, j.src_off < 0 ? nullptr : pull_order.p + j.src_off,
+                     j.nsrc, j.depth_bound, d_err.p, d_dag.p));
+    tm.stop_into(ctx, &ctx.stats.ms_bcreach_large);
+    tr.mark("deep");
   }
   // one source per CTA over the given list; *d_lmax (optional) receives the
   // deepest BFS level any of them reached

@@ -274,7 +274,7 @@ struct BcInput {
 };
 
 // WIDE: the pull kernel; MID: the pull kernel on connected pieces of at most 65,536 vertices
-enum { LARGE_PATH_AUTO = 0, LARGE_PATH_WIDE = 1, LARGE_PATH_BATCHED = 2, LARGE_PATH_PER_SOURCE = 3, LARGE_PATH_MID = 4 };
+enum { LARGE_PATH_AUTO = 0, LARGE_PATH_WIDE = 1, LARGE_PATH_BATCHED = 2, LARGE_PATH_PER_SOURCE = 3, LARGE_PATH_MID = 4, LARGE_PATH_DEEP = 5 };
 
 struct BcPlanOpts {
   bool fp32_delta = false;
@@ -332,20 +332,33 @@ int recip_table(Ctx &ctx, const double **out);
 int pull_depth_limit();
 // bytes of device state one slab of a piece takes, at most
 size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound);
+// Bc-Reach on one deep piece of small degree, each CTA searching several
+// sources at once (deep.cu).  d_bfs, d_parent: the piece's vertices in BFS order
+// and their tree parents (-1: roots); d_sources: local ids, null for every
+// vertex; no source reaches deeper than depth_bound.  deep_takes: whether it
+// can run (degree, sizes, memory).
+int run_deep(Ctx &ctx, const CompDesc &c, const BcInput &in, bool fp32, const int32_t *d_bfs, const int32_t *d_parent,
+             const int32_t *d_sources, int32_t nsrc, int depth_bound, int *d_err, unsigned long long *d_dag);
+bool deep_takes(const CompDesc &c, int depth_bound, size_t free_bytes);
 // BFS of each listed piece from its first vertex, one piece per CTA: the
-// vertices in the order reached at order[ord_off[i] ..), the deepest level and
-// the number reached (host results; synchronises)
+// vertices in the order reached at order[ord_off[i] ..), their tree parents
+// (-1: the root) at parent[ord_off[i] ..), the deepest level and the number
+// reached (host results; synchronises).  A piece of more than
+// PIECE_BFS_MAX_N vertices is given up, reached -1, when a level is wide.
 int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_comps, const std::vector<int32_t> &list,
-              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, std::vector<int32_t> *depth,
-              std::vector<int32_t> *reached);
+              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent,
+              std::vector<int32_t> *depth, std::vector<int32_t> *reached);
 // BFS of a connected graph from `root` (rows at rp[v]..rp[v+1] of col):
 // queue_out[0..*reached) the vertices in the order the search reaches them,
+// parent (nullable) their tree parents by vertex (-1: the root),
 // *depth the deepest level (order.cu)
 int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_t root, int32_t *queue_out,
-              int *depth, int64_t *reached);
+              int32_t *parent, int *depth, int64_t *reached);
 // BFS order of every connected component of g (rows start at 0), each from
 // its smallest vertex, components contiguous; *depth the deepest level
-int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int *depth);
+int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth);
+// pieces of at most this many vertices are searched one per CTA
+constexpr int PIECE_BFS_MAX_N = 32768;
 
 // Bc-Reach after one more articulation split of the merged pieces
 // (resplit.cu): in.bcp (the merged vertices' bc') gains the new pieces' bc'.

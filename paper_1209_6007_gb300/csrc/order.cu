@@ -41,7 +41,8 @@ __global__ void k_order_roots(int64_t n, const int32_t *__restrict__ label, int3
 // The level-synchronous search; lcount[l] counts level l (one counter per
 // level, so one grid-wide wait per level suffices).  out[0] = vertices queued.
 __global__ void k_order_bfs(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int32_t *level,
-                            int32_t *queue, unsigned long long *lcount, int64_t *out, GridBarrier bar) {
+                            int32_t *queue, int32_t *parent, unsigned long long *lcount, int64_t *out,
+                            GridBarrier bar) {
   const int sl = (int)(threadIdx.x % ORDER_SUB);
   const int64_t sub0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / ORDER_SUB;
   const int64_t nsub = (int64_t)gridDim.x * blockDim.x / ORDER_SUB;
@@ -51,7 +52,10 @@ __global__ void k_order_bfs(const int64_t *__restrict__ rp, const int32_t *__res
       const int32_t v = queue[i];
       for (int64_t k = rp[v] + sl; k < rp[v + 1]; k += ORDER_SUB) {
         const int32_t w = col[k];
-        if (uf_vload(level + w) < 0 && atomicCAS(level + w, -1, L + 1) < 0) push_one(queue, lcount + L + 1, hi, w);
+        if (uf_vload(level + w) < 0 && atomicCAS(level + w, -1, L + 1) < 0) {
+          if (parent) parent[w] = v;
+          push_one(queue, lcount + L + 1, hi, w);
+        }
       }
     }
     if (!grid_wait(bar)) return;
@@ -166,7 +170,8 @@ int bfs_order_graph(Ctx &ctx, const DevGraph &g, DBuf<int64_t> *rp2, DBuf<int32_
     int32_t *levelp = level.p, *queuep = queue.p;
     unsigned long long *lcp = lcount.p;
     int64_t *outp = out.p;
-    void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&lcp, (void *)&outp,
+    int32_t *parentp = nullptr;
+    void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
                     (void *)&gb};
     BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                          ctx.stream));
@@ -246,11 +251,14 @@ __global__ void k_bfs_root(int64_t n, int32_t root, int32_t *level, int32_t *que
 }
 
 int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_t root, int32_t *queue_out,
-              int *depth, int64_t *reached) {
+              int32_t *parent, int *depth, int64_t *reached) {
   *depth = 0;
   *reached = n;
   if (n <= 1) {
-    if (n == 1) BCS_CUDA(cudaMemcpyAsync(queue_out, &root, sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
+    if (n == 1) {
+      BCS_CUDA(cudaMemcpyAsync(queue_out, &root, sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
+      if (parent) BCS_CUDA(cudaMemsetAsync(parent, 0xFF, sizeof(int32_t), ctx.stream));
+    }
     return BCS_OK;
   }
   DBuf<int32_t> level;
@@ -258,6 +266,7 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
   BCS_TRY(level.alloc(n, ctx.stream));
   BCS_TRY(lcount.alloc(n + 2, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(lcount.p, 0, (n + 2) * sizeof(unsigned long long), ctx.stream));
+  if (parent) BCS_CUDA(cudaMemsetAsync(parent, 0xFF, n * sizeof(int32_t), ctx.stream));
   k_bfs_root<<<grid_of(n, 256, ctx.num_sms * 8), 256, 0, ctx.stream>>>(n, root, level.p, queue_out, lcount.p);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
@@ -279,7 +288,8 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
   int32_t *levelp = level.p, *queuep = queue_out;
   unsigned long long *lcp = lcount.p;
   int64_t *outp = out.p;
-  void *args[] = {(void *)&rp, (void *)&col, (void *)&levelp, (void *)&queuep, (void *)&lcp, (void *)&outp,
+  int32_t *parentp = parent;
+  void *args[] = {(void *)&rp, (void *)&col, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
                   (void *)&gb};
   BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                        ctx.stream));
@@ -309,7 +319,7 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
 // BFS order of every connected component at once (each from its smallest
 // vertex), the components kept contiguous: queue_out[0..n), *depth the
 // deepest level over all components.
-int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int *depth) {
+int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth) {
   const int64_t n = g.n;
   *depth = 0;
   if (n == 0) return BCS_OK;
@@ -322,6 +332,7 @@ int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int *d
   BCS_TRY(level.alloc(n, ctx.stream));
   BCS_TRY(lcount.alloc(n + 2, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(lcount.p, 0, (n + 2) * sizeof(unsigned long long), ctx.stream));
+  if (parent) BCS_CUDA(cudaMemsetAsync(parent, 0xFF, n * sizeof(int32_t), ctx.stream));
   k_order_roots<<<grid_of(n, 256, ctx.num_sms * 32), 256, 0, ctx.stream>>>(n, label.p, level.p, queue_out, lcount.p);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
@@ -339,7 +350,8 @@ int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int *d
   int32_t *levelp = level.p, *queuep = queue_out;
   unsigned long long *lcp = lcount.p;
   int64_t *outp = out.p;
-  void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&lcp, (void *)&outp,
+  int32_t *parentp = parent;
+  void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
                   (void *)&gb};
   BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                        ctx.stream));

@@ -792,7 +792,8 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
             const double d = REACH ? fma(sg, x, (double)r.init) : sg * x;
             if (l > 1) {  // the sources' own dependencies are not needed
               const double rc = idx ? __ldg(A.recip + idx) : recip_pos(sg);
-              S8[r.at + src] = IDENT && r.id != 1 ? fma((double)r.id, d, (double)r.id) * rc : (d + 1.0) * rc;
+              const double kr = IDENT && r.id != 1 ? (double)r.id * rc : rc;
+              S8[r.at + src] = fma(d, kr, kr);
             }
             return REACH || IDENT ? A.ws[(size_t)U.j * PULL_W + src] * d : d;
           };
@@ -954,16 +955,23 @@ __global__ void k_pull_idmax(int64_t n, const int32_t *__restrict__ ident, int32
 }
 
 // BFS of each listed piece from its first vertex, one piece per CTA at a
-// time: its vertices in the order the search reaches them, the deepest level
-// and how many it reached.
-constexpr int PIECE_BFS_THREADS = 512;
+// time: its vertices in the order the search reaches them, their tree parents,
+// the deepest level and how many it reached.  Levels are narrow or the piece is
+// small (a large piece is given up at a level wider than PIECE_BFS_WIDE: the
+// whole GPU searches it): the wait after a level is CTA-wide, and the level's
+// vertices are kept in shared memory.
+constexpr int PIECE_BFS_THREADS = 1024;
+constexpr int PIECE_BFS_RING = 2048;
+constexpr int PIECE_BFS_WIDE = 8192;
 __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc *__restrict__ comps,
                                                                  const int32_t *__restrict__ list, int nlist,
                                                                  int *next, const int64_t *__restrict__ g_row,
                                                                  const int32_t *__restrict__ g_col,
                                                                  const int64_t *__restrict__ ord_off, int32_t *order,
-                                                                 int32_t *level, int32_t *depth, int32_t *reached) {
+                                                                 int32_t *parent, int32_t *level, int32_t *depth,
+                                                                 int32_t *reached) {
   __shared__ int s_i, s_tail;
+  __shared__ int32_t s_ring[2][PIECE_BFS_RING];
   for (;;) {
     if (threadIdx.x == 0) s_i = atomicAdd(next, 1);
     __syncthreads();
@@ -971,20 +979,38 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
     if (i >= nlist) return;
     const CompDesc c = comps[list[i]];
     const int64_t *row = g_row + c.row_off;
-    int32_t *const q = order + ord_off[i], *const lv = level + ord_off[i];
+    int32_t *const q = order + ord_off[i], *const lv = level + ord_off[i], *const par = parent + ord_off[i];
     for (int32_t v = threadIdx.x; v < c.n; v += PIECE_BFS_THREADS) lv[v] = v == 0 ? 0 : -1;
     if (threadIdx.x == 0) {
-      q[0] = 0;
+      q[0] = s_ring[0][0] = 0;
+      par[0] = -1;
       s_tail = 1;
     }
     __syncthreads();
     int lo = 0, hi = 1, L = 0;
     while (lo < hi) {
+      const int32_t *const ring = s_ring[L & 1];
+      int32_t *const ring_next = s_ring[(L + 1) & 1];
       for (int k = lo + (int)threadIdx.x; k < hi; k += PIECE_BFS_THREADS) {
-        const int32_t v = q[k];
-        for (int64_t e = row[v]; e < row[v + 1]; e++) {
-          const int32_t u = g_col[e];
-          if (*(volatile int32_t *)(lv + u) < 0 && atomicCAS(lv + u, -1, L + 1) < 0) q[atomicAdd(&s_tail, 1)] = u;
+        const int32_t v = k - lo < PIECE_BFS_RING ? ring[k - lo] : q[k];
+        const int64_t e1 = row[v + 1];
+        for (int64_t e = row[v]; e < e1; e += 4) {
+          int32_t u[4], l[4];
+#pragma unroll
+          for (int j = 0; j < 4; j++) u[j] = e + j < e1 ? g_col[e + j] : -1;
+#pragma unroll
+          for (int j = 0; j < 4; j++) l[j] = u[j] >= 0 ? *(volatile int32_t *)(lv + u[j]) : 0;
+#pragma unroll
+          for (int j = 0; j < 4; j++)
+            if (l[j] < 0) l[j] = atomicCAS(lv + u[j], -1, L + 1);
+#pragma unroll
+          for (int j = 0; j < 4; j++)
+            if (l[j] < 0) {
+              const int t = atomicAdd(&s_tail, 1);
+              q[t] = u[j];
+              par[u[j]] = v;
+              if (t - hi < PIECE_BFS_RING) ring_next[t - hi] = u[j];
+            }
         }
       }
       __syncthreads();
@@ -992,17 +1018,18 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
       hi = *(volatile int *)&s_tail;
       __syncthreads();
       L++;
+      if (c.n > PIECE_BFS_MAX_N && hi - lo > PIECE_BFS_WIDE) break;
     }
     if (threadIdx.x == 0) {
       depth[i] = L - 1;
-      reached[i] = hi;
+      reached[i] = lo < hi ? -1 : hi;
     }
   }
 }
 
 int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_comps, const std::vector<int32_t> &list,
-              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, std::vector<int32_t> *depth,
-              std::vector<int32_t> *reached) {
+              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent,
+              std::vector<int32_t> *depth, std::vector<int32_t> *reached) {
   const int P = (int)list.size();
   depth->assign(P, 0);
   reached->assign(P, 0);
@@ -1018,8 +1045,8 @@ int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_co
   BCS_CUDA(cudaMemcpyAsync(d_list.p, list.data(), P * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
   BCS_CUDA(cudaMemcpyAsync(d_off.p, ord_off.data(), P * sizeof(int64_t), cudaMemcpyHostToDevice, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(d_out.p + 2 * P, 0, sizeof(int32_t), ctx.stream));
-  k_piece_bfs<<<std::min(P, ctx.num_sms * 4), PIECE_BFS_THREADS, 0, ctx.stream>>>(
-      d_comps, d_list.p, P, d_out.p + 2 * P, in.row, in.col, d_off.p, order, d_level.p, d_out.p, d_out.p + P);
+  k_piece_bfs<<<std::min(P, ctx.num_sms * 2), PIECE_BFS_THREADS, 0, ctx.stream>>>(
+      d_comps, d_list.p, P, d_out.p + 2 * P, in.row, in.col, d_off.p, order, parent, d_level.p, d_out.p, d_out.p + P);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
   BCS_CUDA(cudaMemcpyAsync(depth->data(), d_out.p, P * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx.stream));
