@@ -519,8 +519,13 @@ __global__ void k_deep_sources(int32_t k, const int32_t *__restrict__ given, con
 __global__ void k_deep_add(int32_t n, const int32_t *__restrict__ order, const double *__restrict__ acc, int copies,
                            double *bcp) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double t = 0.0;
-    for (int c = 0; c < copies; c++) t += acc[(size_t)c * n + i];
+    double t = 0.0, lost = 0.0;  // what the additions round off is kept (hundreds of copies)
+    for (int c = 0; c < copies; c++) {
+      const double a = acc[(size_t)c * n + i], sum = t + a, of_a = sum - t;
+      lost += (t - (sum - of_a)) + (a - of_a);
+      t = sum;
+    }
+    t += lost;
     if (t != 0.0) bcp[order[i]] += t;
   }
 }
