@@ -157,7 +157,7 @@ def workload(name: str, scale: int):
 # ncu summaries of the dominant kernels, each keyed by the SHA-1 of the
 # sources the kernel compiles from; a figure is used only while they match
 PROFILES = {
-    "small": ("bcreach_small_articulation.json", ("bcreach.cu", "bc_math.cuh")),
+    "small": ("bcreach_small_articulation.json", ("small.cu", "bc_math.cuh")),
     "wide": ("bcreach_wide_twins.json", ("pull.cu", "bc_math.cuh", "coop.cuh")),
 }
 

@@ -1,5 +1,6 @@
 // bcreach.cu - Bc-Reach (Algorithm 2 with the identical-vertex terms of
-// Section 3.3.3) over many components in persistent launches.
+// Section 3.3.3) over many components: the plan that sends each to a kernel,
+// the autotuner, and the one-source-per-CTA kernel in global memory.
 //
 // Per source s of a component (local ids, reach r[], ident k[]):
 //   phase 1 (BFS, Algorithm 1):  d[s] = 0, sigma[s] = 1,
@@ -10,12 +11,13 @@
 // Phase 2 is evaluated in the equivalent "coefficient" form
 //     c[w] = k[w] (1 + delta[w]) / sigma[w],   delta[v] = r[v] - 1 + sigma[v] * sum_w c[w]
 // so that each shortest-path-DAG edge costs one addition and each vertex one
-// reciprocal (from a table for small integer counts).
+// reciprocal (in small.cu, pull.cu and deep.cu from a table for small integer
+// counts).
 //
-// A group of threads (one warp up to a whole CTA) runs one source at a time,
-// level-synchronously: the BFS queue doubles as the stack of Algorithm 1 and
-// its level boundaries are kept, so phase 2 walks the levels deepest first
-// and pulls from the successors (no atomics in phase 2).
+// The one-source-per-CTA kernel is level-synchronous: the BFS queue doubles as
+// the stack of Algorithm 1 and its level boundaries are kept, so phase 2 walks
+// the levels deepest first and pulls from the successors (no atomics in phase
+// 2).
 //
 // Path counts are exact 64-bit integers while a level's growth bound stays
 // below 2^62; past it they are FP64 and each level carries a power-of-two
@@ -42,12 +44,6 @@
 
 namespace bcs {
 
-constexpr int SMALL_THREADS = 256;
-// Shared memory one small-path CTA may use: a piece whose state for a single
-// source does not fit goes to the global-memory path.
-constexpr size_t SMALL_SMEM = 100 * 1024;
-constexpr int SMALL_MAX_GROUPS = 8;
-constexpr int DISC_CH = 4;  // row entries per step of the shared-memory discovery pass (divides 32)
 constexpr int LARGE_THREADS = 512;
 // BFS depth above which large pieces run one source per CTA rather than 32
 constexpr int MS_DEPTH_LIMIT = 64;
@@ -56,36 +52,33 @@ constexpr int MS_DEPTH_LIMIT = 64;
 constexpr int PULL_MAX_ECC = 40;
 // and deeper ones than this, of small degree, on the deep kernel (deep.cu)
 constexpr int DEEP_MIN_ECC = 40;
+// The shared memory a small-path CTA gets without the autotuner: four CTAs of
+// an SM's 227 KB (articulation-vertex workload, 130 M (vertex, source) pairs:
+// 5.0 ms; with 72 KB 5.1, with 100 KB 5.8 to 7.9, with 36 KB 6.2)
+constexpr size_t SMALL_BUDGET = 54 * 1024;
+// Pieces that cannot run MID_SOURCES sources at once in that budget (some 800
+// vertices and more) go to the pull kernel instead, if they are shallow and
+// come in numbers: its cost is per level and slab (256 sources of a piece), so
+// it wants few levels and slabs of at least MID_MIN_ROWS rows together.
+// Batch of 16- to 4,096-vertex graphs: small and pull kernel 96 ms without
+// the rule, 56 with it (59 from 1 source on, 56 from 3); a lone piece
+// of 1,400 vertices 0.29 ms here, 1.08 there.
+constexpr int MID_SOURCES = 2;
+constexpr int MID_PIECE_ECC = 8;
+constexpr int64_t MID_MIN_ROWS = 1 << 15;
 // BCS_LARGE_PATH=mid: the pull kernel on connected pieces of at most this
 // many vertices and MID_MAX_ECC levels
 constexpr int MID_MAX_N = 65536;
 constexpr int MID_MAX_ECC = 30;
 
-struct SmallItem {
-  int32_t comp;
-  int32_t s_begin;  // index range into the source list (or local ids)
-  int32_t s_end;
-  int32_t ngroups;  // groups (concurrent sources) per CTA, 1..8
-};
-
-// ------------------------------------------------------------------ group
-struct Group {
-  int rank, size, bar;
-  __device__ __forceinline__ void sync() const {
-    if (size == 32) __syncwarp();
-    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(size) : "memory");
-  }
-};
-
-__device__ __forceinline__ double group_max(const Group &g, double x, volatile double *red) {
+__device__ __forceinline__ double cta_max(double x, volatile double *red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-  if (g.size == 32) return x;
-  if ((g.rank & 31) == 0) red[g.rank >> 5] = x;
-  g.sync();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
   double r = red[0];
-  for (int i = 1; i < (g.size >> 5); i++) r = fmax(r, red[i]);
-  g.sync();
+  for (int i = 1; i < ((int)blockDim.x >> 5); i++) r = fmax(r, red[i]);
+  __syncthreads();
   return r;
 }
 
@@ -111,27 +104,24 @@ __global__ void k_fill_recip_table() {
     g_recip_table[k] = k == 0 ? 0.0 : 1.0 / (double)k;
 }
 
-// State of one source, in shared (small path) or global (large path) memory.
-template <bool FP32, typename QT = int32_t>
+// State of one source in global memory.
+template <bool FP32>
 struct SrcState {
   int32_t *d;
   double *sig;
-  typename CoefT<FP32>::type *coef;  // global path: sigma * ident in phase 1; shared path: == sig
-  QT *queue;                         // 16-bit local ids on the shared-memory path
-  uint32_t *dmask;     // shared-memory path: DAG successors among the first 32 row entries
+  typename CoefT<FP32>::type *coef;  // sigma * ident in phase 1
+  int32_t *queue;
   int32_t *lvl_start;  // levels + 2
   int32_t *lvl_exp;    // levels + 1
   int *qtail;          // shared counter
-  double *red;         // shared, 16 doubles: group maxima, and the source weight
+  double *red;         // shared, 17 doubles: maxima, and the source weight
 };
-constexpr int RED_WS = 15;  // slot of the source weight in SrcState::red
+constexpr int RED_WS = 16;  // slot of the source weight in SrcState::red
 
-struct Weights {  // global-memory path: the int32 arrays; shared path: only the FP64 copies
+struct Weights {
   const int32_t *reach;   // local, nullable
   const int32_t *ident;   // local, nullable
-  const double *init_d;   // reach - 1 as FP64, nullable (converted on the fly)
-  const double *ident_d;  // ident as FP64, nullable
-  bool frac;              // init_d may be fractional: never read reach as an integer
+  const double *init_d;   // reach - 1 as FP64, nullable, possibly fractional (it then replaces reach)
 };
 
 struct Debug {
@@ -141,12 +131,10 @@ struct Debug {
   double *delta;
 };
 
-
-// One source of Bc-Reach over a component held as (row, col) with local ids.
-// RESET_BY_QUEUE: the distances start at -1 and are put back that way
-// through the queue at the end (global-memory path); else they are
-// initialised here (shared-memory path).  acc is private to the group (plain
-// adds).  dag counts the shortest-path DAG edges seen in phase 2.
+// One source of Bc-Reach over a component held as (row, col) with local ids,
+// by one CTA.  The distances start at -1 and are put back that way through the
+// queue at the end.  acc is private to the CTA (plain adds).  dag counts the
+// shortest-path DAG edges seen in phase 2.
 //
 // Path counts are integers.  While the growth bound fan^L of a level stays
 // below 2^62 they are summed as exact 64-bit integers (the FP64 pipe is the
@@ -154,47 +142,20 @@ struct Debug {
 // FP64 sum); the first level whose bound could pass 2^62 converts the level
 // before it to FP64 once, and from there on counts are FP64 with a
 // power-of-two exponent per level.  sig holds int64 on the integer levels.
-//
-// Shared-memory path (!RESET_BY_QUEUE): one pass over a level's rows both
-// discovers the next level and, on the integer levels, pushes the path
-// counts along the DAG edges it finds (shared-memory atomics); each vertex
-// also keeps the DAG edges among its first 32 row entries as a bit mask, so
-// phase 2 visits only the successors; its phase-2 coefficients overwrite the
-// path counts in place.  The global-memory path pulls the counts in a second
-// pass and finds successors by their level (pushing through L2 atomics
-// measured slower on deep graphs, where that path is used).
-template <bool REACH, bool IDENT, bool FP32, bool RESET_BY_QUEUE, typename RowT, typename ColT, typename QT>
-__device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n, const RowT *__restrict__ row,
-                               const ColT *__restrict__ col, const Weights wt, const SrcState<FP32, QT> st,
-                               double *acc, const double fan, int *err, const Debug *dbg,
-                               unsigned long long &dag, int *lmax_out = nullptr) {
-  // reach and ident as integers: from the int32 arrays on the global-memory
-  // path, from the FP64 copies (integer instructions) on the shared path
-  auto ident_i = [&](int32_t v) -> long long {
-    return wt.ident ? (long long)wt.ident[v] : f64_to_i64_exact(wt.ident_d[v]);
-  };
-  auto reach_i = [&](int32_t v) -> long long {
-    return wt.reach ? (long long)wt.reach[v] : f64_to_i64_exact(wt.init_d[v]) + 1;
-  };
+// Counts are pulled in a second pass over a level and successors found by
+// their level (pushing through L2 atomics measured slower on deep graphs).
+template <bool REACH, bool IDENT, bool FP32>
+__device__ void bcreach_source(const int32_t s, const int64_t *__restrict__ row, const int32_t *__restrict__ col,
+                               const Weights wt, const SrcState<FP32> st, double *acc, const double fan, int *err,
+                               const Debug *dbg, unsigned long long &dag, int *lmax_out) {
+  const int rank = (int)threadIdx.x, size = (int)blockDim.x;
   int32_t *const d = st.d;
   double *const sig = st.sig;
   long long *const sigi = (long long *)st.sig;
-  double *const sk = (double *)st.coef;  // global path: sigma[v] * (v == s ? 1 : ident[v]) in phase 1
+  double *const sk = (double *)st.coef;  // sigma[v] * (v == s ? 1 : ident[v]) in phase 1
   long long *const ski = (long long *)st.coef;
-  constexpr bool PUSH = !RESET_BY_QUEUE;
-  // Shared-memory path: the coefficient of phase 2 overwrites the path count
-  // of the same vertex (st.coef == st.sig); phase 1 keeps sigma alone and
-  // multiplies by ident where it reads it.
-  constexpr bool ALIAS = PUSH;
   long long *const pull_src = IDENT ? ski : sigi;  // sigma * ident (the source counts once)
-  if (!RESET_BY_QUEUE) {
-    for (int v = g.rank; v < n; v += g.size) {
-      d[v] = -1;
-      sigi[v] = 0;
-    }
-    g.sync();
-  }
-  if (g.rank == 0) {
+  if (rank == 0) {
     d[s] = 0;
     sigi[s] = 1;
     ski[s] = 1;
@@ -204,7 +165,7 @@ __device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n,
     st.lvl_start[1] = 1;
     st.lvl_exp[0] = 0;
   }
-  g.sync();
+  __syncthreads();
   // ---------------------------------------------------------- phase 1
   int lo = 0, hi = 1, L = 0, ecur = 0;
   int lint = 1 << 30;  // first FP64 level
@@ -213,137 +174,92 @@ __device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n,
   const int flg = ceil_log2_pos(fan);
   int blg = 0;
   for (;;) {
-    // level L+1 keeps integer counts while its growth bound stays below 2^62
-    const bool push = PUSH && lint > L + 1 && blg + flg < 62;
-    // below 2^31 every partial sum fits the low word: 32-bit atomics
-    const bool push32 = push && blg + flg < 31;
     // discover level L+1 (integer work only)
-    for (int i = lo + g.rank; i < hi; i += g.size) {
+    for (int i = lo + rank; i < hi; i += size) {
       const int32_t v = st.queue[i];
-      const RowT eb = row[v], ee = row[v + 1];
-      if (PUSH) {
-        // sigma[v] * ident[v], formed by v's own lane (sigma[v] is final)
-        const long long pv = !push ? 0 : (IDENT && v != s ? sigi[v] * ident_i(v) : sigi[v]);
-        uint32_t m = 0u;
-        // DISC_CH row entries at a time, so that their shared-memory round
-        // trips overlap instead of forming one chain per entry
-        for (RowT e0 = eb; e0 < ee; e0 += DISC_CH) {
-          int32_t w[DISC_CH];
-          int dw[DISC_CH];
-#pragma unroll
-          for (int j = 0; j < DISC_CH; j++) w[j] = e0 + j < ee ? (int32_t)col[e0 + j] : -1;
-#pragma unroll
-          for (int j = 0; j < DISC_CH; j++) dw[j] = w[j] >= 0 ? vld(d + w[j]) : L;  // L: no DAG edge
-          unsigned won = 0u, dagb = 0u;
-#pragma unroll
-          for (int j = 0; j < DISC_CH; j++) {
-            const int r = dw[j] < 0 ? atomicCAS(d + w[j], -1, L + 1) : dw[j];
-            won |= (unsigned)(r < 0) << j;
-            dagb |= (unsigned)(r < 0 || r == L + 1) << j;
-          }
-          if (won) {  // one counter update for the vertices this lane claimed
-            int pos = atomicAdd(st.qtail, __popc(won));
-#pragma unroll
-            for (int j = 0; j < DISC_CH; j++)
-              if (won >> j & 1u) st.queue[pos++] = w[j];
-          }
-#pragma unroll
-          for (int j = 0; j < DISC_CH; j++) {
-            if (dagb >> j & 1u) {
-              if (push32) atomicAdd((unsigned int *)(sigi + w[j]), (unsigned int)pv);
-              else if (push) atomicAdd((unsigned long long *)(sigi + w[j]), (unsigned long long)pv);
-            }
-          }
-          if (e0 - eb < 32) m |= dagb << (int)(e0 - eb);
-        }
-        st.dmask[v] = m;
-      } else {
-        for (RowT e = eb; e < ee; e++) {
-          const int32_t w = (int32_t)col[e];
-          if (vld(d + w) < 0 && atomicCAS(d + w, -1, L + 1) == -1) st.queue[atomicAdd(st.qtail, 1)] = w;
-        }
+      const int64_t eb = row[v], ee = row[v + 1];
+      for (int64_t e = eb; e < ee; e++) {
+        const int32_t w = col[e];
+        if (vld(d + w) < 0 && atomicCAS(d + w, -1, L + 1) == -1) st.queue[atomicAdd(st.qtail, 1)] = w;
       }
     }
-    g.sync();
+    __syncthreads();
     const int nhi = vld(st.qtail);
-    g.sync();
+    __syncthreads();
     if (nhi == hi) break;
     blg += flg;
     if (lint > L + 1 && blg >= 62) {
       // level L+1 may not fit 63 bits: it is pulled in FP64 from level L
-      // (shared-memory path: level L's counts turn FP64 in place, so level L
-      // is the first FP64 level)
-      lint = ALIAS ? L : L + 1;
-      for (int i = lo + g.rank; i < hi; i += g.size) {
+      lint = L + 1;
+      for (int i = lo + rank; i < hi; i += size) {
         const int32_t v = st.queue[i];
-        if (ALIAS) sig[v] = (double)sigi[v];
-        else sk[v] = (double)pull_src[v];
+        sk[v] = (double)pull_src[v];
       }
-      g.sync();
+      __syncthreads();
     }
-    if (push) {
-      // the counts of level L+1 are complete
-    } else if (L + 1 < lint) {  // path counts of level L+1, pulled from level L (one add per DAG edge)
-      for (int i = hi + g.rank; i < nhi; i += g.size) {
+    if (L + 1 < lint) {  // path counts of level L+1, pulled from level L (one add per DAG edge)
+      for (int i = hi + rank; i < nhi; i += size) {
         const int32_t w = st.queue[i];
         long long a = 0;
-        const RowT eb = row[w], ee = row[w + 1];
-        for (RowT e = eb; e < ee; e++) {
-          const int32_t u = (int32_t)col[e];
+        const int64_t eb = row[w], ee = row[w + 1];
+        for (int64_t e = eb; e < ee; e++) {
+          const int32_t u = col[e];
           if (d[u] == L) a += pull_src[u];
         }
         sigi[w] = a;
         if (IDENT) ski[w] = a * (long long)wt.ident[w];
       }
     } else {
-      for (int i = hi + g.rank; i < nhi; i += g.size) {
+      for (int i = hi + rank; i < nhi; i += size) {
         const int32_t w = st.queue[i];
         double a = 0.0;
-        const RowT eb = row[w], ee = row[w + 1];
-        for (RowT e = eb; e < ee; e++) {
-          const int32_t u = (int32_t)col[e];
-          if (d[u] == L) a += ALIAS ? (IDENT && u != s ? sig[u] * wt.ident_d[u] : sig[u]) : sk[u];
+        const int64_t eb = row[w], ee = row[w + 1];
+        for (int64_t e = eb; e < ee; e++) {
+          const int32_t u = col[e];
+          if (d[u] == L) a += sk[u];
         }
         sig[w] = a;
-        if (!ALIAS) sk[w] = IDENT ? a * (wt.ident_d ? wt.ident_d[w] : (double)wt.ident[w]) : a;
+        sk[w] = IDENT ? a * (double)wt.ident[w] : a;
       }
       if (blg > 900) {
-        g.sync();
+        __syncthreads();
         double m = 0.0;
-        for (int i = hi + g.rank; i < nhi; i += g.size) m = fmax(m, sig[st.queue[i]]);
-        m = group_max(g, m, st.red);
+        for (int i = hi + rank; i < nhi; i += size) m = fmax(m, sig[st.queue[i]]);
+        m = cta_max(m, st.red);
         if (!(m <= DBL_MAX)) {
-          if (g.rank == 0) atomicOr(err, ERR_OVERFLOW);
+          if (rank == 0) atomicOr(err, ERR_OVERFLOW);
         } else if (m > 0x1p960) {
           const int k = ilogb(m) - 959;
-          for (int i = hi + g.rank; i < nhi; i += g.size) {
+          for (int i = hi + rank; i < nhi; i += size) {
             const int32_t w = st.queue[i];
             sig[w] = scalbn(sig[w], -k);
-            if (!ALIAS) sk[w] = scalbn(sk[w], -k);
+            sk[w] = scalbn(sk[w], -k);
           }
           m = scalbn(m, -k);
           ecur += k;
         }
         blg = m >= 1.0 ? ceil_log2_pos(m) : 0;
-        g.sync();
+        __syncthreads();
       }
     }
     lo = hi;
     hi = nhi;
     L++;
-    if (g.rank == 0) {
+    if (rank == 0) {
       st.lvl_start[L + 1] = hi;
       st.lvl_exp[L] = ecur;
     }
   }
   const int Lmax = L;
-  if (lmax_out && g.rank == 0) atomicMax(lmax_out, Lmax);
+  if (lmax_out && rank == 0) atomicMax(lmax_out, Lmax);
   // the source's weight reach[s] * ident[s] waits in shared memory: read
   // per vertex, it is never recomputed (FP64) inside the divergent loop
-  if (g.rank == 0)
-    st.red[RED_WS] = (REACH && wt.frac) ? (wt.init_d[s] + 1.0) * (double)(IDENT ? ident_i(s) : 1ll)
-                                        : (double)((REACH ? reach_i(s) : 1ll) * (IDENT ? ident_i(s) : 1ll));
-  g.sync();
+  if (rank == 0) {
+    const long long is = IDENT ? (long long)wt.ident[s] : 1ll;
+    st.red[RED_WS] = (REACH && wt.init_d) ? (wt.init_d[s] + 1.0) * (double)is
+                                          : (double)((REACH ? (long long)wt.reach[s] : 1ll) * is);
+  }
+  __syncthreads();
   // ---------------------------------------------------------- phase 2
   unsigned long long ndag = 0;
   for (int l = Lmax; l >= 0; l--) {
@@ -351,47 +267,34 @@ __device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n,
     const int de = (l < Lmax) ? st.lvl_exp[l] - st.lvl_exp[l + 1] : 0;
     const double scl = pow2_int(de);
     const bool is_int = l < lint;
-    for (int i = a + g.rank; i < b; i += g.size) {
+    for (int i = a + rank; i < b; i += size) {
       const int32_t v = st.queue[i];
       double dv;
-      if (!FP32) {
-        const long long si = is_int ? sigi[v] : 0;
-        const double sv = is_int ? i64_to_f64_pos(si) : sig[v];
-        double sum = 0.0;
-        if (l < Lmax) {
-          // successors first as a bit mask (integer work), then FP64 adds
-          // only for them: an FP64 warp instruction costs the pipe the same
-          // whatever its active lanes, so the FP64 loop should run as few
-          // iterations as possible (the DAG out-degree, not the degree)
-          const RowT eb = row[v], ee = row[v + 1];
-          for (RowT e0 = eb; e0 < ee; e0 += 32) {
-            uint32_t mask = 0u;
-            if (PUSH && e0 == eb) {
-              mask = st.dmask[v];
-            } else {
-              const int cnt = (int)((ee - e0) < 32 ? (ee - e0) : 32);
-              for (int j = 0; j < cnt; j++) mask |= (uint32_t)(d[(int32_t)col[e0 + j]] == l + 1) << j;
-            }
-            ndag += __popc(mask);
-            while (mask) {  // one FP64 add per successor (pairing them measured slower)
-              const int j = __ffs(mask) - 1;
-              mask &= mask - 1u;
-              sum += ((const double *)st.coef)[(int32_t)col[e0 + j]];
-            }
-          }
-          if (de != 0) sum *= scl;
+      // successors first as a bit mask (integer work), then one addition for
+      // each: an FP64 warp instruction costs the pipe the same whatever its
+      // active lanes, so the FP64 loop should run as few iterations as
+      // possible (the DAG out-degree, not the degree)
+      auto successors = [&](auto add) {
+        if (l == Lmax) return;
+        const int64_t eb = row[v], ee = row[v + 1];
+        for (int64_t e0 = eb; e0 < ee; e0 += 32) {
+          uint32_t mask = 0u;
+          const int cnt = (int)((ee - e0) < 32 ? (ee - e0) : 32);
+          for (int j = 0; j < cnt; j++) mask |= (uint32_t)(d[col[e0 + j]] == l + 1) << j;
+          ndag += __popc(mask);
+          for (; mask; mask &= mask - 1u) add(col[e0 + __ffs(mask) - 1]);
         }
+      };
+      if (!FP32) {
+        const double sv = is_int ? i64_to_f64_pos(sigi[v]) : sig[v];
+        double sum = 0.0;
+        successors([&](int32_t w) { sum += ((const double *)st.coef)[w]; });
+        if (de != 0) sum *= scl;
         const double init = REACH ? (wt.init_d ? wt.init_d[v] : (double)(wt.reach[v] - 1)) : 0.0;
         dv = fma(sv, sum, init);
         if (l > 0) {  // the source's coefficient is never read
-          const double kv = IDENT ? (wt.ident_d ? wt.ident_d[v] : (double)wt.ident[v]) : 1.0;
-          // 1/sigma: small integer counts (the usual case) from a table of
-          // correctly rounded reciprocals, so a warp whose lanes all have one
-          // issues no FP64 work for it
-          double r;
-          if (PUSH && is_int && si < RECIP_TABLE) r = g_recip_table[si];
-          else r = recip_pos(sv);
-          ((double *)st.coef)[v] = fma(kv, dv, kv) * r;
+          const double kv = IDENT ? (double)wt.ident[v] : 1.0;
+          ((double *)st.coef)[v] = fma(kv, dv, kv) * recip_pos(sv);
         }
       } else {
         int ev;
@@ -400,35 +303,15 @@ __device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n,
         else split_pow2(sig[v], ev, mv);
         ev += st.lvl_exp[l];
         float sum = 0.0f;
-        if (l < Lmax) {
-          const RowT eb = row[v], ee = row[v + 1];
-          for (RowT e0 = eb; e0 < ee; e0 += 32) {
-            uint32_t mask = 0u;
-            if (PUSH && e0 == eb) {
-              mask = st.dmask[v];
-            } else {
-              const int cnt = (int)((ee - e0) < 32 ? (ee - e0) : 32);
-              for (int j = 0; j < cnt; j++) mask |= (uint32_t)(d[(int32_t)col[e0 + j]] == l + 1) << j;
-            }
-            ndag += __popc(mask);
-            while (mask) {  // two successors per step: their loads overlap
-              const int j0 = __ffs(mask) - 1;
-              mask &= mask - 1u;
-              const int j1 = mask ? __ffs(mask) - 1 : -1;
-              mask &= mask - 1u;
-              const Coef32 c0 = ((const Coef32 *)st.coef)[(int32_t)col[e0 + j0]];
-              const Coef32 c1 = j1 >= 0 ? ((const Coef32 *)st.coef)[(int32_t)col[e0 + j1]] : Coef32{0.0f, ev};
-              const int x0 = ev - c0.e, x1 = ev - c1.e;  // <= 0: sigma[v] <= sigma[w]
-              if (x0 >= -126) sum = fmaf(c0.c, __int_as_float((127 + x0) << 23), sum);
-              if (x1 >= -126) sum = fmaf(c1.c, __int_as_float((127 + x1) << 23), sum);
-            }
-          }
-        }
-        const float df =
-            fmaf(mv, sum, REACH ? (wt.frac ? (float)wt.init_d[v] : (float)(reach_i(v) - 1)) : 0.0f);
+        successors([&](int32_t w) {
+          const Coef32 c = ((const Coef32 *)st.coef)[w];
+          const int x = ev - c.e;  // <= 0: sigma[v] <= sigma[w]
+          if (x >= -126) sum = fmaf(c.c, __int_as_float((127 + x) << 23), sum);
+        });
+        const float df = fmaf(mv, sum, REACH ? (wt.init_d ? (float)wt.init_d[v] : (float)(wt.reach[v] - 1)) : 0.0f);
         dv = (double)df;
         if (l > 0) {
-          const float kv = IDENT ? (float)ident_i(v) : 1.0f;
+          const float kv = IDENT ? (float)wt.ident[v] : 1.0f;
           Coef32 cv;
           cv.c = fmaf(kv, df, kv) / mv;
           cv.e = ev;
@@ -438,151 +321,21 @@ __device__ void bcreach_source(const Group &g, const int32_t s, const int32_t n,
       if (v != s) acc[v] = fma(st.red[RED_WS], dv, acc[v]);
       if (dbg) dbg->delta[v] = dv;
     }
-    g.sync();
+    __syncthreads();
   }
   dag += ndag;
   if (dbg) {
-    for (int i = g.rank; i < hi; i += g.size) {
+    for (int i = rank; i < hi; i += size) {
       const int32_t v = st.queue[i];
       const int lv = d[v];
       dbg->d[v] = lv;
       dbg->sig[v] = lv < lint ? (double)sigi[v] : sig[v];
       dbg->exp[v] = st.lvl_exp[lv];
     }
-    g.sync();
-  }
-  if (RESET_BY_QUEUE) {
-    for (int i = g.rank; i < hi; i += g.size) d[st.queue[i]] = -1;
-    g.sync();
-  }
-}
-
-// ---------------------------------------------------------- small path
-__host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-
-// per group: distances and DAG masks (4 bytes each), the queue (2 bytes),
-// path counts (later the coefficients, in place) and the group's bc
-// accumulator (8 bytes each); the accumulator comes last
-__host__ __device__ inline size_t small_acc_offset(int64_t n) {
-  return align16((size_t)n * 4) * 2 + align16((size_t)n * 2) + align16((size_t)n * 8);
-}
-__host__ __device__ inline size_t small_group_bytes(int64_t n) { return small_acc_offset(n) + align16((size_t)n * 8); }
-
-// bytes of shared memory a component needs with `ng` concurrent sources:
-// the component (rows, 16-bit columns, reach and ident with their FP64 copies) once,
-// and per group the distances, queue, DAG masks, path counts / coefficients
-// and its own bc accumulator
-__host__ __device__ inline size_t small_smem_bytes(int64_t n, int64_t nnz, int ng, bool reach, bool ident) {
-  size_t b = align16((size_t)(n + 1) * 4) + align16((size_t)nnz * 2);
-  if (reach) b += align16((size_t)n * 8);
-  if (ident) b += align16((size_t)n * 8);
-  return b + small_group_bytes(n) * (size_t)ng;
-}
-
-template <bool REACH, bool IDENT, bool FP32>
-__global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
-    const SmallItem *__restrict__ items, int nitems, int *item_counter, const CompDesc *__restrict__ comps,
-    const int64_t *__restrict__ g_row, const int32_t *__restrict__ g_col, const int32_t *__restrict__ g_reach,
-    const int32_t *__restrict__ g_ident, const double *__restrict__ g_init, const int64_t *__restrict__ srcs,
-    double *bcp, int32_t *lvl_scratch, int lvl_stride, int *err, unsigned long long *dag_total) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_item;
-  __shared__ int s_next;                     // the item's next unclaimed source
-  __shared__ int s_claim[SMALL_MAX_GROUPS];  // the source each group claimed last
-  __shared__ int s_qtail[SMALL_MAX_GROUPS];
-  __shared__ double s_red[SMALL_MAX_GROUPS][16];
-  const int tid = threadIdx.x;
-  unsigned long long dag = 0;
-  for (;;) {
-    if (tid == 0) s_item = atomicAdd(item_counter, 1);
-    __syncthreads();
-    const int it = s_item;
-    __syncthreads();
-    if (it >= nitems) break;
-    const SmallItem item = items[it];
-    const CompDesc c = comps[item.comp];
-    const int n = c.n;
-    const int nnz = (int)c.nnz;
-    const int ng = item.ngroups;
-    unsigned char *p = smem;
-    int32_t *row = (int32_t *)p;
-    p += align16((size_t)(n + 1) * 4);
-    uint16_t *col = (uint16_t *)p;  // local ids of a shared-memory piece fit 16 bits
-    p += align16((size_t)nnz * 2);
-    // reach - 1 and ident as FP64 only (integers are read back from them)
-    double *init_d = nullptr, *ident_d = nullptr;
-    if (REACH) {
-      init_d = (double *)p;
-      p += align16((size_t)n * 8);
-    }
-    if (IDENT) {
-      ident_d = (double *)p;
-      p += align16((size_t)n * 8);
-    }
-    const size_t per = small_group_bytes(n);
-    const int64_t r0 = g_row[c.row_off];
-    for (int v = tid; v <= n; v += SMALL_THREADS) row[v] = (int32_t)(g_row[c.row_off + v] - r0);
-    for (int e = tid; e < nnz; e += SMALL_THREADS) col[e] = (uint16_t)g_col[r0 + e];
-    for (int v = tid; v < n; v += SMALL_THREADS) {
-      if (REACH) init_d[v] = g_init ? g_init[c.vtx_off + v] : (double)(g_reach[c.vtx_off + v] - 1);
-      if (IDENT) ident_d[v] = (double)g_ident[c.vtx_off + v];
-    }
-    if (tid == 0) s_next = item.s_begin;
-    // zero every group's accumulator
-    for (int x = tid; x < ng * n; x += SMALL_THREADS) {
-      const int gi = x / n, v = x - gi * n;
-      double *a = (double *)(p + per * gi + small_acc_offset(n));
-      a[v] = 0.0;
-    }
-    __syncthreads();
-    // whole warps per group, every warp in one: group k takes warps
-    // [k W / ng, (k + 1) W / ng), so sizes differ by at most one warp, and
-    // each group claims its next source from the item (a larger group
-    // finishes its sources sooner and takes more of them)
-    constexpr int W = SMALL_THREADS / 32;
-    const int warp = tid >> 5;
-    const int gid = ((warp + 1) * ng - 1) / W;
-    const int w0 = (gid * W) / ng, w1 = ((gid + 1) * W) / ng;
-    Group g{tid - w0 * 32, (w1 - w0) * 32, 1 + gid};
-    unsigned char *q = p + per * gid;
-    SrcState<FP32, uint16_t> st;
-    st.d = (int32_t *)q;
-    q += align16((size_t)n * 4);
-    st.queue = (uint16_t *)q;
-    q += align16((size_t)n * 2);
-    st.dmask = (uint32_t *)q;
-    q += align16((size_t)n * 4);
-    st.sig = (double *)q;
-    st.coef = (typename CoefT<FP32>::type *)q;  // same storage (see bcreach_source)
-    q += align16((size_t)n * 8);
-    double *acc = (double *)q;
-    int32_t *lv = lvl_scratch + ((size_t)blockIdx.x * SMALL_MAX_GROUPS + gid) * (size_t)lvl_stride * 2;
-    st.lvl_start = lv;
-    st.lvl_exp = lv + lvl_stride;
-    st.qtail = &s_qtail[gid];
-    st.red = s_red[gid];
-    Weights wt{nullptr, nullptr, init_d, ident_d, g_init != nullptr};
-    for (;;) {
-      // every member reads the claim before the source's first group wait,
-      // so the next claim cannot overwrite it early
-      if (g.rank == 0) s_claim[gid] = atomicAdd(&s_next, 1);
-      g.sync();
-      const int i = s_claim[gid];
-      if (i >= item.s_end) break;
-      const int32_t s = (srcs && c.src_off >= 0) ? (int32_t)srcs[c.src_off + i] : i;
-      bcreach_source<REACH, IDENT, FP32, false>(g, s, n, row, col, wt, st, acc, c.fan, err, nullptr, dag);
-    }
-    __syncthreads();
-    // add the groups' accumulators in group order and flush once
-    for (int v = tid; v < n; v += SMALL_THREADS) {
-      double t = 0.0;
-      for (int gi = 0; gi < ng; gi++)
-        t += ((const double *)(p + per * gi + small_acc_offset(n)))[v];
-      if (t != 0.0) atomicAdd(bcp + c.vtx_off + v, t);
-    }
     __syncthreads();
   }
-  if (dag_total && dag) atomicAdd(dag_total, dag);
+  for (int i = rank; i < hi; i += size) d[st.queue[i]] = -1;
+  __syncthreads();
 }
 
 // ---------------------------------------------------------- large path
@@ -612,12 +365,11 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_bcreach_large(
     Debug dbg_in, int use_dbg, unsigned long long *dag_total, int *lmax) {
   __shared__ unsigned long long s_idx;
   __shared__ int s_qtail;
-  __shared__ double s_red[16];
+  __shared__ double s_red[RED_WS + 1];
   const size_t b = blockIdx.x;
   SrcState<FP32> st;
   st.d = sc.d + b * sc.nmax;
   st.queue = sc.queue + b * sc.nmax;
-  st.dmask = nullptr;
   st.sig = sc.sig + b * sc.nmax;
   st.coef = (typename CoefT<FP32>::type *)(sc.coef + b * sc.nmax);
   double *acc = sc.acc + b * sc.nmax;
@@ -625,7 +377,6 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_bcreach_large(
   st.lvl_exp = sc.lvl_exp + b * (sc.nmax + 2);
   st.qtail = &s_qtail;
   st.red = s_red;
-  Group g{(int)threadIdx.x, (int)blockDim.x, 0};
   unsigned long long dag = 0;
   int cur = -1;
   for (;;) {
@@ -646,9 +397,9 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_bcreach_large(
     if (next < 0) break;
     const CompDesc c = comps[cur];
     Weights wt{REACH && !g_init ? g_reach + c.vtx_off : nullptr, IDENT ? g_ident + c.vtx_off : nullptr,
-               REACH && g_init ? g_init + c.vtx_off : nullptr, nullptr, g_init != nullptr};
-    bcreach_source<REACH, IDENT, FP32, true>(g, work[idx].s, c.n, g_row + c.row_off, g_col, wt, st, acc, c.fan, err,
-                                             use_dbg ? &dbg_in : nullptr, dag, lmax);
+               REACH && g_init ? g_init + c.vtx_off : nullptr};
+    bcreach_source<REACH, IDENT, FP32>(work[idx].s, g_row + c.row_off, g_col, wt, st, acc, c.fan, err,
+                                       use_dbg ? &dbg_in : nullptr, dag, lmax);
   }
   if (dag_total && dag) atomicAdd(dag_total, dag);
 }
@@ -657,25 +408,6 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_bcreach_large(
 static size_t large_scratch_bytes(int64_t nmax) { return (size_t)nmax * (4 + 4 + 8 + 8 + 8) + (size_t)(nmax + 2) * 8; }
 
 // ---------------------------------------------------------- host side
-// The shared-memory kernel's attribute (opt-in shared memory) and its
-// occupancy per shared-memory size are queried once per device and cached:
-// each query is a driver call on the host's critical path.
-static std::mutex g_small_mu;
-static std::map<long long, int> g_small_occ;  // (variant, device, smem) -> CTAs per SM
-
-template <bool R, bool I, bool F>
-static int small_prepare(int device) {
-  static std::mutex mu;
-  static std::set<int> done;
-  std::lock_guard<std::mutex> lk(mu);
-  if (!done.count(device)) {
-    BCS_CUDA(cudaFuncSetAttribute(k_bcreach_small<R, I, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)SMALL_SMEM));
-    done.insert(device);
-  }
-  return BCS_OK;
-}
-
 // The reciprocal table, filled once per device (on the legacy stream, which
 // orders it before any later work of every blocking stream).
 static int recip_table_ready(int device) {
@@ -696,40 +428,6 @@ int recip_table(Ctx &ctx, const double **out) {
   void *p = nullptr;
   BCS_CUDA(cudaGetSymbolAddress(&p, g_recip_table));
   *out = (const double *)p;
-  return BCS_OK;
-}
-
-// CTAs of the shared-memory kernel that fit on one SM with `smem` bytes each
-template <bool R, bool I, bool F>
-static int small_ctas_per_sm(int device, size_t smem, int *out) {
-  const long long key = ((long long)(R * 4 + I * 2 + F) << 48) | ((long long)device << 32) | (long long)smem;
-  {
-    std::lock_guard<std::mutex> lk(g_small_mu);
-    auto it = g_small_occ.find(key);
-    if (it != g_small_occ.end()) {
-      *out = it->second;
-      return BCS_OK;
-    }
-  }
-  BCS_TRY((small_prepare<R, I, F>(device)));
-  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bcreach_small<R, I, F>, SMALL_THREADS, smem));
-  if (*out < 1) *out = 1;
-  std::lock_guard<std::mutex> lk(g_small_mu);
-  g_small_occ[key] = *out;
-  return BCS_OK;
-}
-
-template <bool R, bool I, bool F>
-static int launch_small_t(Ctx &ctx, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
-                          const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *lvl, int lvl_stride,
-                          int *err, unsigned long long *dag) {
-  BCS_TRY((small_prepare<R, I, F>(ctx.device)));
-  BCS_TRY(recip_table_ready(ctx.device));
-  auto kern = k_bcreach_small<R, I, F>;
-  kern<<<grid, SMALL_THREADS, smem, ctx.stream>>>(items, nitems, counter, comps, in.row, in.col, in.reach, in.ident,
-                                                 in.init, srcs, in.bcp, lvl, lvl_stride, err, dag);
-  ctx.launches++;
-  BCS_CUDA(cudaGetLastError());
   return BCS_OK;
 }
 
@@ -923,7 +621,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       const int64_t ns = nsrc_of(c);
       if (c.n < 2 || ns == 0 || c.n > 65535) continue;
       const size_t s1 = small_smem_bytes(c.n, c.nnz, 1, R, I);
-      if (s1 > SMALL_SMEM) continue;
+      if (s1 > SMALL_SMEM || !small_takes(c.n, c.nnz, 1)) continue;
       elig.push_back(c);
       cost += (double)ns * (double)(c.nnz + c.n);
       if (s1 > lowest) band += (double)ns * (double)(c.nnz + c.n);
@@ -957,6 +655,18 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   std::vector<int32_t> large, small;
   int64_t nmax_large = 0, nmax_small = 0;
   double work_se = 0.0, work_sv = 0.0, total_small_cost = 0.0;
+  std::vector<int32_t> mids;  // pieces of the small path that the pull kernel may take instead
+  const bool mid_rule = !tune && !po.small_limit && lp_mode == LARGE_PATH_AUTO && !dbg && !po.per_source_large;
+  auto small_takes_sources = [&](const CompDesc &c, int g) {
+    return small_takes(c.n, c.nnz, g) && small_smem_bytes(c.n, c.nnz, g, R, I) <= SMALL_BUDGET;
+  };
+  auto pull_rows = [&](const CompDesc &c) { return (nsrc_of(c) + 255) / 256 * (int64_t)c.n; };
+  auto to_small = [&](int32_t ci) {
+    const CompDesc &c = comps[ci];
+    small.push_back(ci);
+    total_small_cost += (double)nsrc_of(c) * (double)(c.nnz + c.n);
+    nmax_small = std::max<int64_t>(nmax_small, c.n);
+  };
   for (int64_t ci = 0; ci < C; ci++) {
     const CompDesc &c = comps[ci];
     if (c.n < 2) continue;
@@ -965,71 +675,24 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     work_se += (double)ns * (double)c.nnz;
     work_sv += (double)ns * (double)c.n;
     const bool fits = !po.force_large && !all_large && !dbg && c.n <= 65535 &&
-                      small_smem_bytes(c.n, c.nnz, 1, R, I) <= small_limit;
-    if (fits) {
-      small.push_back((int32_t)ci);
-      total_small_cost += (double)ns * (double)(c.nnz + c.n);
-      nmax_small = std::max<int64_t>(nmax_small, c.n);
+                      small_takes(c.n, c.nnz, 1) && small_smem_bytes(c.n, c.nnz, 1, R, I) <= small_limit;
+    if (fits && mid_rule && !small_takes_sources(c, MID_SOURCES)) {
+      mids.push_back((int32_t)ci);
+    } else if (fits) {
+      to_small((int32_t)ci);
     } else {
       large.push_back((int32_t)ci);
       nmax_large = std::max<int64_t>(nmax_large, c.n);
     }
   }
-  // The small-path work split: a piece runs up to `ng_cap` sources at once
-  // per CTA (the most that fit in SMALL_SMEM); the launch takes exactly the
-  // shared memory its largest item needs, so occupancy follows the plan.
-  // Items of similar cost go first-largest into a persistent queue.
-  // pieces by cost class (the power of two of n + nnz), largest first, in
-  // piece order within a class: the persistent queue hands out the longest
-  // items first.  A counting sort: one pass, no comparisons.
   {
-    int64_t cnt[65] = {0};
-    std::vector<int32_t> cls(small.size());
-    for (size_t k = 0; k < small.size(); k++) {
-      const CompDesc &c = comps[small[k]];
-      cls[k] = 63 - __builtin_clzll((unsigned long long)(c.nnz + c.n) | 1ull);
-      cnt[cls[k]]++;
+    int64_t rows = 0;
+    for (int32_t ci : mids) rows += pull_rows(comps[ci]);
+    if (rows < MID_MIN_ROWS) {
+      for (int32_t ci : mids) to_small(ci);
+      mids.clear();
     }
-    int64_t off[65], o = 0;
-    for (int b = 64; b >= 0; b--) {
-      off[b] = o;
-      o += cnt[b];
-    }
-    std::vector<int32_t> sorted(small.size());
-    for (size_t k = 0; k < small.size(); k++) sorted[off[cls[k]]++] = small[k];
-    small.swap(sorted);
   }
-  auto plan_small = [&](int ng_cap, size_t budget, std::vector<SmallItem> &out, size_t &smem, int &grid) -> int {
-    out.clear();
-    smem = 0;
-    std::vector<int> ngs(small.size());
-    for (size_t k = 0; k < small.size(); k++) {
-      const CompDesc &c = comps[small[k]];
-      int ng = 1;  // a piece that does not fit the budget even alone still runs (up to SMALL_SMEM)
-      for (int cand = ng_cap; cand >= 1; cand--)
-        if (small_smem_bytes(c.n, c.nnz, cand, R, I) <= budget) {
-          ng = cand;
-          break;
-        }
-      ngs[k] = ng;
-      smem = std::max(smem, small_smem_bytes(c.n, c.nnz, ng, R, I));
-    }
-    int per_sm = 1;
-    BCS_TRY(BCS_DISPATCH3(small_ctas_per_sm, R, I, F, ctx.device, smem, &per_sm));
-    grid = ctx.num_sms * per_sm;
-    const double target = total_small_cost / (double)((int64_t)grid * SMALL_MAX_GROUPS) + 1.0;
-    for (size_t k = 0; k < small.size(); k++) {
-      const CompDesc &c = comps[small[k]];
-      const int ng = ngs[k];
-      const int64_t ns = nsrc_of(c);
-      int64_t chunk = (int64_t)std::max(1.0, target / (double)(c.nnz + c.n));
-      chunk = ((chunk + ng - 1) / ng) * ng;
-      for (int64_t b = 0; b < ns; b += chunk)
-        out.push_back(SmallItem{small[k], (int32_t)b, (int32_t)std::min<int64_t>(ns, b + chunk), ng});
-    }
-    grid = (int)std::min<int64_t>(grid, (int64_t)out.size());
-    return BCS_OK;
-  };
   // Large pieces of small BFS depth: the pull kernel, the sources of a piece
   // taken in the order of its BFS from its first vertex (neighbouring sources
   // share most of their levels).  That search also bounds the depth: no source
@@ -1037,7 +700,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   // every large piece whose depth allows it, mid the connected ones of at most
   // MID_MAX_N vertices; batched|per_source take none.
   DBuf<CompDesc> d_comps;
-  if (!small.empty() || !large.empty()) {
+  if (!small.empty() || !large.empty() || !mids.empty()) {
     BCS_TRY(d_comps.alloc(C, ctx.stream));
     BCS_CUDA(cudaMemcpyAsync(d_comps.p, comps.data(), C * sizeof(CompDesc), cudaMemcpyHostToDevice, ctx.stream));
   }
@@ -1068,13 +731,23 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       off.push_back(total);
       total += c.n + (po.sources ? po.nsources : 0);
     }
+    const size_t nlarge = cand.size();
+    for (int32_t ci : mids) {
+      if (comps[ci].src_off >= 0) {
+        to_small(ci);
+        continue;
+      }
+      cand.push_back(ci);
+      off.push_back(total);
+      total += comps[ci].n;
+    }
     if (!cand.empty()) {
       BCS_TRY(pull_order.alloc(total, ctx.stream));
       BCS_TRY(pull_parent.alloc(total, ctx.stream));
     }
     std::vector<int32_t> cta_depth, cta_reached;
     BCS_TRY(piece_bfs(ctx, comps, d_comps.p, cand, in, off, pull_order.p, pull_parent.p, &cta_depth, &cta_reached));
-    for (size_t k = 0; k < cand.size(); k++) {
+    for (size_t k = 0; k < nlarge; k++) {
       const int32_t ci = cand[k];
       const CompDesc &c = comps[ci];
       int32_t *const ord = pull_order.p + off[k];
@@ -1137,7 +810,71 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       else deep.push_back(DeepJob{ci, (int32_t)nsrc_of(c), bound, off[k], src_off});
     }
     large.swap(rest);
+    int64_t rows = 0;
+    auto shallow = [&](size_t k) { return cta_reached[k] == comps[cand[k]].n && cta_depth[k] <= MID_PIECE_ECC; };
+    for (size_t k = nlarge; k < cand.size(); k++)
+      if (shallow(k)) rows += pull_rows(comps[cand[k]]);
+    for (size_t k = nlarge; k < cand.size(); k++) {
+      const int32_t ci = cand[k];
+      if (rows < MID_MIN_ROWS || !shallow(k)) to_small(ci);
+      else pull.push_back(PullJob{ci, (int32_t)nsrc_of(comps[ci]), 2 * cta_depth[k] + 2, off[k]});
+    }
   }
+  // The small-path work split: a piece runs up to `ng_cap` sources at once
+  // per CTA (the most that fit in SMALL_SMEM); the launch takes exactly the
+  // shared memory its largest item needs, so occupancy follows the plan.
+  // Items of similar cost go first-largest into a persistent queue.
+  // pieces by cost class (the power of two of n + nnz), largest first, in
+  // piece order within a class: the persistent queue hands out the longest
+  // items first.  A counting sort: one pass, no comparisons.
+  {
+    int64_t cnt[65] = {0};
+    std::vector<int32_t> cls(small.size());
+    for (size_t k = 0; k < small.size(); k++) {
+      const CompDesc &c = comps[small[k]];
+      cls[k] = 63 - __builtin_clzll((unsigned long long)(c.nnz + c.n) | 1ull);
+      cnt[cls[k]]++;
+    }
+    int64_t off[65], o = 0;
+    for (int b = 64; b >= 0; b--) {
+      off[b] = o;
+      o += cnt[b];
+    }
+    std::vector<int32_t> sorted(small.size());
+    for (size_t k = 0; k < small.size(); k++) sorted[off[cls[k]]++] = small[k];
+    small.swap(sorted);
+  }
+  auto plan_small = [&](int ng_cap, size_t budget, std::vector<SmallItem> &out, size_t &smem, int &grid) -> int {
+    out.clear();
+    smem = 0;
+    std::vector<int> ngs(small.size());
+    for (size_t k = 0; k < small.size(); k++) {
+      const CompDesc &c = comps[small[k]];
+      int ng = 1;  // a piece that does not fit the budget even alone still runs (up to SMALL_SMEM)
+      for (int cand = ng_cap; cand >= 1; cand--)
+        if (small_takes(c.n, c.nnz, cand) && small_smem_bytes(c.n, c.nnz, cand, R, I) <= budget) {
+          ng = cand;
+          break;
+        }
+      ngs[k] = ng;
+      smem = std::max(smem, small_smem_bytes(c.n, c.nnz, ng, R, I));
+    }
+    int per_sm = 1;
+    BCS_TRY(small_ctas_per_sm(ctx, R, I, F, smem, &per_sm));
+    grid = ctx.num_sms * per_sm;
+    const double target = total_small_cost / (double)((int64_t)grid * 8) + 1.0;
+    for (size_t k = 0; k < small.size(); k++) {
+      const CompDesc &c = comps[small[k]];
+      const int ng = ngs[k];
+      const int64_t ns = nsrc_of(c);
+      int64_t chunk = (int64_t)std::max(1.0, target / (double)(c.nnz + c.n));
+      chunk = ((chunk + ng - 1) / ng) * ng;
+      for (int64_t b = 0; b < ns; b += chunk)
+        out.push_back(SmallItem{small[k], (int32_t)b, (int32_t)std::min<int64_t>(ns, b + chunk), ng});
+    }
+    grid = (int)std::min<int64_t>(grid, (int64_t)out.size());
+    return BCS_OK;
+  };
   nmax_large = 0;  // of what is left for the kernels below
   for (int32_t ci : large) nmax_large = std::max<int64_t>(nmax_large, comps[ci].n);
   for (int32_t ci : ms_tuned) nmax_large = std::max<int64_t>(nmax_large, comps[ci].n);
@@ -1194,8 +931,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   };
   if (!use_ms) build_work(0);
   tr.mark("classify");
-  int ng_cap = SMALL_MAX_GROUPS;
-  size_t budget = SMALL_SMEM;
+  int ng_cap = small_max_sources();
+  size_t budget = SMALL_BUDGET;
   size_t smem_small = 0;
   int grid_small = 0;
   // the autotuner's choice for this shape bucket, if it has one already
@@ -1239,10 +976,9 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   if (!items.empty()) {
     StageTimer tm(ctx.stream);
     tm.start();
-    const int lvl_stride = (int)nmax_small + 2;
-    const size_t grid_cap = (size_t)ctx.num_sms * (2048 / SMALL_THREADS);  // resident CTAs per SM at most
+    const size_t grid_cap = (size_t)ctx.num_sms * 8;  // resident CTAs per SM at most
     DBuf<int32_t> lvl;
-    BCS_TRY(lvl.alloc(grid_cap * SMALL_MAX_GROUPS * lvl_stride * 2, ctx.stream));
+    BCS_TRY(lvl.alloc(small_scratch_words(grid_cap, nmax_small), ctx.stream));
     DBuf<SmallItem> d_items;
     BCS_TRY(d_items.alloc(std::max<size_t>(items.size() * 2, 1), ctx.stream));
     auto run_small = [&](const std::vector<SmallItem> &its, size_t smem, int grid, double *target) -> int {
@@ -1252,8 +988,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       BCS_CUDA(cudaMemsetAsync(d_err.p + 1, 0, sizeof(int), ctx.stream));
       BcInput tin = in;
       tin.bcp = target;
-      return BCS_DISPATCH3(launch_small_t, R, I, F, ctx, grid, smem, d_items.p, (int)its.size(), d_err.p + 1,
-                           d_comps.p, tin, po.sources ? d_srcs.p : po.srcmap, lvl.p, lvl_stride, d_err.p, d_dag.p);
+      return launch_small(ctx, F, grid, smem, d_items.p, (int)its.size(), d_err.p + 1, d_comps.p, tin,
+                          po.sources ? d_srcs.p : po.srcmap, lvl.p, nmax_small, d_err.p, d_dag.p);
     };
     tr.mark("alloc");
     if (ctx.autotune && tuned == 0) {

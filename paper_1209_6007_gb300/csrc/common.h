@@ -325,6 +325,25 @@ struct PullJob {
 int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<PullJob> &jobs, const BcInput &in,
              bool fp32, const int32_t *d_order, const CompDesc *d_comps, int per_batch, int *d_err,
              unsigned long long *d_dag);
+// Bc-Reach on pieces that fit shared memory (small.cu): one persistent launch
+// over items, each a range of a piece's sources, ngroups of them searched at
+// once.  small_smem_bytes: shared memory a piece takes with G sources at once;
+// small_takes: whether its offsets and queue places fit 16 bits.
+constexpr size_t SMALL_SMEM = 100 * 1024;  // most shared memory of a CTA
+struct SmallItem {
+  int32_t comp;
+  int32_t s_begin;  // index range into the source list (or local ids)
+  int32_t s_end;
+  int32_t ngroups;
+};
+size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident);
+bool small_takes(int64_t n, int64_t nnz, int G);
+int small_max_sources();
+int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, size_t smem, int *out);
+size_t small_scratch_words(int64_t ctas, int64_t nmax);  // level offsets and exponents
+int launch_small(Ctx &ctx, bool fp32, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
+                 const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
+                 int *err, unsigned long long *dag);
 // device address of the reciprocals of the integers below RECIP_TABLE
 constexpr int RECIP_TABLE = 1024;
 int recip_table(Ctx &ctx, const double **out);
