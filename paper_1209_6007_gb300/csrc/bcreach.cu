@@ -52,10 +52,6 @@ constexpr int MS_DEPTH_LIMIT = 64;
 constexpr int PULL_MAX_ECC = 40;
 // and deeper ones than this, of small degree, on the deep kernel (deep.cu)
 constexpr int DEEP_MIN_ECC = 40;
-// The shared memory a small-path CTA gets without the autotuner: four CTAs of
-// an SM's 227 KB (articulation-vertex workload, 130 M (vertex, source) pairs:
-// 5.0 ms; with 72 KB 5.1, with 100 KB 5.8 to 7.9, with 36 KB 6.2)
-constexpr size_t SMALL_BUDGET = 54 * 1024;
 // Pieces that cannot run MID_SOURCES sources at once in that budget (some 800
 // vertices and more) go to the pull kernel instead, if they are shallow and
 // come in numbers: its cost is per level and slab (256 sources of a piece), so
@@ -844,10 +840,19 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     for (size_t k = 0; k < small.size(); k++) sorted[off[cls[k]]++] = small[k];
     small.swap(sorted);
   }
+  bool small_coop = false;
+  int64_t small_sources = 0;
+  for (int32_t ci : small) {
+    small_coop = small_coop || comps[ci].maxdeg > SMALL_COOP_DEG;
+    small_sources += nsrc_of(comps[ci]);
+  }
   auto plan_small = [&](int ng_cap, size_t budget, std::vector<SmallItem> &out, size_t &smem, int &grid) -> int {
     out.clear();
     smem = 0;
     std::vector<int> ngs(small.size());
+    // no more sources at once than leave every SM two items (a graph of 312
+    // vertices: 83 us with seven at once on 45 SMs, 47 with one)
+    ng_cap = (int)std::max<int64_t>(1, std::min<int64_t>(ng_cap, small_sources / (2 * (int64_t)ctx.num_sms)));
     for (size_t k = 0; k < small.size(); k++) {
       const CompDesc &c = comps[small[k]];
       int ng = 1;  // a piece that does not fit the budget even alone still runs (up to SMALL_SMEM)
@@ -860,7 +865,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       smem = std::max(smem, small_smem_bytes(c.n, c.nnz, ng, R, I));
     }
     int per_sm = 1;
-    BCS_TRY(small_ctas_per_sm(ctx, R, I, F, smem, &per_sm));
+    BCS_TRY(small_ctas_per_sm(ctx, R, I, F, small_coop, smem, &per_sm));
     grid = ctx.num_sms * per_sm;
     const double target = total_small_cost / (double)((int64_t)grid * 8) + 1.0;
     for (size_t k = 0; k < small.size(); k++) {
@@ -988,7 +993,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       BCS_CUDA(cudaMemsetAsync(d_err.p + 1, 0, sizeof(int), ctx.stream));
       BcInput tin = in;
       tin.bcp = target;
-      return launch_small(ctx, F, grid, smem, d_items.p, (int)its.size(), d_err.p + 1, d_comps.p, tin,
+      return launch_small(ctx, F, small_coop, grid, smem, d_items.p, (int)its.size(), d_err.p + 1, d_comps.p, tin,
                           po.sources ? d_srcs.p : po.srcmap, lvl.p, nmax_small, d_err.p, d_dag.p);
     };
     tr.mark("alloc");
@@ -1171,80 +1176,5 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
 // caller-given scratch region instead of allocated.  Used by the
 // allocation-free entry point.
 
-__global__ void k_fixed_setup(LargeSrc *work, int32_t n, CompDesc *comp, CompDesc desc,
-                              unsigned long long *counter, int *err) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) work[i] = LargeSrc{0, i};
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *comp = desc;
-    *counter = 0ull;
-    *err = 0;
-  }
-}
-
-static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
-static_assert(sizeof(LargeSrc) == FIXED_WORK_ITEM_BYTES, "work item size");
-static_assert(sizeof(CompDesc) <= 256, "component descriptor size");
-
-int launch_plain_fixed_scratch(Ctx &ctx, const int64_t *row, const int32_t *col, int32_t n, double *bc,
-                               unsigned char *scratch, int64_t nmax, int ctas, bool fp32) {
-  const size_t G = (size_t)ctas, N = (size_t)nmax;
-  unsigned char *p = scratch;
-  LargeSrc *work = (LargeSrc *)p;
-  p += up256(N * sizeof(LargeSrc));
-  CompDesc *comp = (CompDesc *)p;
-  p += up256(sizeof(CompDesc));
-  unsigned long long *counter = (unsigned long long *)p;
-  p += 256;
-  int *err = (int *)p;
-  p += 256;
-  if (p != scratch + fixed_scratch_arrays_offset(N)) {
-    set_error("fixed scratch layout mismatch");
-    return BCS_ECUDA;
-  }
-  LargeScratch sc;
-  sc.nmax = (int64_t)N;
-  sc.d = (int32_t *)p;
-  p += up256(G * N * 4);
-  sc.queue = (int32_t *)p;
-  p += up256(G * N * 4);
-  sc.sig = (double *)p;
-  p += up256(G * N * 8);
-  sc.coef = (double *)p;
-  p += up256(G * N * 8);
-  sc.acc = (double *)p;
-  p += up256(G * N * 8);
-  sc.lvl_start = (int32_t *)p;
-  p += up256(G * (N + 2) * 4);
-  sc.lvl_exp = (int32_t *)p;
-  // the region keeps whatever the previous call left: put back the states
-  // the kernel expects at its start (d = -1, sigma = 0, accumulators 0)
-  BCS_CUDA(cudaMemsetAsync(sc.d, 0xFF, G * N * 4, ctx.stream));
-  BCS_CUDA(cudaMemsetAsync(sc.sig, 0, G * N * 8, ctx.stream));
-  BCS_CUDA(cudaMemsetAsync(sc.acc, 0, G * N * 8, ctx.stream));
-  BCS_CUDA(cudaMemsetAsync(bc, 0, (size_t)n * sizeof(double), ctx.stream));
-  // n bounds the degree, hence the growth of path counts per level
-  CompDesc desc{0, 0, n, n, 0, (double)(n > 1 ? n : 1)};
-  k_fixed_setup<<<(n + 255) / 256, 256, 0, ctx.stream>>>(work, n, comp, desc, counter, err);
-  ctx.launches++;
-  BCS_CUDA(cudaGetLastError());
-  Debug none{nullptr, nullptr, nullptr, nullptr};
-  BcInput in;
-  in.row = row;
-  in.col = col;
-  in.bcp = bc;
-  const int grid = (int)std::min<int64_t>(ctas, n);
-  if (fp32)
-    BCS_TRY((launch_large_t<false, false, true>(ctx, grid, work, n, counter, comp, in, sc, err, none, 0, nullptr)));
-  else
-    BCS_TRY((launch_large_t<false, false, false>(ctx, grid, work, n, counter, comp, in, sc, err, none, 0, nullptr)));
-  int h_err = 0;
-  BCS_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
-  BCS_CUDA(cudaStreamSynchronize(ctx.stream));
-  if (h_err & ERR_OVERFLOW) {
-    set_error("shortest-path counts overflowed the FP64 range within one BFS level");
-    return BCS_EOVERFLOW;
-  }
-  return BCS_OK;
-}
 
 }  // namespace bcs

@@ -330,6 +330,10 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
 // once.  small_smem_bytes: shared memory a piece takes with G sources at once;
 // small_takes: whether its offsets and queue places fit 16 bits.
 constexpr size_t SMALL_SMEM = 100 * 1024;  // most shared memory of a CTA
+// The shared memory a small-path CTA gets without the autotuner: four CTAs of
+// an SM's 227 KB (articulation-vertex workload, 130 M (vertex, source) pairs:
+// 5.0 ms; with 72 KB 5.1, with 100 KB 5.8 to 7.9, with 36 KB 6.2)
+constexpr size_t SMALL_BUDGET = 54 * 1024;
 struct SmallItem {
   int32_t comp;
   int32_t s_begin;  // index range into the source list (or local ids)
@@ -339,9 +343,13 @@ struct SmallItem {
 size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident);
 bool small_takes(int64_t n, int64_t nnz, int G);
 int small_max_sources();
-int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, size_t smem, int *out);
+int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, bool coop, size_t smem, int *out);
 size_t small_scratch_words(int64_t ctas, int64_t nmax);  // level offsets and exponents
-int launch_small(Ctx &ctx, bool fp32, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
+// coop: long rows are taken by whole warps; pays when some row is longer than
+// SMALL_COOP_DEG (1,370 vertices, hubs of 90: 0.29 to 0.26 ms; a batch of small
+// graphs with rows up to 60: 0.50 to 0.62)
+constexpr int SMALL_COOP_DEG = 64;
+int launch_small(Ctx &ctx, bool fp32, bool coop, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
                  const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
                  int *err, unsigned long long *dag);
 // device address of the reciprocals of the integers below RECIP_TABLE
@@ -392,20 +400,11 @@ int run_bcreach_side(Ctx &ctx, const DevMerged &m, const std::vector<CompDesc> &
 }  // namespace bcs
 
 namespace bcs {
-// Plain Brandes over one component with all device state carved out of
-// `scratch` (fixed_scratch_bytes(nmax, ctas) bytes); allocates nothing.
-constexpr size_t FIXED_WORK_ITEM_BYTES = 8;
+// Plain Brandes over one graph of at most 16,384 vertices with all device
+// state in `scratch` (`bytes` of it); allocates nothing (small.cu).  The word
+// at FIXED_ERR, reset by the launcher, may serve as a flag before the launch.
+constexpr size_t FIXED_ERR = 512, FIXED_HEAD = 768;
 constexpr size_t fixed_up256(size_t x) { return (x + 255) & ~(size_t)255; }
-// Layout of the region, in order: work items (nmax), the component
-// descriptor, the work counter and the error word (256 bytes each), then the
-// per-CTA arrays.  fixed_scratch_arrays_offset(nmax) is where the per-CTA
-// arrays start; the first of them (distances, reset by the launcher) may
-// serve as a one-word flag before the launch.
-constexpr size_t fixed_scratch_arrays_offset(size_t nmax) { return fixed_up256(nmax * FIXED_WORK_ITEM_BYTES) + 3 * 256; }
-constexpr size_t fixed_scratch_bytes(size_t nmax, size_t ctas) {
-  return fixed_scratch_arrays_offset(nmax) + fixed_up256(ctas * nmax * 4) * 2 + fixed_up256(ctas * nmax * 8) * 3 +
-         fixed_up256(ctas * (nmax + 2) * 4) * 2;
-}
-int launch_plain_fixed_scratch(Ctx &ctx, const int64_t *row, const int32_t *col, int32_t n, double *bc,
-                               unsigned char *scratch, int64_t nmax, int ctas, bool fp32);
+int launch_plain_fixed_scratch(Ctx &ctx, const int64_t *row, const int32_t *col, int32_t n, int64_t nnz, double *bc,
+                               unsigned char *scratch, size_t bytes, bool fp32);
 }  // namespace bcs

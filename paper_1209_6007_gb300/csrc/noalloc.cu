@@ -14,8 +14,7 @@
 namespace bcs {
 
 constexpr int64_t NOALLOC_MAX_N = BCS_NOALLOC_MAX_N;  // vertices
-constexpr int NOALLOC_CTAS = 64;                      // CTAs sharing the scratch
-constexpr size_t NOALLOC_BYTES = fixed_scratch_bytes(NOALLOC_MAX_N, NOALLOC_CTAS);
+constexpr size_t NOALLOC_BYTES = 42 * 1000 * 1000 / 256 * 256;  // shared by a call's CTAs (80 at the largest graph)
 
 // The scratch.  In host code this name is only a host-side stand-in for the
 // array; its device address comes from cudaGetSymbolAddress below.
@@ -89,10 +88,9 @@ extern "C" __attribute__((visibility("default"))) int bcs_bc_plain_noalloc(const
     unsigned char *scratch = nullptr;
     rc = noalloc_scratch(ctx.device, &scratch);
     if (rc == BCS_OK) {
-      // The CSR check needs one int of device memory: it borrows the first
-      // word of the per-CTA distance arrays, which the launcher
-      // re-initialises right after.
-      int *flags = (int *)(scratch + fixed_scratch_arrays_offset(NOALLOC_MAX_N));
+      // The CSR check needs one int of device memory: it borrows the error
+      // word, which the launcher resets right after.
+      int *flags = (int *)(scratch + FIXED_ERR);
       DevGraph g;
       g.n = csr->n;
       g.nnz = csr->nnz;
@@ -111,8 +109,8 @@ extern "C" __attribute__((visibility("default"))) int bcs_bc_plain_noalloc(const
         }
       }
       if (rc == BCS_OK)
-        rc = launch_plain_fixed_scratch(ctx, csr->row_ptr, csr->col, (int32_t)csr->n, bc_out, scratch,
-                                        NOALLOC_MAX_N, NOALLOC_CTAS, opts && opts->delta_fp32);
+        rc = launch_plain_fixed_scratch(ctx, csr->row_ptr, csr->col, (int32_t)csr->n, csr->nnz, bc_out, scratch,
+                                        NOALLOC_BYTES, opts && opts->delta_fp32);
     }
   }
   if (prev >= 0) cudaSetDevice(prev);

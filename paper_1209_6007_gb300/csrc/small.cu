@@ -46,8 +46,12 @@
 namespace bcs {
 
 constexpr int SMALL_THREADS = 320;
+constexpr int SMALL_GLOBAL_THREADS = 512;
+constexpr int SMALL_LONGS = 8;    // long rows of a warp's pairs taken by the whole warp, at most
 constexpr int SMALL_MAX_G = 16;   // sources per CTA at once, at most (two bits each in a word)
-constexpr int SMALL_FLUSH = 16;   // rounds of G sources between additions to bc'
+// rounds of G sources between additions to bc': both chains of additions stay short
+__host__ __device__ constexpr int small_flush(bool global) { return global ? 64 : 16; }
+constexpr int FIXED_COPIES = 32;  // of bc', in the fixed-scratch launch
 constexpr int SMALL_LEVELS = 64;  // level offsets kept in shared memory, the rest in global scratch
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -69,13 +73,20 @@ bool small_takes(int64_t n, int64_t nnz, int G) {
 }
 int small_max_sources() { return SMALL_MAX_G; }
 
-template <bool REACH, bool IDENT, bool FP32>
-__global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
+// COOP: where a warp's pairs have at most SMALL_LONGS rows of more than 32
+// entries, the warp takes those together: a hub's row taken by one lane holds
+// up the level.  Where no row is long the ballots and the registers cost more
+// than they give (articulation-vertex workload: 5.0 ms without, 6.2 with).
+// GLOBAL (a piece above shared memory, G = 1): codes and queue in shared
+// memory, the counts and sums in global memory (`state`), the rows the caller's.
+template <bool REACH, bool IDENT, bool FP32, bool COOP, bool GLOBAL>
+__global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, GLOBAL ? 2 : COOP ? 4 : 0) k_bcreach_small(
     const SmallItem *__restrict__ items, int nitems, int *item_counter, const CompDesc *__restrict__ comps,
     const int64_t *__restrict__ g_row, const int32_t *__restrict__ g_col, const int32_t *__restrict__ g_reach,
     const int32_t *__restrict__ g_ident, const double *__restrict__ g_init, const int64_t *__restrict__ srcs,
-    const double *__restrict__ recip, double *bcp, int32_t *lvl_scratch, int lvl_stride, int *err,
-    unsigned long long *dag_total) {
+    const double *__restrict__ recip, double *bcp, size_t bcp_stride, int32_t *lvl_scratch, int lvl_stride, int lvl_G,
+    unsigned char *state, size_t state_stride, int *err, unsigned long long *dag_total) {
+  constexpr int NT = GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_max[SMALL_MAX_G];  // largest count of each source on the level, as bits
   __shared__ double s_ws[SMALL_MAX_G];
@@ -85,8 +96,10 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
   __shared__ int s_lvl[SMALL_LEVELS];
   __shared__ int s_item, s_tail, s_top;
   const int tid = threadIdx.x, lane = tid & 31;
-  int32_t *const lvl_far = lvl_scratch + (size_t)blockIdx.x * lvl_stride * (SMALL_MAX_G + 1);
+  const int tid0 = COOP ? tid & ~31 : tid;  // COOP: whole warps run through a level together
+  int32_t *const lvl_far = lvl_scratch + (size_t)blockIdx.x * lvl_stride * (lvl_G + 1);
   int32_t *const exps = lvl_far + lvl_stride;  // [level][G]
+  double *const bcp_cta = bcp + bcp_stride * (blockIdx.x % FIXED_COPIES);  // stride 0: one bc' for all
   unsigned long long dag = 0;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(item_counter, 1);
@@ -99,11 +112,16 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
     const uint32_t G = (uint32_t)item.ngroups;
     const int gs = 32 - __clz((int)G - 1);  // ceil(log2 G) (G = 1: 0)
     const uint32_t gmask = (1u << gs) - 1u;
-    unsigned char *p = smem;
-    uint16_t *const row = (uint16_t *)p;
-    p += align16((size_t)(n + 1) * 2);
-    uint16_t *const col = (uint16_t *)p;
-    p += align16((size_t)(nnz + 3) * 2);
+    unsigned char *p = GLOBAL ? state + state_stride * blockIdx.x : smem;
+    uint16_t *row = nullptr, *col = nullptr;
+    if (!GLOBAL) {
+      row = (uint16_t *)p;
+      p += align16((size_t)(n + 1) * 2);
+      col = (uint16_t *)p;
+      p += align16((size_t)(nnz + 3) * 2);
+    }
+    auto row_of = [&](uint32_t v) -> int { return GLOBAL ? (int)__ldg(g_row + v) : (int)row[v]; };
+    auto col_at = [&](int e) -> uint32_t { return GLOBAL ? (uint32_t)__ldg(g_col + e) : (uint32_t)col[e]; };
     double *init = nullptr;
     int32_t *ident = nullptr;
     if (REACH) {
@@ -114,8 +132,8 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
       ident = (int32_t *)p;
       p += align16((size_t)n * 4);
     }
-    uint32_t *const code = (uint32_t *)p;
-    p += align16((size_t)n * 4);
+    uint32_t *const code = (uint32_t *)(GLOBAL ? smem : p);
+    if (!GLOBAL) p += align16((size_t)n * 4);
     const size_t pairs = (size_t)n * G;
     double *const S = (double *)p;
     long long *const Si = (long long *)p;
@@ -124,22 +142,24 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
     p += align16(pairs * 8);
     uint32_t *const succ_of = (uint32_t *)p;
     p += align16(pairs * 4);
-    uint16_t *const Q = (uint16_t *)p;
-    const int64_t *const grow = g_row + c.row_off;
-    const int64_t r0 = grow[0];
-    for (int v = tid; v <= n; v += SMALL_THREADS) row[v] = (uint16_t)(grow[v] - r0);
-    for (int e = tid; e < nnz + 3; e += SMALL_THREADS) col[e] = e < nnz ? (uint16_t)__ldg(g_col + r0 + e) : (uint16_t)0;
-    for (int v = tid; v < n; v += SMALL_THREADS) {
+    uint16_t *const Q = (uint16_t *)(GLOBAL ? smem + align16((size_t)n * 4) : p);
+    if (!GLOBAL) {
+      const int64_t *const grow = g_row + c.row_off;
+      const int64_t r0 = grow[0];
+      for (int v = tid; v <= n; v += NT) row[v] = (uint16_t)(grow[v] - r0);
+      for (int e = tid; e < nnz + 3; e += NT) col[e] = e < nnz ? (uint16_t)__ldg(g_col + r0 + e) : (uint16_t)0;
+    }
+    for (int v = tid; v < n; v += NT) {
       if (REACH) init[v] = g_init ? g_init[c.vtx_off + v] : (double)(g_reach[c.vtx_off + v] - 1);
       if (IDENT) ident[v] = g_ident[c.vtx_off + v];
     }
-    for (uint32_t x = tid; x < (uint32_t)pairs; x += SMALL_THREADS) acc[x] = 0.0;
+    for (uint32_t x = tid; x < (uint32_t)pairs; x += NT) acc[x] = 0.0;
     // bound on the growth of a level's stored counts: the degree, and ident (at most a degree)
     const int flg = max(1, ceil_log2_pos(c.fan) * (IDENT ? 2 : 1));
     int rounds = 0;
     for (int first = item.s_begin; first < item.s_end; first += (int)G) {
       const int cnt = min((int)G, item.s_end - first);
-      for (int i = tid; i < n; i += SMALL_THREADS) code[i] = 0u;
+      for (int i = tid; i < n; i += NT) code[i] = 0u;
       __syncthreads();  // the piece is loaded; the codes are clear
       if (tid < cnt) {
         const int i = first + tid;
@@ -171,46 +191,82 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
         // mode 0: integer counts, 1: FP64 from the integers of the level above, 2: FP64
         auto pass = [&](auto mode) {
           constexpr int MODE = decltype(mode)::value;
-          for (int i = lo + tid; i < hi; i += SMALL_THREADS) {
-            const uint32_t it = Q[i], v = it >> gs, g = it & gmask, x = v * G + g;
+          for (int i0 = lo + tid0; i0 < hi; i0 += NT) {
+            const int i = COOP ? i0 + lane : i0;
+            const bool valid = !COOP || i < hi;
+            const uint32_t it = valid ? Q[i] : 0u, v = it >> gs, g = it & gmask, x = v * G + g;
             const uint32_t sh = 2 * g, field = 3u << sh, above = cp << sh, same = cc << sh;
-            const int qb = row[v], qe = row[v + 1];
-            const double *const Sg = S + g;
+            const int rb = valid ? row_of(v) : 0, re = valid ? row_of(v + 1) : 0;
+            unsigned longs = COOP ? __ballot_sync(0xffffffffu, re - rb > 32) : 0u;
+            if (COOP && __popc(longs) > SMALL_LONGS) longs = 0u;
             long long ai = 0;
             double ad = 0.0;
             uint32_t succ0 = 0u;
-            for (int e0 = qb; e0 < qe; e0 += 32) {
-              uint32_t succ = 0u, open = 0u;  // on the level below, and of these not reached yet
-              const int e1 = min(qe, e0 + 32);
-              for (int e = e0; e < e1; e += 4) {
-                uint32_t u[4], f[4];  // past the row's end: the next row's, taken as on the level at hand
+            auto claim = [&](uint32_t u, uint32_t g, uint32_t field) {  // the first to set the bits has claimed the vertex
+              if ((atomicOr(code + u, cn << (2 * g)) & field) == 0u)
+                Q[atomicAdd(&s_tail, 1)] = (uint16_t)((u << gs) | g);
+            };
+            if (!(longs >> lane & 1u)) {
+              const double *const Sg = S + g;
+              for (int e0 = rb; e0 < re; e0 += 32) {
+                uint32_t succ = 0u, open = 0u;  // on the level below, and of these not reached yet
+                const int e1 = min(re, e0 + 32);
+                for (int e = e0; e < e1; e += 4) {
+                  uint32_t u[4], f[4];  // past the row's end: taken as on the level at hand
 #pragma unroll
-                for (int j = 0; j < 4; j++) u[j] = col[e + j];
+                  for (int j = 0; j < 4; j++) u[j] = col_at(GLOBAL ? min(e + j, e1 - 1) : e + j);
 #pragma unroll
-                for (int j = 0; j < 4; j++) f[j] = *(volatile uint32_t *)(code + u[j]) & field;
+                  for (int j = 0; j < 4; j++) f[j] = *(volatile uint32_t *)(code + u[j]) & field;
 #pragma unroll
-                for (int j = 1; j < 4; j++) f[j] = e + j < e1 ? f[j] : same;
-                uint32_t s4 = 0u, o4 = 0u;
+                  for (int j = 1; j < 4; j++) f[j] = e + j < e1 ? f[j] : same;
+                  uint32_t s4 = 0u, o4 = 0u;
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                  double y = 0.0;
-                  if (f[j] == above) y = Sg[u[j] * G];
-                  s4 |= (f[j] != same && f[j] != above) ? 1u << j : 0u;
-                  o4 |= f[j] == 0u ? 1u << j : 0u;
-                  if (MODE == 0) ai += __double_as_longlong(y);
-                  else if (MODE == 1) ad += f[j] == above ? i64_to_f64_pos(__double_as_longlong(y)) : 0.0;
-                  else ad += y;
+                  for (int j = 0; j < 4; j++) {
+                    double y = 0.0;
+                    if (f[j] == above) y = Sg[u[j] * G];
+                    s4 |= (f[j] != same && f[j] != above) ? 1u << j : 0u;
+                    o4 |= f[j] == 0u ? 1u << j : 0u;
+                    if (MODE == 0) ai += __double_as_longlong(y);
+                    else if (MODE == 1) ad += f[j] == above ? i64_to_f64_pos(__double_as_longlong(y)) : 0.0;
+                    else ad += y;
+                  }
+                  succ |= s4 << (e - e0);
+                  open |= o4 << (e - e0);
                 }
-                succ |= s4 << (e - e0);
-                open |= o4 << (e - e0);
+                for (uint32_t m = open; m; m &= m - 1u) claim(col_at(e0 + __ffs(m) - 1), g, field);
+                edges += __popc(succ);
+                if (e0 == rb) succ0 = succ;
               }
-              for (uint32_t m = open; m; m &= m - 1u) {  // the first to set the bits has claimed the vertex
-                const uint32_t u = col[e0 + __ffs(m) - 1];
-                if ((atomicOr(code + u, cn << sh) & field) == 0u) Q[atomicAdd(&s_tail, 1)] = (uint16_t)((u << gs) | g);
-              }
-              edges += __popc(succ);
-              if (e0 == qb) succ0 = succ;
             }
+            for (unsigned m = longs; COOP && m; m &= m - 1u) {  // long rows: the warp
+              const int l = __ffs(m) - 1;
+              const uint32_t gl = __shfl_sync(0xffffffffu, it, l) & gmask, fl = 3u << (2 * gl);
+              const int b = __shfl_sync(0xffffffffu, rb, l), e = __shfl_sync(0xffffffffu, re, l);
+              long long si = 0;
+              double sd = 0.0;
+              for (int k = b + lane; k < e; k += 32) {
+                const uint32_t u = col_at(k), f = *(volatile uint32_t *)(code + u) & fl;
+                if (f == cp << (2 * gl)) {
+                  const double y = S[u * G + gl];
+                  if (MODE == 0) si += __double_as_longlong(y);
+                  else if (MODE == 1) sd += i64_to_f64_pos(__double_as_longlong(y));
+                  else sd += y;
+                } else if (f != cc << (2 * gl)) {
+                  edges++;
+                  if (f == 0u) claim(u, gl, fl);
+                }
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) {
+                if (MODE == 0) si += __shfl_xor_sync(0xffffffffu, si, o);
+                else sd += __shfl_xor_sync(0xffffffffu, sd, o);
+              }
+              if (lane == l) {
+                ai = si;
+                ad = sd;
+              }
+            }
+            if (!valid) continue;
             succ_of[x] = succ0;
             if (L > 0) {
               const int id = IDENT ? ident[v] : 1;
@@ -284,32 +340,43 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
           }
           __syncthreads();
         }
-        for (int i = a + tid; i < b; i += SMALL_THREADS) {
-          const uint32_t it = Q[i], v = it >> gs, g = it & gmask, x = v * G + g;
-          const int eb = row[v];
-          uint32_t m = succ_of[x];
+        for (int i0 = a + tid0; i0 < b; i0 += NT) {
+          const int i = COOP ? i0 + lane : i0;
+          const bool valid = !COOP || i < b;
+          const uint32_t it = valid ? Q[i] : 0u, v = it >> gs, g = it & gmask, x = v * G + g;
+          const int rb = valid ? row_of(v) : 0;
+          uint32_t m = valid ? succ_of[x] : 0u;
+          int re = 0;
+          unsigned longs = 0u;
+          if (COOP) {
+            re = valid ? row_of(v + 1) : 0;
+            longs = __ballot_sync(0xffffffffu, re - rb > 32);
+            if (__popc(longs) > SMALL_LONGS) longs = 0u;
+          }
           const int id = IDENT ? ident[v] : 1;
           int ev = 0;
           float mv = 1.0f;
           double sv = 1.0;
           int idx = 0;  // the count, if it is an integer in the table of reciprocals
-          if (kind) {
-            long long s = Si[x];
-            if (IDENT && id != 1) s /= id;  // exact: the stored count is a multiple of ident
-            if (FP32) {
-              split_pow2_i64(s, ev, mv);
+          if (valid) {
+            if (kind) {
+              long long s = Si[x];
+              if (IDENT && id != 1) s /= id;  // exact: the stored count is a multiple of ident
+              if (FP32) {
+                split_pow2_i64(s, ev, mv);
+              } else {
+                idx = s < RECIP_TABLE ? (int)s : 0;
+                sv = i64_to_f64_pos(s);
+              }
             } else {
-              idx = s < RECIP_TABLE ? (int)s : 0;
-              sv = i64_to_f64_pos(s);
+              sv = IDENT && id != 1 ? S[x] / (double)id : S[x];
+              if (FP32) split_pow2(sv, ev, mv);
             }
-          } else {
-            sv = IDENT && id != 1 ? S[x] / (double)id : S[x];
-            if (FP32) split_pow2(sv, ev, mv);
+            if (FP32 && absolute) ev += s_exp[g];
           }
-          if (FP32 && absolute) ev += s_exp[g];
           double sum = 0.0;
           float sumf = 0.0f;
-          auto add = [&](double cw) {
+          auto add = [&](double cw, int ev) {
             if (!FP32) {
               sum += cw;
             } else {
@@ -317,17 +384,42 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
               if (d >= -126) sumf = fmaf(__int_as_float(__double2loint(cw)), __int_as_float((127 + d) << 23), sumf);
             }
           };
+          if (COOP && l < Lmax)
+            for (unsigned ml = longs; ml; ml &= ml - 1u) {  // long rows: the warp, by the codes
+              const int from = __ffs(ml) - 1;
+              const uint32_t gl = __shfl_sync(0xffffffffu, it, from) & gmask;
+              const int rl = __shfl_sync(0xffffffffu, rb, from), el = __shfl_sync(0xffffffffu, re, from);
+              const int evl = FP32 ? __shfl_sync(0xffffffffu, ev, from) : 0;
+              const double sum0 = sum;
+              const float sumf0 = sumf;
+              sum = 0.0;
+              sumf = 0.0f;
+              for (int e = rl + lane; e < el; e += 32) {
+                const uint32_t w = col_at(e);
+                if (((code[w] >> (2 * gl)) & 3u) == cn) add(S[w * G + gl], evl);
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) {
+                if (!FP32) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                else sumf += __shfl_xor_sync(0xffffffffu, sumf, o);
+              }
+              if (lane != from) {
+                sum = sum0;
+                sumf = sumf0;
+              }
+            }
+          if (!valid) continue;
           if (m) {  // the first one is taken as it is
             if (!FP32) {
-              sum = S[(uint32_t)col[eb + __ffs(m) - 1] * G + g];
+              sum = S[col_at(rb + __ffs(m) - 1) * G + g];
               m &= m - 1u;
             }
-            for (; m; m &= m - 1u) add(S[(uint32_t)col[eb + __ffs(m) - 1] * G + g]);
+            for (; m; m &= m - 1u) add(S[col_at(rb + __ffs(m) - 1) * G + g], ev);
           }
-          if (l < Lmax)
-            for (int e = eb + 32; e < row[v + 1]; e++) {  // entries past the 32nd: by their codes
-              const uint32_t w = col[e];
-              if (((code[w] >> (2 * g)) & 3u) == cn) add(S[w * G + g]);
+          if (l < Lmax && !(longs >> lane & 1u))
+            for (int e = rb + 32; e < (COOP ? re : row_of(v + 1)); e++) {  // entries past the 32nd: by their codes
+              const uint32_t w = col_at(e);
+              if (((code[w] >> (2 * g)) & 3u) == cn) add(S[w * G + g], ev);
             }
           double dv;
           if (!FP32) {
@@ -349,16 +441,16 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
         b = a;
         cc = cc == 1u ? 3u : cc - 1u;
       }
-      // the places' bc' terms, added up in order; every SMALL_FLUSH rounds, so
+      // the places' bc' terms, added up in order; every small_flush rounds, so
       // that no sum is a long chain of additions
-      if (first + (int)G < item.s_end && ++rounds % SMALL_FLUSH) continue;
-      for (int v = tid; v < n; v += SMALL_THREADS) {
+      if (first + (int)G < item.s_end && ++rounds % small_flush(GLOBAL)) continue;
+      for (int v = tid; v < n; v += NT) {
         double t = 0.0;
         for (uint32_t g = 0; g < G; g++) {
           t += acc[(uint32_t)v * G + g];
           acc[(uint32_t)v * G + g] = 0.0;
         }
-        if (t != 0.0) atomicAdd(bcp + c.vtx_off + v, t);
+        if (t != 0.0) atomicAdd(bcp_cta + c.vtx_off + v, t);
       }
     }
     __syncthreads();
@@ -374,22 +466,23 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bcreach_small(
 static std::mutex g_small_mu;
 static std::map<long long, int> g_small_occ;  // (variant, device, smem) -> CTAs per SM
 
-template <bool R, bool I, bool F>
+template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
 static int small_prepare(int device) {
   static std::mutex mu;
   static std::set<int> done;
   std::lock_guard<std::mutex> lk(mu);
   if (!done.count(device)) {
-    BCS_CUDA(cudaFuncSetAttribute(k_bcreach_small<R, I, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    BCS_CUDA(cudaFuncSetAttribute(k_bcreach_small<R, I, F, COOP, GLOBAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)SMALL_SMEM));
     done.insert(device);
   }
   return BCS_OK;
 }
 
-template <bool R, bool I, bool F>
-static int small_ctas_t(int device, size_t smem, int *out) {
-  const long long key = ((long long)(R * 4 + I * 2 + F) << 48) | ((long long)device << 32) | (long long)smem;
+template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
+static int small_ctas_c(int device, size_t smem, int *out) {
+  const long long key = ((long long)(R * 16 + I * 8 + F * 4 + COOP * 2 + GLOBAL) << 48) | ((long long)device << 32) |
+                        (long long)smem;
   {
     std::lock_guard<std::mutex> lk(g_small_mu);
     auto it = g_small_occ.find(key);
@@ -398,41 +491,173 @@ static int small_ctas_t(int device, size_t smem, int *out) {
       return BCS_OK;
     }
   }
-  BCS_TRY((small_prepare<R, I, F>(device)));
-  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bcreach_small<R, I, F>, SMALL_THREADS, smem));
+  BCS_TRY((small_prepare<R, I, F, COOP, GLOBAL>(device)));
+  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bcreach_small<R, I, F, COOP, GLOBAL>,
+                                                         GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, smem));
   if (*out < 1) *out = 1;
   std::lock_guard<std::mutex> lk(g_small_mu);
   g_small_occ[key] = *out;
   return BCS_OK;
 }
 
-int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, size_t smem, int *out) {
-  return BCS_DISPATCH3(small_ctas_t, R, I, F, ctx.device, smem, out);
+template <bool R, bool I, bool F>
+static int small_ctas_t(int device, bool coop, size_t smem, int *out) {
+  return coop ? small_ctas_c<R, I, F, true, false>(device, smem, out)
+              : small_ctas_c<R, I, F, false, false>(device, smem, out);
+}
+
+int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, bool coop, size_t smem, int *out) {
+  return BCS_DISPATCH3(small_ctas_t, R, I, F, ctx.device, coop, smem, out);
 }
 
 size_t small_scratch_words(int64_t ctas, int64_t nmax) { return (size_t)ctas * (SMALL_MAX_G + 1) * (nmax + 2); }
 
-template <bool R, bool I, bool F>
-static int small_launch_t(Ctx &ctx, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
-                          const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
-                          int *err, unsigned long long *dag) {
-  BCS_TRY((small_prepare<R, I, F>(ctx.device)));
+struct SmallLaunch {
+  const SmallItem *items;
+  int nitems;
+  int *counter;
+  const CompDesc *comps;
+  const int64_t *srcs;
+  size_t bcp_stride;
+  int32_t *lvl;
+  int lvl_stride, lvl_G;
+  unsigned char *state;
+  size_t state_stride;
+  int *err;
+  unsigned long long *dag;
+};
+
+template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
+static int small_launch_c(Ctx &ctx, int grid, size_t smem, const BcInput &in, const SmallLaunch &a) {
+  BCS_TRY((small_prepare<R, I, F, COOP, GLOBAL>(ctx.device)));
   const double *recip = nullptr;
   BCS_TRY(recip_table(ctx, &recip));
-  k_bcreach_small<R, I, F><<<grid, SMALL_THREADS, smem, ctx.stream>>>(items, nitems, counter, comps, in.row, in.col,
-                                                                     in.reach, in.ident, in.init, srcs, recip, in.bcp,
-                                                                     scratch, (int)nmax + 2, err, dag);
+  k_bcreach_small<R, I, F, COOP, GLOBAL><<<grid, GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, smem, ctx.stream>>>(
+      a.items, a.nitems, a.counter, a.comps, in.row, in.col, in.reach, in.ident, in.init, a.srcs, recip,
+      in.bcp, a.bcp_stride, a.lvl, a.lvl_stride, a.lvl_G, a.state, a.state_stride, a.err, a.dag);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
   return BCS_OK;
 }
 
-int launch_small(Ctx &ctx, bool fp32, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
+template <bool R, bool I, bool F>
+static int small_launch_t(Ctx &ctx, bool coop, int grid, size_t smem, const BcInput &in, const SmallLaunch &a) {
+  return coop ? small_launch_c<R, I, F, true, false>(ctx, grid, smem, in, a)
+              : small_launch_c<R, I, F, false, false>(ctx, grid, smem, in, a);
+}
+
+int launch_small(Ctx &ctx, bool fp32, bool coop, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
                  const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
                  int *err, unsigned long long *dag) {
   const bool R = in.reach != nullptr || in.init != nullptr, I = in.ident != nullptr;
-  return BCS_DISPATCH3(small_launch_t, R, I, fp32, ctx, grid, smem, items, nitems, counter, comps, in, srcs, scratch, nmax,
-                       err, dag);
+  const SmallLaunch a{items, nitems, counter, comps, srcs, 0, scratch, (int)nmax + 2, SMALL_MAX_G, nullptr, 0, err, dag};
+  return BCS_DISPATCH3(small_launch_t, R, I, fp32, ctx, coop, grid, smem, in, a);
+}
+
+// ------------------------------------- plain Brandes in a fixed scratch
+// The scratch: the descriptor, the item counter and the error word (256 bytes
+// each), the items, copies of bc', then per CTA the level offsets and exponents
+// and, for a piece above shared memory, its counts and sums.
+
+__global__ void k_fixed_setup(CompDesc *comp, CompDesc desc, int *counter, int *err, SmallItem *items, int nitems, int per,
+                              int G) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nitems) items[i] = SmallItem{0, i * per, min(desc.n, (i + 1) * per), G};
+  if (i == 0) {
+    *comp = desc;
+    *counter = 0;
+    *err = 0;
+  }
+}
+
+// One bc' of thousands of sources' terms would round as often: there are
+// FIXED_COPIES, and adding those up keeps what the additions round off (2,600
+// vertices: error 5.9e-16 in one, 1.2e-16 so).
+__global__ void k_fixed_add(int n, const double *__restrict__ part, double *bc) {
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    double t = 0.0, lost = 0.0;
+    for (int c = 0; c < FIXED_COPIES; c++) {
+      const double a = part[(size_t)c * n + v], sum = t + a, of_a = sum - t;
+      lost += (t - (sum - of_a)) + (a - of_a);
+      t = sum;
+    }
+    bc[v] = t + lost;
+  }
+}
+
+template <bool F, bool GLOBAL>
+static int fixed_launch(Ctx &ctx, const CompDesc &desc, size_t smem, int G, size_t lvl_bytes, size_t state_bytes,
+                        BcInput in, unsigned char *scratch, size_t bytes) {
+  const int64_t n = desc.n;
+  const size_t head = FIXED_HEAD + fixed_up256((size_t)n * sizeof(SmallItem));
+  int per_sm = 1;
+  BCS_TRY((small_ctas_c<false, false, F, true, GLOBAL>(ctx.device, smem, &per_sm)));
+  const size_t part_bytes = fixed_up256((size_t)FIXED_COPIES * n * 8);
+  const int64_t fit = (int64_t)((bytes - head - part_bytes) / (lvl_bytes + state_bytes));
+  const int64_t ctas = std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx.num_sms * per_sm, fit));
+  // two items per CTA, or more of as many rounds as are added up at once
+  const int per = G * (int)std::max<int64_t>(1, std::min<int64_t>(n / (ctas * 2 * G), small_flush(GLOBAL)));
+  SmallLaunch a{};
+  a.nitems = (int)((n + per - 1) / per);
+  const int grid = (int)std::min<int64_t>(ctas, a.nitems);
+  double *const part = (double *)(scratch + head), *const bc = in.bcp;
+  a.comps = (const CompDesc *)scratch;
+  a.counter = (int *)(scratch + 256);
+  a.err = (int *)(scratch + FIXED_ERR);
+  a.items = (const SmallItem *)(scratch + FIXED_HEAD);
+  a.lvl = (int32_t *)(scratch + head + part_bytes);
+  a.lvl_stride = (int)n + 2;
+  a.lvl_G = G;
+  a.bcp_stride = (size_t)n;
+  a.state = scratch + head + part_bytes + (size_t)grid * lvl_bytes;
+  a.state_stride = state_bytes;
+  in.bcp = part;
+  BCS_CUDA(cudaMemsetAsync(part, 0, part_bytes, ctx.stream));
+  k_fixed_setup<<<(a.nitems + 255) / 256, 256, 0, ctx.stream>>>((CompDesc *)scratch, desc, a.counter, a.err,
+                                                                (SmallItem *)(scratch + FIXED_HEAD), a.nitems, per, G);
+  ctx.launches++;
+  BCS_CUDA(cudaGetLastError());
+  BCS_TRY((small_launch_c<false, false, F, true, GLOBAL>(ctx, grid, smem, in, a)));
+  k_fixed_add<<<(int)((n + 63) / 64), 64, 0, ctx.stream>>>((int)n, part, bc);
+  ctx.launches++;
+  BCS_CUDA(cudaGetLastError());
+  return BCS_OK;
+}
+
+int launch_plain_fixed_scratch(Ctx &ctx, const int64_t *row, const int32_t *col, int32_t n, int64_t nnz, double *bc,
+                               unsigned char *scratch, size_t bytes, bool fp32) {
+  int *const err = (int *)(scratch + FIXED_ERR);
+  // n bounds the degree, hence the growth of path counts per level
+  CompDesc desc{};
+  desc.n = n;
+  desc.nnz = nnz;
+  desc.src_off = -1;
+  desc.fan = (double)std::max(n, 1);
+  BcInput in;
+  in.row = row;
+  in.col = col;
+  in.bcp = bc;
+  if (small_takes(n, nnz, 1) && small_smem_bytes(n, nnz, 1, false, false) <= SMALL_SMEM) {
+    // no more sources at once than leave every SM two items
+    int G = (int)std::max<int64_t>(1, std::min<int64_t>(SMALL_MAX_G, n / (2 * (int64_t)ctx.num_sms)));
+    while (G > 1 && small_smem_bytes(n, nnz, G, false, false) > SMALL_BUDGET) G--;
+    const size_t smem = small_smem_bytes(n, nnz, G, false, false), lvl = fixed_up256((size_t)(G + 1) * (n + 2) * 4);
+    if (fp32) BCS_TRY((fixed_launch<true, false>(ctx, desc, smem, G, lvl, 0, in, scratch, bytes)));
+    else BCS_TRY((fixed_launch<false, false>(ctx, desc, smem, G, lvl, 0, in, scratch, bytes)));
+  } else {
+    const size_t smem = align16((size_t)n * 4) + align16((size_t)n * 2), lvl = fixed_up256((size_t)2 * (n + 2) * 4);
+    const size_t state = fixed_up256(align16((size_t)n * 8) * 2 + align16((size_t)n * 4));
+    if (fp32) BCS_TRY((fixed_launch<true, true>(ctx, desc, smem, 1, lvl, state, in, scratch, bytes)));
+    else BCS_TRY((fixed_launch<false, true>(ctx, desc, smem, 1, lvl, state, in, scratch, bytes)));
+  }
+  int h_err = 0;
+  BCS_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
+  BCS_CUDA(cudaStreamSynchronize(ctx.stream));
+  if (h_err & ERR_OVERFLOW) {
+    set_error("shortest-path counts overflowed the FP64 range within one BFS level");
+    return BCS_EOVERFLOW;
+  }
+  return BCS_OK;
 }
 
 }  // namespace bcs

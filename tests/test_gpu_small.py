@@ -88,3 +88,20 @@ def test_shallow_pieces_of_many_vertices_go_to_the_pull_kernel(gpu, graphs, pull
     assert (st["n_wide_batches"] > 0) == pull
     if not pull:
         assert st["n_large_sources"] == 0
+
+
+@pytest.mark.parametrize("g", [gg.path(1), gg.path(2), gg.star(40), gg.chung_lu(300, 2.3, 8.0, 2), gg.chung_lu(1300, 2.3, 20.0, 2),
+                               gg.star(2300), gg.star(4500), gg.chung_lu(4001, 2.3, 8.0, 2), gg.complete(300), gg.cycle(3001),
+                               gg.disjoint_union(gg.grid(60, 50), gg.path(9), gg.gnp(3, 0.0, 0), gg.star(900)),
+                               ladder(1100, 2, False), ladder(1900, 2, True)], ids=lambda g: g.name)
+def test_without_allocations(gpu, g):
+    """The allocation-free call on both sides of the shared memory, hubs taken
+    by whole warps (up to eight of a warp's rows, and more), several
+    components, path counts past the double range."""
+    import torch
+    ref = oracle.bc(g)
+    scale = max(1.0, float(np.abs(ref).max()))
+    rp, col = torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col).cuda()
+    for fp32, tol in ((False, 1e-12), (True, 1e-5), (False, 1e-12)):
+        got = gpu.bc_plain_noalloc(rp, col, delta_fp32=fp32).cpu().numpy()
+        assert float(np.abs(got - ref).max()) <= tol * scale
