@@ -17,6 +17,7 @@ namespace bcs {
 
 constexpr int ORDER_THREADS = 1024;
 constexpr int ORDER_SUB = 8;  // lanes per frontier row
+constexpr int ORDER_LONG = 256;
 
 __device__ __forceinline__ void push_one(int32_t *queue, unsigned long long *count, int64_t base_off, int32_t v) {
   const unsigned mask = __activemask();
@@ -38,31 +39,58 @@ __global__ void k_order_roots(int64_t n, const int32_t *__restrict__ label, int3
   }
 }
 
-// The level-synchronous search; lcount[l] counts level l (one counter per
-// level, so one grid-wide wait per level suffices).  out[0] = vertices queued.
+// The level-synchronous search; the low half of lcount[l] counts level l (one
+// counter per level, so one grid-wide wait per level suffices), the high half
+// its vertices with rows of more than ORDER_LONG entries, which are listed in
+// longs and walked by a whole CTA each: eight lanes on a hub's row hold up the
+// level.  out[0] = vertices queued.
 __global__ void k_order_bfs(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int32_t *level,
-                            int32_t *queue, int32_t *parent, unsigned long long *lcount, int64_t *out,
+                            int32_t *queue, int32_t *longs, int32_t *parent, unsigned long long *lcount, int64_t *out,
                             GridBarrier bar) {
   const int sl = (int)(threadIdx.x % ORDER_SUB);
   const int64_t sub0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / ORDER_SUB;
   const int64_t nsub = (int64_t)gridDim.x * blockDim.x / ORDER_SUB;
-  int64_t lo = 0, hi = (int64_t)*(volatile unsigned long long *)lcount;
+  int64_t lo = 0, hi = (int64_t)*(volatile unsigned long long *)lcount, long_lo = 0, long_hi = 0;
+  const bool roots_by_cta = hi <= 4 * (int64_t)gridDim.x;
   for (int L = 0;; L++) {
-    for (int64_t i = lo + sub0; i < hi; i += nsub) {
-      const int32_t v = queue[i];
-      for (int64_t k = rp[v] + sl; k < rp[v + 1]; k += ORDER_SUB) {
-        const int32_t w = col[k];
-        if (uf_vload(level + w) < 0 && atomicCAS(level + w, -1, L + 1) < 0) {
-          if (parent) parent[w] = v;
-          push_one(queue, lcount + L + 1, hi, w);
-        }
+    auto visit = [&](int32_t v, int64_t k) {
+      const int32_t w = col[k];
+      if (uf_vload(level + w) < 0 && atomicCAS(level + w, -1, L + 1) < 0) {
+        if (parent) parent[w] = v;
+        const bool is_long = rp[w + 1] - rp[w] > ORDER_LONG;
+        const unsigned mask = __activemask();
+        const int lane = (int)(threadIdx.x & 31), leader = __ffs(mask) - 1;
+        const unsigned ml = __ballot_sync(mask, is_long);
+        unsigned long long base = 0;
+        if (lane == leader)
+          base = atomicAdd(lcount + L + 1, (unsigned long long)__popc(mask) | (unsigned long long)__popc(ml) << 32);
+        base = __shfl_sync(mask, base, leader);
+        const unsigned below = (1u << lane) - 1u;
+        queue[hi + (int64_t)(base & 0xffffffffu) + __popc(mask & below)] = w;
+        if (is_long) longs[long_hi + (int64_t)(base >> 32) + __popc(ml & below)] = w;
       }
+    };
+    if (L > 0 || !roots_by_cta)
+      for (int64_t i = lo + sub0; i < hi; i += nsub) {
+        const int32_t v = queue[i];
+        const int64_t b = rp[v], e = rp[v + 1];
+        if (L > 0 && e - b > ORDER_LONG) continue;
+        for (int64_t k = b + sl; k < e; k += ORDER_SUB) visit(v, k);
+      }
+    const int32_t *const by_cta = L > 0 ? longs : queue;
+    const int64_t c0 = L > 0 ? long_lo : lo, c1 = L > 0 ? long_hi : (roots_by_cta ? hi : lo);
+    for (int64_t i = c0 + blockIdx.x; i < c1; i += gridDim.x) {
+      const int32_t v = by_cta[i];
+      const int64_t e = rp[v + 1];
+      for (int64_t k = rp[v] + threadIdx.x; k < e; k += blockDim.x) visit(v, k);
     }
     if (!grid_wait(bar)) return;
-    const int64_t nhi = hi + (int64_t)*(volatile unsigned long long *)(lcount + L + 1);
-    if (nhi == hi) break;
+    const unsigned long long found = *(volatile unsigned long long *)(lcount + L + 1);
+    if ((found & 0xffffffffu) == 0) break;
     lo = hi;
-    hi = nhi;
+    hi += (int64_t)(found & 0xffffffffu);
+    long_lo = long_hi;
+    long_hi += (int64_t)(found >> 32);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = hi;
 }
@@ -158,6 +186,8 @@ int bfs_order_graph(Ctx &ctx, const DevGraph &g, DBuf<int64_t> *rp2, DBuf<int32_
     DBuf<int> err;
     DBuf<unsigned int> barw;
     DBuf<int64_t> out;
+    DBuf<int32_t> longs;
+    BCS_TRY(longs.alloc(n, ctx.stream));
     BCS_TRY(err.alloc(1, ctx.stream));
     BCS_TRY(barw.alloc(2, ctx.stream));
     BCS_TRY(out.alloc(1, ctx.stream));
@@ -170,8 +200,8 @@ int bfs_order_graph(Ctx &ctx, const DevGraph &g, DBuf<int64_t> *rp2, DBuf<int32_
     int32_t *levelp = level.p, *queuep = queue.p;
     unsigned long long *lcp = lcount.p;
     int64_t *outp = out.p;
-    int32_t *parentp = nullptr;
-    void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
+    int32_t *parentp = nullptr, *longsp = longs.p;
+    void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&longsp, (void *)&parentp, (void *)&lcp, (void *)&outp,
                     (void *)&gb};
     BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                          ctx.stream));
@@ -279,6 +309,8 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
   DBuf<int> err;
   DBuf<unsigned int> barw;
   DBuf<int64_t> out;
+  DBuf<int32_t> longs;
+  BCS_TRY(longs.alloc(n, ctx.stream));
   BCS_TRY(err.alloc(1, ctx.stream));
   BCS_TRY(barw.alloc(2, ctx.stream));
   BCS_TRY(out.alloc(1, ctx.stream));
@@ -288,8 +320,8 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
   int32_t *levelp = level.p, *queuep = queue_out;
   unsigned long long *lcp = lcount.p;
   int64_t *outp = out.p;
-  int32_t *parentp = parent;
-  void *args[] = {(void *)&rp, (void *)&col, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
+  int32_t *parentp = parent, *longsp = longs.p;
+  void *args[] = {(void *)&rp, (void *)&col, (void *)&levelp, (void *)&queuep, (void *)&longsp, (void *)&parentp, (void *)&lcp, (void *)&outp,
                   (void *)&gb};
   BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                        ctx.stream));
@@ -339,6 +371,8 @@ int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_
   DBuf<int> err;
   DBuf<unsigned int> barw;
   DBuf<int64_t> out;
+  DBuf<int32_t> longs;
+  BCS_TRY(longs.alloc(n, ctx.stream));
   BCS_TRY(err.alloc(1, ctx.stream));
   BCS_TRY(barw.alloc(2, ctx.stream));
   BCS_TRY(out.alloc(1, ctx.stream));
@@ -350,8 +384,8 @@ int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_
   int32_t *levelp = level.p, *queuep = queue_out;
   unsigned long long *lcp = lcount.p;
   int64_t *outp = out.p;
-  int32_t *parentp = parent;
-  void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&parentp, (void *)&lcp, (void *)&outp,
+  int32_t *parentp = parent, *longsp = longs.p;
+  void *args[] = {(void *)&rpp, (void *)&colp, (void *)&levelp, (void *)&queuep, (void *)&longsp, (void *)&parentp, (void *)&lcp, (void *)&outp,
                   (void *)&gb};
   BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_order_bfs, dim3(ctx.num_sms), dim3(ORDER_THREADS), args, 0,
                                        ctx.stream));

@@ -962,6 +962,14 @@ __global__ void k_pull_idmax(int64_t n, const int32_t *__restrict__ ident, int32
 // vertices are kept in shared memory.
 constexpr int PIECE_BFS_THREADS = 1024;
 constexpr int PIECE_BFS_RING = 2048;
+// Rows of more than PIECE_BFS_LONG entries wait for the end of their level and
+// are taken by a warp each, those of more than PIECE_BFS_HUGE by the whole CTA:
+// one thread on a hub's row holds up everybody (a power-law piece of 13,700
+// vertices: 0.72 to 0.29 ms).
+constexpr int PIECE_BFS_LONG = 64;
+constexpr int PIECE_BFS_HUGE = 2048;
+constexpr int PIECE_BFS_LONGS = 1024;  // kept of a level; more are walked by their thread
+constexpr int PIECE_BFS_HUGES = 64;
 constexpr int PIECE_BFS_WIDE = 8192;
 __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc *__restrict__ comps,
                                                                  const int32_t *__restrict__ list, int nlist,
@@ -970,8 +978,11 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
                                                                  const int64_t *__restrict__ ord_off, int32_t *order,
                                                                  int32_t *parent, int32_t *level, int32_t *depth,
                                                                  int32_t *reached) {
-  __shared__ int s_i, s_tail;
+  __shared__ int s_i, s_tail, s_nlong, s_nhuge;
   __shared__ int32_t s_ring[2][PIECE_BFS_RING];
+  __shared__ int32_t s_long[PIECE_BFS_LONGS], s_huge[PIECE_BFS_HUGES];
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  constexpr int WARPS = PIECE_BFS_THREADS / 32;
   for (;;) {
     if (threadIdx.x == 0) s_i = atomicAdd(next, 1);
     __syncthreads();
@@ -985,37 +996,65 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
       q[0] = s_ring[0][0] = 0;
       par[0] = -1;
       s_tail = 1;
+      s_nlong = s_nhuge = 0;
     }
     __syncthreads();
+    // v's entries e, e + step, ... below e1
+    auto walk = [&](int32_t v, int64_t e, int64_t e1, int step, int32_t *ring_next, int hi, int L) {
+      for (; e < e1; e += 4 * step) {
+        int32_t u[4], l[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) u[j] = e + j * step < e1 ? g_col[e + j * step] : -1;
+#pragma unroll
+        for (int j = 0; j < 4; j++) l[j] = u[j] >= 0 ? *(volatile int32_t *)(lv + u[j]) : 0;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (l[j] < 0) l[j] = atomicCAS(lv + u[j], -1, L + 1);
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (l[j] < 0) {
+            const int t = atomicAdd(&s_tail, 1);
+            q[t] = u[j];
+            par[u[j]] = v;
+            if (t - hi < PIECE_BFS_RING) ring_next[t - hi] = u[j];
+          }
+      }
+    };
     int lo = 0, hi = 1, L = 0;
     while (lo < hi) {
       const int32_t *const ring = s_ring[L & 1];
       int32_t *const ring_next = s_ring[(L + 1) & 1];
-      for (int k = lo + (int)threadIdx.x; k < hi; k += PIECE_BFS_THREADS) {
+      // a next level found too wide ends the search at once
+      auto too_wide = [&]() { return c.n > PIECE_BFS_MAX_N && *(volatile int *)&s_tail - hi > PIECE_BFS_WIDE; };
+      for (int k = lo + (int)threadIdx.x; k < hi && !too_wide(); k += PIECE_BFS_THREADS) {
         const int32_t v = k - lo < PIECE_BFS_RING ? ring[k - lo] : q[k];
-        const int64_t e1 = row[v + 1];
-        for (int64_t e = row[v]; e < e1; e += 4) {
-          int32_t u[4], l[4];
-#pragma unroll
-          for (int j = 0; j < 4; j++) u[j] = e + j < e1 ? g_col[e + j] : -1;
-#pragma unroll
-          for (int j = 0; j < 4; j++) l[j] = u[j] >= 0 ? *(volatile int32_t *)(lv + u[j]) : 0;
-#pragma unroll
-          for (int j = 0; j < 4; j++)
-            if (l[j] < 0) l[j] = atomicCAS(lv + u[j], -1, L + 1);
-#pragma unroll
-          for (int j = 0; j < 4; j++)
-            if (l[j] < 0) {
-              const int t = atomicAdd(&s_tail, 1);
-              q[t] = u[j];
-              par[u[j]] = v;
-              if (t - hi < PIECE_BFS_RING) ring_next[t - hi] = u[j];
-            }
+        const int64_t e0 = row[v], e1 = row[v + 1];
+        if (e1 - e0 > PIECE_BFS_HUGE) {
+          const int t = atomicAdd(&s_nhuge, 1);
+          if (t < PIECE_BFS_HUGES) {
+            s_huge[t] = v;
+            continue;
+          }
         }
+        if (e1 - e0 > PIECE_BFS_LONG) {
+          const int t = atomicAdd(&s_nlong, 1);
+          if (t < PIECE_BFS_LONGS) {
+            s_long[t] = v;
+            continue;
+          }
+        }
+        walk(v, e0, e1, 1, ring_next, hi, L);
       }
+      __syncthreads();
+      const int nlong = min(s_nlong, PIECE_BFS_LONGS), nhuge = min(s_nhuge, PIECE_BFS_HUGES);
+      for (int j = 0; j < nhuge && !too_wide(); j++)
+        walk(s_huge[j], row[s_huge[j]] + threadIdx.x, row[s_huge[j] + 1], PIECE_BFS_THREADS, ring_next, hi, L);
+      for (int j = warp; j < nlong && !too_wide(); j += WARPS)
+        walk(s_long[j], row[s_long[j]] + lane, row[s_long[j] + 1], 32, ring_next, hi, L);
       __syncthreads();
       lo = hi;
       hi = *(volatile int *)&s_tail;
+      if (threadIdx.x == 0) s_nlong = s_nhuge = 0;
       __syncthreads();
       L++;
       if (c.n > PIECE_BFS_MAX_N && hi - lo > PIECE_BFS_WIDE) break;
