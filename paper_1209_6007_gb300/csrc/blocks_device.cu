@@ -121,6 +121,27 @@ __global__ void k_bfs_init(int64_t n, const uint8_t *__restrict__ alive, const i
   }
 }
 
+// Rows of more than LONG_ROW entries are walked by the whole warp: one thread
+// on a hub's row holds up the launch (a power-law graph of 194,000 vertices: low
+// and high, unions and rows 6.0 ms with a thread each, 2.6 so).  WARP_STRIDE: a grid-stride loop that whole
+// warps run through together (i may be past n).
+constexpr int LONG_ROW = 32;
+#define WARP_STRIDE(i, n)                                                                              \
+  for (int64_t i##0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll, i = i##0 + (threadIdx.x & 31); \
+       i##0 < (n); i##0 += (int64_t)gridDim.x * blockDim.x, i += (int64_t)gridDim.x * blockDim.x)
+
+// f(v, entry, 32-entry step's end) for the entries [b, e) of each lane in `longs`, in order
+template <typename F>
+__device__ __forceinline__ void for_long_rows(unsigned longs, int32_t v, int64_t b, int64_t e, F f) {
+  for (unsigned m = longs; m; m &= m - 1u) {
+    const int l = __ffs(m) - 1;
+    const int32_t vl = __shfl_sync(0xffffffffu, v, l);
+    const int64_t bl = __shfl_sync(0xffffffffu, b, l), el = __shfl_sync(0xffffffffu, e, l);
+    for (int64_t k = bl + (threadIdx.x & 31); k < el; k += 32) f(vl, k, el);
+    __syncwarp();
+  }
+}
+
 __device__ __forceinline__ bool is_tree_edge(const int32_t *parent, int32_t u, int32_t w) {
   return parent[w] == u || parent[u] == w;
 }
@@ -253,15 +274,35 @@ __global__ void k_forest_coop(const int64_t *__restrict__ rp, const int32_t *__r
   }
   if (!grid_wait(bar)) return;
   stamp(stamps, 3);
-  COOP_STRIDE(i, 0, cnt) {  // own pre and the far ends of non-tree edges
-    const int32_t u = order[i];
-    int32_t a = pre[u], b = pre[u];
-    for (int64_t k = rp[u]; k < rp[u + 1]; k++) {
+  WARP_STRIDE(i, cnt) {  // own pre and the far ends of non-tree edges
+    const bool valid = i < cnt;
+    const int32_t u = valid ? order[i] : 0;
+    int32_t a = valid ? pre[u] : 0, b = a;
+    const int64_t k0 = valid ? rp[u] : 0, k1 = valid ? rp[u + 1] : 0;
+    auto far_end = [&](int32_t u, int64_t k, int32_t &a, int32_t &b) {
       const int32_t w = col[k];
-      if (!alive[w] || parent[w] == u || parent[u] == w) continue;
-      a = min(a, pre[w]);
-      b = max(b, pre[w]);
+      if (!alive[w] || parent[w] == u || parent[u] == w) return;
+      const int32_t pw = pre[w];
+      a = min(a, pw);
+      b = max(b, pw);
+    };
+    const unsigned longs = __ballot_sync(0xffffffffu, k1 - k0 > LONG_ROW);
+    if (k1 - k0 <= LONG_ROW)
+      for (int64_t k = k0; k < k1; k++) far_end(u, k, a, b);
+    for (unsigned m = longs; m; m &= m - 1u) {
+      const int l = __ffs(m) - 1;
+      const int32_t ul = __shfl_sync(0xffffffffu, u, l);
+      const int64_t l0 = __shfl_sync(0xffffffffu, k0, l), l1 = __shfl_sync(0xffffffffu, k1, l);
+      int32_t al = pre[ul], bl = al;
+      for (int64_t k = l0 + (threadIdx.x & 31); k < l1; k += 32) far_end(ul, k, al, bl);
+      al = __reduce_min_sync(0xffffffffu, al);
+      bl = __reduce_max_sync(0xffffffffu, bl);
+      if ((int)(threadIdx.x & 31) == l) {
+        a = al;
+        b = bl;
+      }
     }
+    if (!valid) continue;
     low[u] = a;
     high[u] = b;
     done[u] = 0;
@@ -293,13 +334,20 @@ __global__ void k_tv_unite(int64_t cnt, const int32_t *__restrict__ order, const
                            const int32_t *__restrict__ parent, const int32_t *__restrict__ level,
                            const int32_t *__restrict__ pre, const int32_t *__restrict__ nd,
                            const int32_t *__restrict__ low, const int32_t *__restrict__ high, int32_t *uf) {
-  GRID_STRIDE(i, cnt) {
-    const int32_t u = order[i];
-    if (level[u] == 0) continue;  // roots carry no tree edge
-    for (int64_t k = rp[u]; k < rp[u + 1]; k++) {
+  WARP_STRIDE(i, cnt) {
+    const bool valid = i < cnt;
+    const int32_t u = valid ? order[i] : 0;
+    const bool edge = valid && level[u] > 0;  // roots carry no tree edge
+    const int64_t b = edge ? rp[u] : 0, e = edge ? rp[u + 1] : 0;
+    auto unite = [&](int32_t u, int64_t k) {
       const int32_t w = col[k];
       if (w > u && alive[w] && !is_tree_edge(parent, u, w)) uf_unite(uf, u, w);  // rule (1)
-    }
+    };
+    const unsigned longs = __ballot_sync(0xffffffffu, e - b > LONG_ROW);
+    if (e - b <= LONG_ROW)
+      for (int64_t k = b; k < e; k++) unite(u, k);
+    for_long_rows(longs, u, b, e, [&](int32_t u, int64_t k, int64_t) { unite(u, k); });
+    if (!edge) continue;
     const int32_t v = parent[u];
     if (level[v] > 0 && (low[u] < pre[v] || high[u] >= pre[v] + nd[v])) uf_unite(uf, u, v);  // rule (2)
   }
@@ -425,19 +473,31 @@ __global__ void k_slot_degrees(int64_t cnt, const int32_t *__restrict__ verts, b
                                const int32_t *__restrict__ parent, const int32_t *__restrict__ level,
                                const int32_t *__restrict__ bid, const int32_t *__restrict__ home_slot,
                                const int32_t *__restrict__ top_slot, int64_t *sdeg) {
-  GRID_STRIDE(i, cnt) {
-    const int32_t v = verts[i];
-    const int32_t hs = home_slot[v];  // most of v's entries go to its home slot: counted in a register
+  WARP_STRIDE(i, cnt) {
+    const bool valid = i < cnt;
+    const int32_t v = valid ? verts[i] : 0;
+    const int32_t hs = valid ? home_slot[v] : -1;  // most of v's entries go to its home slot: counted in a register
     int64_t nh = 0;
-    for (int64_t k = rp[v]; k < rp[v + 1]; k++) {
+    const int64_t b = valid ? rp[v] : 0, e = valid ? rp[v + 1] : 0;
+    const unsigned longs = __ballot_sync(0xffffffffu, e - b > LONG_ROW);
+    if (e - b <= LONG_ROW)
+      for (int64_t k = b; k < e; k++) {
+        const int32_t w = col[k];
+        if (!alive[w]) continue;
+        int32_t sv, sw;
+        edge_slots(art, v, w, parent, level, bid, home_slot, top_slot, sv, sw);
+        if (sv == hs) nh++;
+        else sdeg[sv]++;  // every slot of v is written only by v's thread (or its warp, below)
+      }
+    if (nh > 0) sdeg[hs] += nh;  // nh > 0 implies a home slot
+    for_long_rows(longs, v, b, e, [&](int32_t v, int64_t k, int64_t) {
       const int32_t w = col[k];
-      if (!alive[w]) continue;
+      if (!alive[w]) return;
       int32_t sv, sw;
       edge_slots(art, v, w, parent, level, bid, home_slot, top_slot, sv, sw);
-      if (sv == hs) nh++;
-      else sdeg[sv]++;  // every slot of v is written only by v's thread
-    }
-    if (nh > 0) sdeg[hs] += nh;  // nh > 0 implies a home slot
+      const unsigned act = __activemask(), same = __match_any_sync(act, sv);
+      if (__ffs(same) - 1 == (int)(threadIdx.x & 31)) atomicAdd((unsigned long long *)(sdeg + sv), (unsigned long long)__popc(same));
+    });
   }
 }
 
@@ -446,17 +506,45 @@ __global__ void k_slot_fill(int64_t cnt, const int32_t *__restrict__ verts, bool
                             const int32_t *__restrict__ parent, const int32_t *__restrict__ level,
                             const int32_t *__restrict__ bid, const int32_t *__restrict__ home_slot,
                             const int32_t *__restrict__ top_slot, int64_t *cursor, int32_t *scol) {
-  GRID_STRIDE(i, cnt) {
-    const int32_t v = verts[i];
-    const int32_t hs = home_slot[v];
-    int64_t hpos = hs >= 0 ? cursor[hs] : 0;  // the home slot's cursor stays in a register
-    for (int64_t k = rp[v]; k < rp[v + 1]; k++) {
-      const int32_t w = col[k];
-      if (!alive[w]) continue;
-      int32_t sv, sw;
-      edge_slots(art, v, w, parent, level, bid, home_slot, top_slot, sv, sw);
-      if (sv == hs) scol[hpos++] = sw;
-      else scol[cursor[sv]++] = sw;
+  const int lane = threadIdx.x & 31;
+  WARP_STRIDE(i, cnt) {
+    const bool valid = i < cnt;
+    const int32_t v = valid ? verts[i] : 0;
+    const int64_t b = valid ? rp[v] : 0, e = valid ? rp[v + 1] : 0;
+    const unsigned longs = __ballot_sync(0xffffffffu, e - b > LONG_ROW);
+    if (e - b <= LONG_ROW) {
+      const int32_t hs = home_slot[v];
+      int64_t hpos = valid && hs >= 0 ? cursor[hs] : 0;  // the home slot's cursor stays in a register
+      for (int64_t k = b; k < e; k++) {
+        const int32_t w = col[k];
+        if (!alive[w]) continue;
+        int32_t sv, sw;
+        edge_slots(art, v, w, parent, level, bid, home_slot, top_slot, sv, sw);
+        if (sv == hs) scol[hpos++] = sw;
+        else scol[cursor[sv]++] = sw;
+      }
+    }
+    for (unsigned m = longs; m; m &= m - 1u) {  // the warp; entries of a slot keep their order
+      const int l = __ffs(m) - 1;
+      const int32_t vl = __shfl_sync(0xffffffffu, v, l);
+      const int64_t bl = __shfl_sync(0xffffffffu, b, l), el = __shfl_sync(0xffffffffu, e, l);
+      for (int64_t k0 = bl; k0 < el; k0 += 32) {
+        const int64_t k = k0 + lane;
+        const int32_t w = k < el ? col[k] : -1;
+        int32_t sv = -1, sw = -1;
+        if (w >= 0 && alive[w]) edge_slots(art, vl, w, parent, level, bid, home_slot, top_slot, sv, sw);
+        const unsigned same = __match_any_sync(0xffffffffu, sv);
+        const int first = __ffs(same) - 1;
+        int64_t at = 0;
+        if (sv >= 0 && lane == first) {
+          volatile int64_t *const cur = (volatile int64_t *)(cursor + sv);
+          at = *cur;
+          *cur = at + __popc(same);
+        }
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (sv >= 0) scol[at + __popc(same & ((1u << lane) - 1u))] = sw;
+        __syncwarp();
+      }
     }
   }
 }
