@@ -71,7 +71,7 @@ def parse():
                          "side: the articulation workload with added side vertices, shattered with and without "
                          "the side-vertex step; unequal: a twin-heavy graph whose twins carry pendants, with and "
                          "without merging twins of unequal reach; twins-batch: one 64-source batch of the "
-                         "twin workload's largest piece through the whole-GPU kernel, run twice (for profilers)")
+                         "twin workload's largest piece through the pull kernel, run twice (for profilers)")
     ap.add_argument("--batch-count", type=int, default=20000)
     ap.add_argument("--batch-nmax", type=int, default=4096)
     return ap.parse_args()
@@ -158,7 +158,7 @@ def workload(name: str, scale: int):
 # sources the kernel compiles from; a figure is used only while they match
 PROFILES = {
     "small": ("bcreach_small_articulation.json", ("small.cu", "bc_math.cuh")),
-    "wide": ("bcreach_wide_twins.json", ("pull.cu", "bc_math.cuh", "coop.cuh")),
+    "wide": ("bcreach_pull_twins.json", ("pull.cu", "bc_math.cuh", "coop.cuh")),
 }
 
 
@@ -240,7 +240,7 @@ def run_reference(args):
 def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
     """Roofline of the call's dominant Bc-Reach kernel.
 
-    Large pieces (the whole-GPU kernel): HBM.  Algorithmic bytes per
+    Large pieces (the pull kernel): HBM.  Algorithmic bytes per
     (source, CSR entry) of a piece, with S sources sharing one adjacency
     read: 8/S (the row) + 2/8 (level bits) + f_DAG * 28 (path count written
     and read, coefficient, weights, per shortest-path DAG edge) + (n / 2m) *
@@ -258,7 +258,7 @@ def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
     wse, wsv = float(st["work_sources_entries"]), float(st["work_sources_vertices"])
     sm_mhz = clk.get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))
     if st["ms_bcreach_large"] > st["ms_bcreach_small"]:
-        # sources sharing one batch of the whole-GPU kernel (32 or 64)
+        # sources sharing one batch of the pull kernel (32 or 64)
         S = 64 if st["n_wide_batches"] and st["n_large_sources"] > 32 * st["n_wide_batches"] else 32
         f_dag = dag / wse if wse else 0.0
         by = wse * (8.0 / S + 2.0 / 8.0 + f_dag * 28.0) + wsv * 32.0
@@ -272,7 +272,7 @@ def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
                 "work": {"bytes": by, "f_dag": f_dag, "sources_x_entries": wse, "sources_x_vertices": wsv,
                          "batches": int(st["n_wide_batches"]), "ms": ms,
-                         "traffic_scaled_from": "ncu DRAM bytes of a full launch per batch (profiles/bcreach_wide_twins.json) "
+                         "traffic_scaled_from": "ncu DRAM bytes of a full launch per batch (profiles/bcreach_pull_twins.json) "
                                                 "x this call's batches" if traffic else None}}
     flop = 2.0 * dag + 9.0 * wsv
     ms = st["ms_bcreach_small"]

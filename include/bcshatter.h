@@ -126,7 +126,7 @@ typedef struct bcs_opts {
                          once), the small/large threshold (the shared memory
                          a piece may need to take the small path), and the
                          kernel of each large piece with many sources
-                         (whole-GPU, 32-source batches or one source per
+                         (pull, deep, 32-source batches or one source per
                          CTA, each timed on a sample of its sources) */
   int32_t device;     /* CUDA device ordinal; -1 = the current device */
   void *stream;       /* cudaStream_t for all device work; NULL = default */
@@ -162,7 +162,7 @@ typedef struct bcs_stats {
                               to take the small path: fixed, or the autotuner's */
   int64_t tuned;           /* the autotuner's choices this call, as bits: 1 the
                               small/large threshold; 1 << k a large piece on
-                              kernel k (1 whole-GPU, 2 32-source batches, 3 one
+                              kernel k (1 pull, 2 32-source batches, 3 one
                               source per CTA, 5 a thread per pair) */
   double work_nm;          /* sum over pieces of n_c * m_c (m_c undirected) */
   double work_sources_entries; /* sum over processed sources of the piece's CSR entries */

@@ -28,7 +28,7 @@
 // the pipe whatever its active lanes, so the loop runs over successors, not
 // entries), delta = reach - 1 + sigma * sum, c = ident (1 + delta) / sigma.
 //
-// Bound by issue (59 %) and the waits between short levels: 20 bytes of state
+// Bound by issue (54 %) and the waits between short levels: 22 bytes of state
 // per pair leave some 300 pairs of a level in flight per CTA.  On the
 // articulation-vertex workload (130 M pairs, 788 M row entries) 5.0 ms against
 // 7.1 with a group of warps per source, four groups at most and 100 KB; 10
