@@ -469,7 +469,7 @@ static void remember_split(long long key, int choice) {
 //  * the small/large threshold: the shared memory a piece may need for one
 //    source to take the small path (SMALL_LIMITS); pieces above it take the
 //    large-piece path.  Timed over the pieces that fit the largest limit.
-//  * the kernel of each large piece: the whole-GPU kernel (where the
+//  * the kernel of each large piece: the pull kernel (where the
 //    piece's depth allows it), 32-source batches (where its depth is below
 //    4 x MS_DEPTH_LIMIT: their cost grows with the levels of a batch), or
 //    one source per CTA, each timed on a sample of the piece's sources that
@@ -525,7 +525,7 @@ static int time_candidate(Ctx &ctx, const std::vector<CompDesc> &comps, const Bc
 // Times the large-piece kernels on samples of one piece's sources (every
 // vertex a source) and sets *choice to the fastest per source.  The samples
 // are what each kernel sees in a full run: consecutive vertices of the BFS
-// order from the piece's first vertex (d_ord) for the whole-GPU kernel,
+// order from the piece's first vertex (d_ord) for the pull kernel,
 // consecutive ids for the others.
 static int tune_large_piece(Ctx &ctx, const CompDesc &c, const BcInput &in, const BcPlanOpts &po, bool wide_ok,
                             bool deep_ok, int depth, const int32_t *d_ord, int *choice) {
@@ -621,7 +621,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   const std::vector<CompDesc> &comps = po.sources ? comps_src : comps_in;
   // the large-piece kernel, if fixed: by the caller, or by BCS_LARGE_PATH
   // (wide|batched|per_source; wide_all, for tests: every piece runs on the
-  // large-piece path, and on the whole-GPU kernel wherever that can take it)
+  // large-piece path, and on the pull kernel wherever that can take it)
   int lp_mode = po.large_path;
   bool all_large = false;
   if (const char *e = std::getenv("BCS_LARGE_PATH")) {

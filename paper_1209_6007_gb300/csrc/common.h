@@ -52,7 +52,7 @@ struct Status {
 //   BCS_TEST_FAIL_ALLOC=k  the call's device allocations after the first k
 //                          fail as if the device were out of memory;
 //   BCS_TEST_SIGMA_CAP=k   path counts above 2^k count as out of range (the
-//                          whole-GPU Bc-Reach kernel reports BCS_EOVERFLOW).
+//                          pull kernel reports BCS_EOVERFLOW).
 // alloc_budget() < 0: no limit.
 int64_t &alloc_budget();
 

@@ -6,7 +6,7 @@
 // A slab is 256 sources of one piece (consecutive vertices of a BFS order of
 // it, so they sit close together and reach most vertices on the same level)
 // and one row of state per vertex of the piece.  A wave is as many slabs, of
-// any pieces, as give the GPU about PULL_ROWS rows, and the grid-wide wait
+// any pieces, as give the GPU a million rows or more, and the grid-wide wait
 // after every BFS level is paid once per wave.
 //
 // Per row v of a slab:
@@ -53,9 +53,9 @@
 // 2^18 measured 10-15 % slower (the tail of every pass).  Four CTAs per SM: at
 // 48 registers (five) it spills and the FP64 cases lose what FP32 gains.
 // On one GB300, whole calls: 87,000 vertices, 1.15 M entries, FP32 dependencies,
-// every vertex a source 311 ms (1,340 ms with one 64-source batch on the whole
-// GPU and pushed counts); 13,690 vertices FP64 17 ms (80 ms with 32 sources
-// per CTA); 7,009 vertices plain 4.3 ms (21.5 ms with one source per CTA).
+// every vertex a source 303 ms (1,340 ms with one 64-source batch on the whole
+// GPU and pushed counts); 13,690 vertices FP64 14.6 ms (80 ms with 32 sources
+// per CTA); 7,009 vertices plain 3.8 ms (21.5 ms with one source per CTA).
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -76,8 +76,14 @@ constexpr int PULL_WORDS = PULL_W / 32;
 constexpr int PULL_UNIT = 16;    // rows handed out together
 constexpr int PULL_LIST = 64;    // neighbours a warp keeps; longer rows are cut into items
 constexpr int PULL_SHARDS = 8;   // work counters, on separate cache lines
-constexpr int64_t PULL_ROWS = 1 << 20;     // rows of a wave,
-constexpr size_t PULL_BYTES = (size_t)12 << 30;  // and the state they may take (one slab at least)
+// Rows of a wave: PULL_SLABS slabs of the largest piece, from PULL_ROWS to
+// PULL_ROWS_TOP.  Few slabs of a large piece leave a pass uneven (424,000 vertices,
+// two slabs a wave 7.65 s, nine 7.26; 87,000 vertices, 12 slabs 298 ms, 24 289),
+// many of small ones leave L2 (pieces up to 4,096 vertices, 2^20 rows 51.4 ms,
+// 2^21 52.9).
+constexpr int64_t PULL_ROWS = 1 << 20, PULL_ROWS_TOP = 1 << 22;
+constexpr int PULL_SLABS = 24;
+constexpr size_t PULL_BYTES = (size_t)12 << 30;  // the state they may take (one slab at least)
 constexpr int64_t PULL_ROWS_MAX = 1 << 24; // slots of a wave are indexed in 32 bits
 constexpr int PULL_REC = 600;    // log2 of a level's largest count from which the next level keeps one per source
 
@@ -1191,7 +1197,8 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
   size_t free_b = 0, total_b = 0;
   BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
   const size_t per_row = pull_row_bytes(depth), budget = std::min<size_t>(free_b / 2, PULL_BYTES);
-  const int64_t nw = (rows_total + PULL_ROWS - 1) / PULL_ROWS;
+  const int64_t wave_rows = std::max(PULL_ROWS, std::min(PULL_ROWS_TOP, PULL_SLABS * nmax));
+  const int64_t nw = (rows_total + wave_rows - 1) / wave_rows;
   const int64_t target = std::max(up(nmax), up((rows_total + nw - 1) / std::max<int64_t>(nw, 1)) + up(nmax) / 2);
   std::vector<PullSlab> slabs;
   std::vector<int32_t> wave(1, 0);
