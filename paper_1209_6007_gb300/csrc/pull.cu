@@ -53,9 +53,9 @@
 // 2^18 measured 10-15 % slower (the tail of every pass).  Four CTAs per SM: at
 // 48 registers (five) it spills and the FP64 cases lose what FP32 gains.
 // On one GB300, whole calls: 87,000 vertices, 1.15 M entries, FP32 dependencies,
-// every vertex a source 303 ms (1,340 ms with one 64-source batch on the whole
-// GPU and pushed counts); 13,690 vertices FP64 14.6 ms (80 ms with 32 sources
-// per CTA); 7,009 vertices plain 3.8 ms (21.5 ms with one source per CTA).
+// every vertex a source 295 ms (1,340 ms with one 64-source batch on the whole
+// GPU and pushed counts); 13,690 vertices FP64 14.5 ms (80 ms with 32 sources
+// per CTA); 7,009 vertices plain 3.9 ms (21.5 ms with one source per CTA).
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
