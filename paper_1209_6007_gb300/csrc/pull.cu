@@ -73,7 +73,14 @@ constexpr int PULL_WARPS = PULL_THREADS / 32;
 constexpr int PULL_CTAS = 4;     // per SM (register budget: 64)
 constexpr int PULL_W = 256;      // sources of a slab
 constexpr int PULL_WORDS = PULL_W / 32;
-constexpr int PULL_UNIT = 16;    // rows handed out together
+constexpr int PULL_LGU = 4;
+constexpr int PULL_UNIT = 1 << PULL_LGU;  // rows handed out together
+// or fewer (a power of two) while a wave has no more than PULL_SPREAD of these
+// per warp: a warp takes its rows one after the other, and few units leave the
+// other warps idle (a ring of 1,600 vertices joined to 21 neighbours on either
+// side: 9.8 ms in sixteens, 3.0 with 2 per warp, 2.6 with 4 and with 8).  Not
+// where most rows are long: those are items, and the units would be empty.
+constexpr int PULL_SPREAD = 4;
 constexpr int PULL_LIST = 64;    // neighbours a warp keeps; longer rows are cut into items
 constexpr int PULL_SHARDS = 8;   // work counters, on separate cache lines
 // Rows of a wave: PULL_SLABS slabs of the largest piece, from PULL_ROWS to
@@ -392,6 +399,7 @@ template <bool REACH, bool IDENT, bool FP32>
 __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const __grid_constant__ PullArgs A) {
   using Real = typename std::conditional<FP32, float, double>::type;
   __shared__ PullWarp s_warp[PULL_WARPS];
+  __shared__ int s_lgu;  // log2 of a unit's rows (in a register it costs the FP32 case 2.7 %)
   const int lane = threadIdx.x & 31;
   PullWarp &W = s_warp[threadIdx.x >> 5];
   const int64_t gtid = (int64_t)blockIdx.x * PULL_THREADS + threadIdx.x;
@@ -428,10 +436,16 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
     const PullSlab *const slabs = A.slabs + s0;
     const int nu = (slabs[J - 1].row0 + slabs[J - 1].n + PULL_UNIT - 1) / PULL_UNIT;
     const int nh = slabs[J - 1].h0 + slabs[J - 1].nh;
-    const int total = nh + nu;  // items first
+    int total;  // items first
+    {
+      int lgu = PULL_LGU;
+      while (lgu > 0 && nh < nu * (PULL_UNIT / 2) && nh + (nu << (PULL_LGU + 1 - lgu)) <= PULL_SPREAD * nwarps) lgu--;
+      if (threadIdx.x == 0) s_lgu = lgu;  // read after the waits below
+      total = nh + (nu << (PULL_LGU - lgu));
+    }
     const int take = max(1, min(8, nu / (nwarps * 8)));
     // ---------------------------------------------- the wave's tables
-    for (int64_t i = gtid; i < total; i += nthreads) {
+    for (int64_t i = gtid; i < nh + nu; i += nthreads) {
       const bool item = i < nh;
       const int key = item ? (int)i : (int)(i - nh) * PULL_UNIT;
       int lo = 0, hi = J;  // the last slab that starts at or before the key
@@ -482,7 +496,9 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
     // Unit u of a pass; its rows' masks (of `masks`, complemented with flip)
     // in W.want.  Rows without a source, and long rows, are not walked.
     auto load_unit = [&](int u, PullUnit &U, PullItem &it, bool walk, const uint32_t *masks, uint32_t flip) {
-      U.j = A.umap[u];
+      const int lgu = *(volatile int *)&s_lgu;
+      const uint32_t r0 = (uint32_t)(u - nh) << lgu;
+      U.j = A.umap[u < nh ? (uint32_t)u : nh + r0 / PULL_UNIT];
       const PullSlab sl = slabs[U.j];
       const PullJobDev jb = A.jobs[sl.job];
       U.row0 = (uint32_t)sl.row0;
@@ -491,9 +507,9 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
       int64_t b = 0, e = 0;
       int rows = 1;
       if (u >= nh) {
-        U.r0 = (uint32_t)(u - nh) * PULL_UNIT;
+        U.r0 = r0;
         U.v0 = (int32_t)(U.r0 - U.row0);
-        rows = min(PULL_UNIT, sl.n - U.v0);
+        rows = min(1 << lgu, sl.n - U.v0);  // none past the slab's last row
         if (lane <= rows) b = __ldg(row + U.v0 + lane);
         e = __shfl_down_sync(0xffffffffu, b, 1);
         U.own = __ballot_sync(0xffffffffu, lane < rows && e - b <= PULL_LIST);
