@@ -62,6 +62,28 @@ constexpr int DEEP_MIN_ECC = 40;
 constexpr int MID_SOURCES = 2;
 constexpr int MID_PIECE_ECC = 8;
 constexpr int64_t MID_MIN_ROWS = 1 << 15;
+// Source lists of at most one round of CTAs (three per SM).  All kernels then
+// wait for the latency of their levels, one source per CTA for the fewest, and
+// the search by one CTA that orders the sources for the others takes about as
+// long as one source.
+// Graphs of up to FEW_MAX_N vertices whose entries and longest row take one
+// source in a CTA of its own less than FEW_US: no search (15,200 vertices in 38
+// layers, 32 sources, 0.93 ms, 2.4 on the pull kernel; a ring of 6,000, 1 source,
+// 9.7 ms, 18 on the deep one).  Above it the pull kernel is sooner (20,000
+// vertices of a power law, 300 sources, 1.4 ms and 2.4), if the graph is not
+// deep.  Of mean degree FEW_MEAN_DEG or less it may be a road, where more than
+// FEW_ROAD_SOURCES are worth the order (a square grid of 10,000: 400 sources
+// 1.8 ms on the deep kernel, 2.8; 1 source 1.5 and 1.1).  Above FEW_DENSE_DEG the
+// pull kernel cuts the rows, and is sooner (800 vertices of degree 100 in a few
+// levels, 1 source 0.48 ms and 0.58; 1,600 in 16 levels 0.86 and 1.02).
+constexpr int32_t FEW_MAX_N = 16384;
+constexpr double FEW_US = 470.0;
+constexpr int64_t FEW_MEAN_DEG = 6, FEW_ROAD_SOURCES = 32, FEW_DENSE_DEG = 64;
+static double one_source_us(const CompDesc &c) { return 1.8e-3 * (double)c.nnz + 1.2 * c.maxdeg; }
+// The search is given up after these levels: of any width where a graph is small
+// and no road, else when they hold few vertices (20,000 in a path, 30 sources: 54
+// ms so, 105 with the order).
+constexpr PieceBfsEnd FEW_END = {12, INT32_MAX}, FEW_NARROW_END = {256, 16};
 // BCS_LARGE_PATH=mid: the pull kernel on connected pieces of at most this
 // many vertices and MID_MAX_ECC levels
 constexpr int MID_MAX_N = 65536;
@@ -745,9 +767,17 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     std::vector<int32_t> rest, cand;
     std::vector<int64_t> off;
     int64_t total = 0;
+    PieceBfsEnd end;
+    bool no_search = false;
+    if (po.sources && po.nsources <= 3 * (int64_t)ctx.num_sms && lp_mode == LARGE_PATH_AUTO) {
+      const CompDesc &c = comps[0];
+      const bool road = c.nnz <= FEW_MEAN_DEG * c.n, small_n = c.n < FEW_MAX_N && c.nnz <= FEW_DENSE_DEG * c.n;
+      no_search = small_n && one_source_us(c) < FEW_US && (po.nsources <= FEW_ROAD_SOURCES || !road);
+      end = small_n && !road ? FEW_END : FEW_NARROW_END;
+    }
     for (int32_t ci : large) {
       const CompDesc &c = comps[ci];
-      if (none || (c.src_off >= 0 && !po.sources) || (force_mid && c.n > MID_MAX_N)) {
+      if (none || no_search || (c.src_off >= 0 && !po.sources) || (force_mid && c.n > MID_MAX_N)) {
         rest.push_back(ci);
         continue;
       }
@@ -770,13 +800,17 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       BCS_TRY(pull_parent.alloc(total, ctx.stream));
     }
     std::vector<int32_t> cta_depth, cta_reached;
-    BCS_TRY(piece_bfs(ctx, comps, d_comps.p, cand, in, off, pull_order.p, pull_parent.p, &cta_depth, &cta_reached));
+    BCS_TRY(piece_bfs(ctx, comps, d_comps.p, cand, in, off, pull_order.p, pull_parent.p, end, &cta_depth, &cta_reached));
     for (size_t k = 0; k < nlarge; k++) {
       const int32_t ci = cand[k];
       const CompDesc &c = comps[ci];
       int32_t *const ord = pull_order.p + off[k];
       int depth = cta_depth[k];
       int64_t reached = cta_reached[k];
+      if (reached == -2) {
+        rest.push_back(ci);
+        continue;
+      }
       if (reached < 0)  // large and wide: the whole GPU
         BCS_TRY(bfs_queue(ctx, in.row + c.row_off, in.col, c.n, 0, ord, pull_parent.p + off[k], &depth, &reached));
       if (reached != c.n && c.row_off == 0 && !force_mid) {
@@ -829,7 +863,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         BCS_CUDA(cudaMemcpyAsync(ord + c.n, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
         BCS_CUDA(cudaStreamSynchronize(ctx.stream));
       }
-      if (po.sources && take) BCS_TRY(sort_by_position(ctx, c.n, ord, ord + c.n, po.nsources));
+      if (po.sources && take && po.nsources > 256)  // one slab's order is no matter
+        BCS_TRY(sort_by_position(ctx, c.n, ord, ord + c.n, po.nsources));
       const int64_t src_off = po.sources ? off[k] + c.n : -1;
       if (take) pull.push_back(PullJob{ci, (int32_t)nsrc_of(c), bound, po.sources ? src_off : off[k]});
       else deep.push_back(DeepJob{ci, (int32_t)nsrc_of(c), bound, off[k], src_off});

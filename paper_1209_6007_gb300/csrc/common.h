@@ -371,9 +371,14 @@ bool deep_takes(const CompDesc &c, int depth_bound, size_t free_bytes);
 // vertices in the order reached at order[ord_off[i] ..), their tree parents
 // (-1: the root) at parent[ord_off[i] ..), the deepest level and the number
 // reached (host results; synchronises).  A piece of more than
-// PIECE_BFS_MAX_N vertices is given up, reached -1, when a level is wide.
+// PIECE_BFS_MAX_N vertices is given up, reached -1, when a level is wide; any
+// piece, reached -2, when it has `levels` or more of at most `width` vertices
+// each on average.
+struct PieceBfsEnd {
+  int levels = INT32_MAX, width = 0;
+};
 int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_comps, const std::vector<int32_t> &list,
-              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent,
+              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent, PieceBfsEnd end,
               std::vector<int32_t> *depth, std::vector<int32_t> *reached);
 // BFS of a connected graph from `root` (rows at rp[v]..rp[v+1] of col):
 // queue_out[0..*reached) the vertices in the order the search reaches them,

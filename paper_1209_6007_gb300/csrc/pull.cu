@@ -999,7 +999,7 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
                                                                  const int32_t *__restrict__ g_col,
                                                                  const int64_t *__restrict__ ord_off, int32_t *order,
                                                                  int32_t *parent, int32_t *level, int32_t *depth,
-                                                                 int32_t *reached) {
+                                                                 int32_t *reached, PieceBfsEnd end) {
   __shared__ int s_i, s_tail, s_nlong, s_nhuge;
   __shared__ int32_t s_ring[2][PIECE_BFS_RING];
   __shared__ int32_t s_long[PIECE_BFS_LONGS], s_huge[PIECE_BFS_HUGES];
@@ -1080,16 +1080,17 @@ __global__ void __launch_bounds__(PIECE_BFS_THREADS) k_piece_bfs(const CompDesc 
       __syncthreads();
       L++;
       if (c.n > PIECE_BFS_MAX_N && hi - lo > PIECE_BFS_WIDE) break;
+      if (lo < hi && L >= end.levels && hi <= (int64_t)end.width * L) break;
     }
     if (threadIdx.x == 0) {
       depth[i] = L - 1;
-      reached[i] = lo < hi ? -1 : hi;
+      reached[i] = lo == hi ? hi : L >= end.levels && hi <= (int64_t)end.width * L ? -2 : -1;
     }
   }
 }
 
 int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_comps, const std::vector<int32_t> &list,
-              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent,
+              const BcInput &in, const std::vector<int64_t> &ord_off, int32_t *order, int32_t *parent, PieceBfsEnd end,
               std::vector<int32_t> *depth, std::vector<int32_t> *reached) {
   const int P = (int)list.size();
   depth->assign(P, 0);
@@ -1107,7 +1108,8 @@ int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_co
   BCS_CUDA(cudaMemcpyAsync(d_off.p, ord_off.data(), P * sizeof(int64_t), cudaMemcpyHostToDevice, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(d_out.p + 2 * P, 0, sizeof(int32_t), ctx.stream));
   k_piece_bfs<<<std::min(P, ctx.num_sms * 2), PIECE_BFS_THREADS, 0, ctx.stream>>>(
-      d_comps, d_list.p, P, d_out.p + 2 * P, in.row, in.col, d_off.p, order, parent, d_level.p, d_out.p, d_out.p + P);
+      d_comps, d_list.p, P, d_out.p + 2 * P, in.row, in.col, d_off.p, order, parent, d_level.p, d_out.p, d_out.p + P,
+      end);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
   BCS_CUDA(cudaMemcpyAsync(depth->data(), d_out.p, P * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx.stream));
