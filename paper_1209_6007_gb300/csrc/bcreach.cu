@@ -50,6 +50,16 @@ constexpr int MS_DEPTH_LIMIT = 64;
 // Large pieces whose BFS eccentricity (from their first vertex) is at most
 // PULL_MAX_ECC run on the pull kernel (pull.cu)
 constexpr int PULL_MAX_ECC = 40;
+// (a whole graph of several components, of n vertices of which `pairs` ordered
+// pairs share one: unless they are many small ones.  The pull kernel looks at
+// every vertex for every slab of sources, some 0.65 ps a level and (source,
+// vertex), and at the pairs for 60; the kernels below at the pairs alone, for
+// 200 to 400, and 20 ns a source.  1,000 paths of 30 vertices: 18 ms on it, 2.0
+// on them, 10,000 paths 1,071 and 13; 30 power-law graphs of 1,000 8.3 and 6.6;
+// one of 5,000 and 3,000 rings of 9 5.2 and 12)
+static bool pull_reaches(int64_t n, int64_t pairs, int depth) {
+  return (depth + 1.0) * (double)n * (double)n < 370.0 * (double)pairs + 3e4 * (double)n;
+}
 // and deeper ones than this, of small degree, on the deep kernel (deep.cu)
 constexpr int DEEP_MIN_ECC = 40;
 // Pieces that cannot run MID_SOURCES sources at once in that budget (some 800
@@ -82,7 +92,10 @@ constexpr int64_t FEW_MEAN_DEG = 6, FEW_ROAD_SOURCES = 32, FEW_DENSE_DEG = 64;
 static double one_source_us(const CompDesc &c) { return 1.8e-3 * (double)c.nnz + 1.2 * c.maxdeg; }
 // The search is given up after these levels: of any width where a graph is small
 // and no road, else when they hold few vertices (20,000 in a path, 30 sources: 54
-// ms so, 105 with the order).
+// ms so, 105 with the order).  Where it ends in a small component of such a graph
+// (and of at most FEW_APART_MAX_N vertices: a CTA's state is cleared for it) the
+// others are not searched: 5,000 rings of 9, 200 sources 0.36 ms, 0.66 with them.
+constexpr int32_t FEW_APART_MAX_N = 1 << 17;
 constexpr PieceBfsEnd FEW_END = {12, INT32_MAX}, FEW_NARROW_END = {256, 16};
 // BCS_LARGE_PATH=mid: the pull kernel on connected pieces of at most this
 // many vertices and MID_MAX_ECC levels
@@ -769,7 +782,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     int64_t total = 0;
     PieceBfsEnd end;
     bool no_search = false;
-    if (po.sources && po.nsources <= 3 * (int64_t)ctx.num_sms && lp_mode == LARGE_PATH_AUTO) {
+    const bool few = po.sources && po.nsources <= 3 * (int64_t)ctx.num_sms && lp_mode == LARGE_PATH_AUTO;
+    if (few) {
       const CompDesc &c = comps[0];
       const bool road = c.nnz <= FEW_MEAN_DEG * c.n, small_n = c.n < FEW_MAX_N && c.nnz <= FEW_DENSE_DEG * c.n;
       no_search = small_n && one_source_us(c) < FEW_US && (po.nsources <= FEW_ROAD_SOURCES || !road);
@@ -807,7 +821,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       int32_t *const ord = pull_order.p + off[k];
       int depth = cta_depth[k];
       int64_t reached = cta_reached[k];
-      if (reached == -2) {
+      bool apart = false;  // a graph of many small components
+      if (reached == -2 || (few && reached >= 0 && reached < c.n / 4 && c.n <= FEW_APART_MAX_N && one_source_us(c) < FEW_US)) {
         rest.push_back(ci);
         continue;
       }
@@ -817,8 +832,10 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         // a whole graph of several components (the plain calls; pieces are
         // connected): every component searched from its smallest vertex
         DevGraph g{c.n, c.nnz, in.row, in.col};
-        BCS_TRY(bfs_queue_components(ctx, g, ord, pull_parent.p + off[k], &depth));
+        int64_t pairs = 0;
+        BCS_TRY(bfs_queue_components(ctx, g, ord, pull_parent.p + off[k], &depth, &pairs));
         reached = c.n;
+        apart = !pull_reaches(c.n, pairs, depth);
       }
       // every source's BFS depth is at most twice its component's root's
       const int bound = 2 * depth + 2;
@@ -845,7 +862,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         if (choice == LARGE_PATH_PER_SOURCE) ps_tuned.push_back(ci);
         if (choice != LARGE_PATH_WIDE && choice != LARGE_PATH_DEEP) continue;
       }
-      bool take = ok && lp_mode != LARGE_PATH_DEEP && choice != LARGE_PATH_DEEP;
+      bool take = ok && lp_mode != LARGE_PATH_DEEP && choice != LARGE_PATH_DEEP && (!apart || force_wide || choice == LARGE_PATH_WIDE);
       if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) take = take && depth <= PULL_MAX_ECC;
       const size_t state = pull_piece_bytes(c.n, c.nnz, bound);
       if (take && state > ((size_t)1 << 30)) {  // its state has to fit

@@ -387,8 +387,9 @@ int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_co
 int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_t root, int32_t *queue_out,
               int32_t *parent, int *depth, int64_t *reached);
 // BFS order of every connected component of g (rows start at 0), each from
-// its smallest vertex, components contiguous; *depth the deepest level
-int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth);
+// its smallest vertex, components contiguous; *depth the deepest level, *pairs
+// the ordered pairs of vertices (v, v among them) that share a component
+int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth, int64_t *pairs);
 // pieces of at most this many vertices are searched one per CTA
 constexpr int PIECE_BFS_MAX_N = 32768;
 

@@ -348,12 +348,21 @@ int bfs_queue(Ctx &ctx, const int64_t *rp, const int32_t *col, int64_t n, int32_
   return BCS_OK;
 }
 
+__global__ void k_sum_i64(int64_t n, const int64_t *__restrict__ x, unsigned long long *sum) {
+  unsigned long long t = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) t += x[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(sum, t);
+}
+
 // BFS order of every connected component at once (each from its smallest
 // vertex), the components kept contiguous: queue_out[0..n), *depth the
-// deepest level over all components.
-int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth) {
+// deepest level over all components, *pairs the vertex pairs that share one.
+int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_t *parent, int *depth, int64_t *pairs) {
   const int64_t n = g.n;
   *depth = 0;
+  *pairs = 0;
   if (n == 0) return BCS_OK;
   DBuf<int32_t> label, level;
   DBuf<int64_t> N;
@@ -361,6 +370,12 @@ int bfs_queue_components(Ctx &ctx, const DevGraph &g, int32_t *queue_out, int32_
   BCS_TRY(label.alloc(n, ctx.stream));
   BCS_TRY(N.alloc(n, ctx.stream));
   BCS_TRY(launch_cc(ctx, g, label.p, N.p));
+  DBuf<unsigned long long> sum;
+  BCS_TRY(sum.alloc(1, ctx.stream));
+  BCS_CUDA(cudaMemsetAsync(sum.p, 0, sizeof(unsigned long long), ctx.stream));
+  k_sum_i64<<<grid_of(n, 256, ctx.num_sms * 8), 256, 0, ctx.stream>>>(n, N.p, sum.p);
+  ctx.launches++;
+  BCS_CUDA(cudaMemcpyAsync(pairs, sum.p, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx.stream));
   BCS_TRY(level.alloc(n, ctx.stream));
   BCS_TRY(lcount.alloc(n + 2, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(lcount.p, 0, (n + 2) * sizeof(unsigned long long), ctx.stream));
