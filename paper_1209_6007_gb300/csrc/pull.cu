@@ -1241,8 +1241,12 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
   A.flg = 0;
   while (((int64_t)1 << A.flg) < fan) A.flg++;
   // counts can only come near the end of the double range when the levels
-  // allow it (ident adds at most flg bits per level)
-  const bool may_scale = (int64_t)lcap * 2 * std::max(A.flg, 1) > PULL_REC;
+  // allow it (ident is at most fan: pieces merged more than once have few
+  // neighbours of large ident, so the degree alone is no bound)
+  int fan_lg = 0;
+  for (const PullJob &j : jobs)
+    while ((double)((int64_t)1 << fan_lg) < comps[j.ci].fan) fan_lg++;
+  const bool may_scale = (int64_t)lcap * std::max(A.flg + (in.ident ? fan_lg : 0), 1) > PULL_REC;
   DBuf<PullSlab> d_slabs;
   DBuf<int32_t> d_wave, umap, ctr, hctr, idmax;
   DBuf<PullJobDev> d_jobs;
@@ -1318,7 +1322,7 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
   A.bar = GridBarrier{(unsigned int *)barw.p, (unsigned int *)barw.p + 1, d_err, (long long)ctx.max_wait};
   A.err = d_err;
   A.dag_total = d_dag;
-  A.sig_cap = ctx.sigma_cap_lg2;
+  A.sig_cap = std::min(ctx.sigma_cap_lg2, 1024);  // 1024: infinities
   const bool R = in.reach != nullptr || in.init != nullptr, I = in.ident != nullptr;
   BCS_TRY(BCS_DISPATCH3(pull_launch_t, R, I, fp32, ctx, A));
   ctx.stats.n_wide_batches += nbatches;
