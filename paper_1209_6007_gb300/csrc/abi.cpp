@@ -22,7 +22,40 @@ int64_t &alloc_budget() {
   static thread_local int64_t budget = -1;
   return budget;
 }
+int64_t &test_memory() {
+  static thread_local int64_t bytes = 0;
+  return bytes;
+}
 const std::string &get_error() { return t_err; }
+
+static bool pool_bytes(uint64_t *reserved, uint64_t *used) {
+  int dev = 0;
+  cudaMemPool_t pool;
+  return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+         cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, reserved) == cudaSuccess &&
+         cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, used) == cudaSuccess;
+}
+
+size_t pool_used() {
+  uint64_t reserved = 0, used = 0;
+  return pool_bytes(&reserved, &used) ? (size_t)used : 0;
+}
+
+int device_free_bytes(size_t *out) {
+  size_t free_b = 0, total_b = 0;
+  uint64_t reserved = 0, used = 0;
+  BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  if (!pool_bytes(&reserved, &used)) {
+    set_error("the device's memory pool cannot be read");
+    return BCS_ECUDA;
+  }
+  *out = free_b + (size_t)(reserved > used ? reserved - used : 0);
+  if (test_memory() > 0) {
+    const size_t limit = (size_t)test_memory();
+    *out = std::min(*out, limit > used ? limit - (size_t)used : 0);
+  }
+  return BCS_OK;
+}
 
 StageTimer::StageTimer(cudaStream_t stream) : s(stream) {
   cudaEventCreate(&a);
@@ -138,6 +171,8 @@ int make_ctx(const bcs_opts *opts, Ctx *ctx) {
   ctx->autotune = opts && opts->autotune;
   const char *fa = std::getenv("BCS_TEST_FAIL_ALLOC");
   alloc_budget() = fa ? std::max<int64_t>(0, std::atoll(fa)) : -1;
+  const char *tm = std::getenv("BCS_TEST_MEMORY");
+  test_memory() = tm ? std::max<int64_t>(0, std::atoll(tm)) : 0;
   if (const char *sc = std::getenv("BCS_TEST_SIGMA_CAP")) ctx->sigma_cap_lg2 = std::max(1, std::atoi(sc));
   return BCS_OK;
 }

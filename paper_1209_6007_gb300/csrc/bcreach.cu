@@ -842,8 +842,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       const bool ok = bound <= pull_depth_limit() && reached == c.n && (!force_mid || depth <= MID_MAX_ECC);
       bool deep_ok = false;
       if (reached == c.n && (lp_mode == LARGE_PATH_DEEP || (depth > DEEP_MIN_ECC && !force_wide && !force_mid))) {
-        size_t free_b = 0, total_b = 0;
-        BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        size_t free_b = 0;
+        BCS_TRY(device_free_bytes(&free_b));
         deep_ok = deep_takes(c, bound, free_b);
       }
       // tuning pays only over many sources
@@ -866,8 +866,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) take = take && depth <= PULL_MAX_ECC;
       const size_t state = pull_piece_bytes(c.n, c.nnz, bound);
       if (take && state > ((size_t)1 << 30)) {  // its state has to fit
-        size_t free_b = 0, total_b = 0;
-        BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        size_t free_b = 0;
+        BCS_TRY(device_free_bytes(&free_b));
         take = state <= free_b / 4 * 3;
       }
       if (!take && !deep_ok) {
@@ -1153,8 +1153,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     BCS_CUDA(cudaMemsetAsync(counter.p, 0, sizeof(unsigned long long), ctx.stream));
     // CTAs: up to 3 per SM, fewer when the scratch would take more than half
     // of the free device memory
-    size_t free_b = 0, total_b = 0;
-    BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    size_t free_b = 0;
+    BCS_TRY(device_free_bytes(&free_b));
     int64_t grid = (int64_t)ctx.num_sms * 3;
     grid = std::min<int64_t>(grid, (int64_t)w.size());
     const size_t per = large_scratch_bytes(nmax_large);

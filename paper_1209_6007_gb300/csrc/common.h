@@ -53,8 +53,17 @@ struct Status {
 //                          fail as if the device were out of memory;
 //   BCS_TEST_SIGMA_CAP=k   path counts above 2^k count as out of range (the
 //                          pull kernel reports BCS_EOVERFLOW).
-// alloc_budget() < 0: no limit.
+//   BCS_TEST_MEMORY=k      the device counts as one with k bytes for this
+//                          library: what does not fit is refused.
+// alloc_budget() < 0: no limit; test_memory() 0: no limit.
 int64_t &alloc_budget();
+int64_t &test_memory();
+// bytes of the current device's memory pool in use
+size_t pool_used();
+// Device memory a call can still get: what is free, and what the pool holds
+// without using it (the blocks that earlier calls gave back to it count as used
+// for cudaMemGetInfo: a second call would find less than the first).
+int device_free_bytes(size_t *out);
 
 // ------------------------------------------------------- device buffers
 // Stream-ordered device allocation from the device's default memory pool
@@ -90,6 +99,10 @@ struct DBuf {
     s = stream;
     n = count;
     size_t bytes = (count > 0 ? count : 1) * sizeof(T);
+    if (test_memory() > 0 && pool_used() + bytes > (size_t)test_memory()) {
+      set_error("device allocation refused by BCS_TEST_MEMORY");
+      return BCS_ENOMEM;
+    }
     cudaError_t e = cudaMallocAsync((void **)&p, bytes, stream);
     if (e != cudaSuccess) {
       p = nullptr;

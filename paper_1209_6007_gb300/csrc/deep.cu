@@ -561,8 +561,8 @@ int run_deep(Ctx &ctx, const CompDesc &c, const BcInput &in, bool fp32, const in
   const bool R = in.reach != nullptr || in.init != nullptr, I = in.ident != nullptr;
   // enough sources per CTA that one round of CTAs takes them all, as far as
   // memory and the 32-bit pair ids allow
-  size_t free_b = 0, total_b = 0;
-  BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  BCS_TRY(device_free_bytes(&free_b));
   const size_t budget = std::min<size_t>(free_b / 2, DEEP_BYTES);
   int64_t grid = std::min<int64_t>((int64_t)ctx.num_sms * DEEP_CTAS, nsrc);
   grid = std::max<int64_t>(1, std::min<int64_t>(grid, (int64_t)(budget / deep_cta_bytes(n, depth_bound, 1))));

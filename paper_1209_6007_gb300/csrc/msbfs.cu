@@ -396,8 +396,8 @@ static size_t ms_bytes_per_cta(int64_t nmax) {
 }
 
 int ms_ctas_that_fit(int64_t nmax, int64_t *out) {
-  size_t free_b = 0, total_b = 0;
-  BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  BCS_TRY(device_free_bytes(&free_b));
   *out = (int64_t)(free_b / 2 / ms_bytes_per_cta(nmax));
   return BCS_OK;
 }
@@ -425,8 +425,8 @@ int run_ms(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<int32
   }
   const int64_t qcap = 32 * nmax + 32;
   const size_t per = ms_bytes_per_cta(nmax);
-  size_t free_b = 0, total_b = 0;
-  BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  BCS_TRY(device_free_bytes(&free_b));
   int64_t grid = std::min<int64_t>((int64_t)ctx.num_sms * 2, (int64_t)batches.size());
   if ((size_t)grid * per > free_b / 2) grid = std::max<int64_t>(1, (int64_t)(free_b / 2 / per));
   const size_t G = (size_t)grid, NM = (size_t)nmax;

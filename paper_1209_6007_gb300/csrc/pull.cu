@@ -1198,8 +1198,8 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
     rows_total += (j.nsrc + per_slab - 1) / per_slab * up(comps[j.ci].n);
     nbatches += (j.nsrc + per_batch - 1) / per_batch;
   }
-  size_t free_b = 0, total_b = 0;
-  BCS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  size_t free_b = 0;
+  BCS_TRY(device_free_bytes(&free_b));
   const size_t per_row = pull_row_bytes(depth), budget = std::min<size_t>(free_b / 2, PULL_BYTES);
   const int64_t wave_rows = std::max(PULL_ROWS, std::min(PULL_ROWS_TOP, PULL_SLABS * nmax));
   const int64_t nw = (rows_total + wave_rows - 1) / wave_rows;

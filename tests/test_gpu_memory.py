@@ -1,0 +1,42 @@
+"""Kernels are chosen by the device memory a call can get (needs a CUDA device).
+BCS_TEST_MEMORY=k makes the device one of k bytes for the library (on the host
+only: what does not fit is refused)."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def wheel(n):
+    e = [(0, i) for i in range(1, n)] + [(i, i % (n - 1) + 1) for i in range(1, n)]
+    return gg.from_edges(n, np.array(e), "wheel%d" % n)
+
+
+def test_a_second_call_gets_what_the_first_got(gpu, monkeypatch):
+    """The state of 330,000 vertices, 1.1 GB, has to fit three quarters of what
+    there is: 2.4 GB, less the 1.1 if what the pool keeps counted as used."""
+    g = wheel(330_000)
+    src = np.arange(0, 330_000, 3301)
+    ref = oracle.bc_sources(g, src)
+    monkeypatch.setenv("BCS_TEST_MEMORY", str(2400 * 10**6))
+    for _ in range(2):
+        got = gpu.bc_sources(g.row_ptr, g.col, src)
+        assert gpu.last_stats()["n_wide_batches"] > 0
+        assert float(np.abs(got - ref).max()) <= 1e-12 * float(np.abs(ref).max())
+
+
+def test_state_that_does_not_fit(gpu, monkeypatch):
+    g = wheel(330_000)
+    src = np.arange(0, 330_000, 33001)
+    ref = oracle.bc_sources(g, src)
+    monkeypatch.setenv("BCS_TEST_MEMORY", str(10**9))
+    got = gpu.bc_sources(g.row_ptr, g.col, src)  # another kernel
+    assert gpu.last_stats()["n_wide_batches"] == 0
+    assert float(np.abs(got - ref).max()) <= 1e-12 * float(np.abs(ref).max())
+    monkeypatch.setenv("BCS_TEST_MEMORY", str(10**6))
+    with pytest.raises(gpu.BcsError) as e:
+        gpu.bc_sources(g.row_ptr, g.col, src)
+    assert e.value.code == gpu._lib.BCS_ENOMEM
