@@ -39,6 +39,18 @@
  * reciprocals that the first Bc-Reach call on a device fills (one kernel
  * launch and a device-wide synchronisation).
  *
+ * Device memory: a call allocates what it needs from the device's default
+ * memory pool and gives it back before it returns.  Besides the graph and its
+ * pieces (0.12 GB for 648,000 vertices and 3.4 M entries) that is the searches'
+ * state: of a shallow piece that does not fit shared memory some 3.4 KB per
+ * vertex and batch of 256 sources, for as many batches as fit 12 GB or half of
+ * what is free (one at least); of a deep one 12 bytes per vertex and source
+ * searched at once, up to 32 GB or half of what is free; of the others up to
+ * half of what is free; at most 0.25 GB for the pieces in shared memory.  Where
+ * that does not fit, kernels with less state run.  The pool keeps up to 36 GB
+ * between calls, for the process's next ones (and the pool's other users);
+ * cudaMemPoolTrimTo on the default pool gives it back.
+ *
  * Environment: BCS_TRACE (any value) prints per-stage timings to stderr;
  * BCS_LARGE_PATH=wide|batched|per_source|mid|deep forces the kernel used for
  * pieces too large for shared memory (the whole GPU on one BFS level of many

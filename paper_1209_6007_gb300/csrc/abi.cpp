@@ -160,7 +160,7 @@ int make_ctx(const bcs_opts *opts, Ctx *ctx) {
     if (!g_pool_ready.count(dev)) {
       cudaMemPool_t pool;
       BCS_CUDA(cudaDeviceGetDefaultMemPool(&pool, dev));
-      uint64_t thr = UINT64_MAX;
+      uint64_t thr = POOL_KEEP;
       BCS_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr));
       g_pool_ready.insert(dev);
     }

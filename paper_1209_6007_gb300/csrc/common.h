@@ -66,9 +66,13 @@ size_t pool_used();
 int device_free_bytes(size_t *out);
 
 // ------------------------------------------------------- device buffers
-// Stream-ordered device allocation from the device's default memory pool
-// (its release threshold is raised once per device so freed blocks stay
-// cached between calls).
+// Stream-ordered device allocation from the device's default memory pool.  Its
+// release threshold is raised once per device to POOL_KEEP: blocks that calls
+// give back stay for the next one, as far as the kernels' own limits go (12 GB of
+// the pull kernel, 32 of the deep one); what a piece of tens of millions of
+// vertices takes on top goes back to the device when the call ends (getting a GB
+// and giving it back costs 2 ms).
+constexpr uint64_t POOL_KEEP = (uint64_t)36 << 30;
 template <class T>
 struct DBuf {
   T *p = nullptr;

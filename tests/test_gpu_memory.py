@@ -1,6 +1,8 @@
 """Kernels are chosen by the device memory a call can get (needs a CUDA device).
 BCS_TEST_MEMORY=k makes the device one of k bytes for the library (on the host
 only: what does not fit is refused)."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -40,3 +42,15 @@ def test_state_that_does_not_fit(gpu, monkeypatch):
     with pytest.raises(gpu.BcsError) as e:
         gpu.bc_sources(g.row_ptr, g.col, src)
     assert e.value.code == gpu._lib.BCS_ENOMEM
+
+
+def test_the_pool_keeps_a_bounded_amount(gpu):
+    g = gg.config(1)
+    gpu.bc_shattered(g.row_ptr, g.col)
+    cuda = ctypes.CDLL("libcuda.so.1")
+    dev, pool, keep = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_uint64()
+    assert cuda.cuDeviceGet(ctypes.byref(dev), 0) == 0
+    assert cuda.cuDeviceGetDefaultMemPool(ctypes.byref(pool), dev) == 0
+    release_threshold = 4  # CU_MEMPOOL_ATTR_RELEASE_THRESHOLD
+    assert cuda.cuMemPoolGetAttribute(pool, release_threshold, ctypes.byref(keep)) == 0
+    assert 0 < keep.value <= 40 * 2**30
