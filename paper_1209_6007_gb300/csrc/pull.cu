@@ -1132,17 +1132,10 @@ static int pull_launch_t(Ctx &ctx, PullArgs &A) {
   return BCS_OK;
 }
 
-int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<PullJob> &jobs_in, const BcInput &in,
-             bool fp32, const int32_t *d_order, const CompDesc *d_comps, int per_batch, int *d_err,
-             unsigned long long *d_dag) {
+static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<PullJob> &jobs,
+                         const BcInput &in, bool fp32, const int32_t *d_order, const CompDesc *d_comps, int per_batch,
+                         int *d_err, unsigned long long *d_dag) {
   const cudaStream_t s = ctx.stream;
-  // deep pieces apart from shallow ones (a wave runs as many levels as its
-  // deepest slab), large ones first
-  std::vector<PullJob> jobs(jobs_in);
-  std::stable_sort(jobs.begin(), jobs.end(), [&](const PullJob &a, const PullJob &b) {
-    const int da = a.depth_bound / 8, db = b.depth_bound / 8;
-    return da != db ? da > db : comps[a.ci].n > comps[b.ci].n;
-  });
   const int NJ = (int)jobs.size();
   // items of long rows
   std::vector<int32_t> nitems(NJ, 0), job_comp(NJ);
@@ -1341,6 +1334,38 @@ int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<Pul
       line += buf;
     }
     std::fprintf(stderr, "[bcs trace] pull passes us:%s\n", line.c_str());
+  }
+  return BCS_OK;
+}
+
+int run_pull(Ctx &ctx, const std::vector<CompDesc> &comps, const std::vector<PullJob> &jobs_in, const BcInput &in,
+             bool fp32, const int32_t *d_order, const CompDesc *d_comps, int per_batch, int *d_err,
+             unsigned long long *d_dag) {
+  // deep pieces apart from shallow ones (a wave runs as many levels as its
+  // deepest slab), large ones first
+  std::vector<PullJob> jobs(jobs_in);
+  std::stable_sort(jobs.begin(), jobs.end(), [&](const PullJob &a, const PullJob &b) {
+    const int da = a.depth_bound / 8, db = b.depth_bound / 8;
+    return da != db ? da > db : comps[a.ci].n > comps[b.ci].n;
+  });
+  // A launch's rows have masks for the levels of its deepest piece.  Where a
+  // shallow piece would outgrow a launch's memory by that (it was let in by its
+  // own levels), a launch for every depth.
+  int depth = 0;
+  for (const PullJob &j : jobs) depth = std::max(depth, j.depth_bound);
+  bool apart = false;
+  for (const PullJob &j : jobs)
+    apart = apart || (j.depth_bound / 8 != depth / 8 &&
+                      pull_piece_bytes(comps[j.ci].n, comps[j.ci].nnz, depth) > PULL_ONE_LAUNCH);
+  for (size_t a = 0; a < jobs.size();) {
+    size_t b = jobs.size();
+    if (apart) {
+      b = a;
+      while (b < jobs.size() && jobs[b].depth_bound / 8 == jobs[a].depth_bound / 8) b++;
+    }
+    BCS_TRY(run_pull_jobs(ctx, comps, std::vector<PullJob>(jobs.begin() + a, jobs.begin() + b), in, fp32, d_order,
+                          d_comps, per_batch, d_err, d_dag));
+    a = b;
   }
   return BCS_OK;
 }

@@ -54,3 +54,20 @@ def test_the_pool_keeps_a_bounded_amount(gpu):
     release_threshold = 4  # CU_MEMPOOL_ATTR_RELEASE_THRESHOLD
     assert cuda.cuMemPoolGetAttribute(pool, release_threshold, ctypes.byref(keep)) == 0
     assert 0 < keep.value <= 40 * 2**30
+
+
+def test_a_large_shallow_piece_beside_a_small_deep_one(gpu, monkeypatch):
+    """330,000 vertices of two levels take 1.2 GB of the 1.9 there are; with room
+    for the 80 levels of a ring of 1,600 in the same batch it would be 2."""
+    m = 329_999  # vertices of the rim
+    a = np.arange(1600)
+    ring = gg.from_edges(1600, np.concatenate([np.stack([a, (a + j) % 1600], 1) for j in range(1, 22)]))
+    both = gg.disjoint_union(wheel(m + 1), ring)
+    monkeypatch.setenv("BCS_TEST_MEMORY", str(1900 * 10**6))
+    got = gpu.bc_shattered_batch(np.array([0, m + 1, both.n]), both.row_ptr, both.col)
+    assert gpu.last_stats()["n_wide_batches"] == -(-(m + 1) // 64) + 25
+    # of a rim's ordered pairs that are not neighbours the paths cross the hub, those two apart the one between as well
+    assert got[0] == m * (m - 3) - m
+    assert np.array_equal(got[1:m + 1], np.ones(m))
+    ref = oracle.bc(ring)
+    assert float(np.abs(got[m + 1:] - ref).max()) <= 1e-12 * float(ref.max())
