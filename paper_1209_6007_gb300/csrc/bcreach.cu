@@ -864,11 +864,10 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       }
       bool take = ok && lp_mode != LARGE_PATH_DEEP && choice != LARGE_PATH_DEEP && (!apart || force_wide || choice == LARGE_PATH_WIDE);
       if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) take = take && depth <= PULL_MAX_ECC;
-      const size_t state = pull_piece_bytes(c.n, c.nnz, bound);
-      if (take && state > PULL_ONE_LAUNCH) {  // its state has to fit
+      if (take && (test_memory() > 0 || pull_piece_bytes(c.n, c.nnz, bound) > PULL_ONE_LAUNCH)) {  // its state has to fit
         size_t free_b = 0;
         BCS_TRY(device_free_bytes(&free_b));
-        take = state <= free_b / 4 * 3;
+        take = pull_width(c.n, c.nnz, bound, free_b) > 0;
       }
       if (!take && !deep_ok) {
         rest.push_back(ci);

@@ -375,8 +375,10 @@ int recip_table(Ctx &ctx, const double **out);
 // deepest BFS level run_pull can index
 int pull_depth_limit();
 // bytes of device state one slab of a piece takes, at most; above
-// PULL_ONE_LAUNCH a piece is taken if three quarters of the memory there is hold it
+// PULL_ONE_LAUNCH a piece is taken if three quarters of the memory there is hold
+// it, if need be with fewer sources to a slab: pull_width, 0 if with none
 constexpr size_t PULL_ONE_LAUNCH = (size_t)1 << 30;
+int pull_width(int64_t n, int64_t nnz, int depth_bound, size_t free_bytes);
 size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound);
 // Bc-Reach on one deep piece of small degree, each CTA searching several
 // sources at once (deep.cu).  d_bfs, d_parent: the piece's vertices in BFS order

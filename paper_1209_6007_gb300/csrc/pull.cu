@@ -91,7 +91,8 @@ constexpr int PULL_SHARDS = 8;   // work counters, on separate cache lines
 constexpr int64_t PULL_ROWS = 1 << 20, PULL_ROWS_TOP = 1 << 22;
 constexpr int PULL_SLABS = 24;
 constexpr size_t PULL_BYTES = (size_t)12 << 30;  // the state they may take (one slab at least)
-constexpr int64_t PULL_ROWS_MAX = 1 << 24; // slots of a wave are indexed in 32 bits
+constexpr int64_t PULL_ROWS_MAX = 1 << 30; // rows of a wave are indexed in 32 bits
+constexpr int PULL_W_MIN = 32;   // fewest values of a row where memory is short
 constexpr int PULL_REC = 600;    // log2 of a level's largest count from which the next level keeps one per source
 
 struct PullSlab {
@@ -138,6 +139,7 @@ struct PullArgs {
   const int32_t *idmax;     // largest ident
   const double *recip;      // reciprocals of the integers below RECIP_TABLE
   int64_t rows;             // row capacity of a wave
+  uint32_t w;               // NARROW: values of a row in S4 and S8, the most sources of a slab
   int64_t slabs_cap;
   int32_t lcap, flg;        // flg: log2 of the most neighbours of a row
   GridBarrier bar;
@@ -220,11 +222,12 @@ struct SumPairs {  // partial sums of either
   __device__ __forceinline__ double bits() const { return __hiloint2double(__float_as_int(lo), __float_as_int(hi)); }
 };
 
-// Add up the values of source src (< 0: none) of the list entries [i, i + c).
+// Add up the values of source src (< 0: none) of the list entries [i, i + c), w
+// values to a row of V.
 // Every sum takes zeros for the entries the source is not in, so that the
 // loads of four entries are in flight together and no lane branches.
 template <class Sum>
-__device__ __forceinline__ void pull_sum(Sum &a, const PullWarp &W, int i, int c, const void *V, int src) {
+__device__ __forceinline__ void pull_sum(Sum &a, const PullWarp &W, int i, int c, const void *V, int src, uint32_t w) {
   using T = typename Sum::Val;
   const uint32_t bit = src < 0 ? 0u : 1u << (src & 31);
   const uint32_t *m = &W.ent[i].mask[src < 0 ? 0 : src >> 5];
@@ -236,15 +239,15 @@ __device__ __forceinline__ void pull_sum(Sum &a, const PullWarp &W, int i, int c
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       x[q] = 0;
-      if (m[q * STEP] & bit) x[q] = v[(size_t)e[q].from * PULL_W];
+      if (m[q * STEP] & bit) x[q] = v[(size_t)e[q].from * w];
     }
 #pragma unroll
     for (int q = 0; q < 4; q++) a.add(x[q]);
   }
   if (c & 2) {
     T x0 = 0, x1 = 0;
-    if (m[0] & bit) x0 = v[(size_t)e[0].from * PULL_W];
-    if (m[STEP] & bit) x1 = v[(size_t)e[1].from * PULL_W];
+    if (m[0] & bit) x0 = v[(size_t)e[0].from * w];
+    if (m[STEP] & bit) x1 = v[(size_t)e[1].from * w];
     a.add(x0);
     a.add(x1);
     e += 2;
@@ -252,7 +255,7 @@ __device__ __forceinline__ void pull_sum(Sum &a, const PullWarp &W, int i, int c
   }
   if (c & 1) {
     T x0 = 0;
-    if (m[0] & bit) x0 = v[(size_t)e[0].from * PULL_W];
+    if (m[0] & bit) x0 = v[(size_t)e[0].from * w];
     a.add(x0);
   }
 }
@@ -385,7 +388,9 @@ __device__ __forceinline__ int pull_lg(unsigned long long g, bool is_int) {
   return is_int ? 63 - __clzll((long long)g) : (int)((g >> 52) & 0x7ff) - 1023;
 }
 
-template <bool REACH, bool IDENT, bool FP32>
+// NARROW: rows of A.w values, for pieces whose state does not fit with PULL_W (as
+// a number known to the compiler only there: it costs the other 1 to 3 %).
+template <bool REACH, bool IDENT, bool FP32, bool NARROW>
 __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const __grid_constant__ PullArgs A) {
   using Real = typename std::conditional<FP32, float, double>::type;
   __shared__ PullWarp s_warp[PULL_WARPS];
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
   const int64_t gtid = (int64_t)blockIdx.x * PULL_THREADS + threadIdx.x;
   const int64_t nthreads = (int64_t)gridDim.x * PULL_THREADS;
   const int nwarps = (int)(nthreads >> 5);
+  const uint32_t SW = NARROW ? A.w : (uint32_t)PULL_W;
   double *const S8 = A.S8;
   uint32_t *const S4 = A.S4;
   const int idl = IDENT ? 32 - __clz(max(*A.idmax, 1) - 1) : 0;  // ceil(log2)
@@ -470,7 +476,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
         const size_t r = (size_t)sl.row0 + s;
         atomicOr(A.M + r * PULL_WORDS + (k >> 5), 1u << (k & 31));  // a repeated source is two bits of one row
         atomicOr(A.seen + r * PULL_WORDS + (k >> 5), 1u << (k & 31));
-        S4[r * PULL_W + k] = 1u;
+        S4[r * SW + k] = 1u;
         if (REACH || IDENT)
           wsv = (REACH ? (A.g_init ? __ldg(A.g_init + jb.vtx_off + s) + 1.0 : (double)__ldg(A.g_reach + jb.vtx_off + s))
                        : 1.0) *
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
           // the sums of the row's list for src, in the types of the two levels
           auto counts = [&](int i, int c, int src, auto done) {
             auto sum = [&](auto a, const void *V) {
-              pull_sum(a, W, i, c, V, src);
+              pull_sum(a, W, i, c, V, src, SW);
               done(a);
             };
             if (short_next) sum(SumCount<uint32_t, uint32_t>(), S4);
@@ -656,7 +662,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
               const uint32_t g = pull_union(W, i, c, lane);
               if (lane < PULL_WORDS) W.got[k][lane] = g;
               const int n = pull_rank(W, g, lane), id = ident(k);
-              const size_t at = (size_t)(U.r0 + k) * PULL_W;
+              const size_t at = (size_t)(U.r0 + k) * SW;
               for (int t = 0; t < n; t += 32) {
                 const int src = t + lane < n ? (int)W.rank[t + lane] : -1;
                 counts(i, c, src, [&](const auto &a) { store(at, src, a.bits(), id); });
@@ -702,16 +708,16 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
           list_items(u, it);
           const uint32_t g = pull_union(W, 0, it.count, lane);
           const int n = pull_rank(W, g, lane), id = ident(0);
-          const size_t at = (size_t)U.r0 * PULL_W;
+          const size_t at = (size_t)U.r0 * SW;
           for (int t = 0; t < n; t += 32) {
             const int src = t + lane < n ? (int)W.rank[t + lane] : -1;
             if (kind_next) {
               SumI64 a;
-              pull_sum(a, W, 0, it.count, A.hpart, src);
+              pull_sum(a, W, 0, it.count, A.hpart, src, PULL_W);
               store(at, src, a.bits(), id);
             } else {
               SumF64 a;
-              pull_sum(a, W, 0, it.count, A.hpart, src);
+              pull_sum(a, W, 0, it.count, A.hpart, src, PULL_W);
               store(at, src, a.bits(), id);
             }
           }
@@ -752,7 +758,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
           };
           auto row_of = [&](int k) {
             const int64_t v = U.vtx_off + U.v0 + k;
-            return Row{(size_t)(U.r0 + k) * PULL_W, IDENT ? __ldg(A.g_ident + v) : 1,
+            return Row{(size_t)(U.r0 + k) * SW, IDENT ? __ldg(A.g_ident + v) : 1,
                        REACH ? (A.g_init ? (Real)__ldg(A.g_init + v) : (Real)(__ldg(A.g_reach + v) - 1)) : (Real)0};
           };
           // an integer count (exact: the stored value is a multiple of ident)
@@ -845,16 +851,16 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
                 float hi, lo;
                 if (items) {
                   SumPairs a;
-                  pull_sum(a, W, i, c, A.hpart, src);
+                  pull_sum(a, W, i, c, A.hpart, src, PULL_W);
                   hi = a.hi, lo = a.lo;
                 } else if (kind_next) {
                   SumFloat a;
-                  pull_sum(a, W, i, c, S4, src);
+                  pull_sum(a, W, i, c, S4, src, SW);
                   hi = a.hi, lo = a.lo;
                 } else {
                   SumScaled a;
                   a.ex = exponent(r, src);
-                  pull_sum(a, W, i, c, S8, src);
+                  pull_sum(a, W, i, c, S8, src, SW);
                   hi = a.hi, lo = a.lo;
                 }
                 sum = settle32(r, src, hi, lo, sum);
@@ -865,7 +871,7 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
               for (int t = 0; t < n; t += 32) {
                 const int src = t + lane < n ? (int)W.rank[t + lane] : -1;
                 SumF64 a;
-                pull_sum(a, W, i, c, items ? A.hpart : S8, src);
+                pull_sum(a, W, i, c, items ? A.hpart : S8, src, items ? PULL_W : SW);
                 sum += settle64(r, src, a.x);
               }
               add_bc(k, sum);
@@ -903,17 +909,17 @@ __global__ void __launch_bounds__(PULL_THREADS, PULL_CTAS) k_bcreach_pull(const 
                 if constexpr (FP32) {
                   if (kind_next) {
                     SumFloat a;
-                    pull_sum(a, W, i, c, S4, src);
+                    pull_sum(a, W, i, c, S4, src, SW);
                     leave(u, src, have, a, SumPairs());
                   } else {
                     SumScaled a;
                     a.ex = exponent(r, src);
-                    pull_sum(a, W, i, c, S8, src);
+                    pull_sum(a, W, i, c, S8, src, SW);
                     leave(u, src, have, a, SumPairs());
                   }
                 } else {
                   SumF64 a;
-                  pull_sum(a, W, i, c, S8, src);
+                  pull_sum(a, W, i, c, S8, src, SW);
                   leave(u, src, have, a, SumF64());
                 }
               }
@@ -1108,25 +1114,38 @@ int piece_bfs(Ctx &ctx, const std::vector<CompDesc> &comps, const CompDesc *d_co
 int pull_depth_limit() { return 250; }
 
 // bytes of state per row for levels up to depth_bound, and per item of a long row
-static size_t pull_row_bytes(int depth_bound) { return 12 * PULL_W + 4 * PULL_WORDS * (size_t)(depth_bound + 4) + 1; }
+static size_t pull_row_bytes(int depth_bound, int w) { return 12 * (size_t)w + 4 * PULL_WORDS * (size_t)(depth_bound + 4) + 1; }
 constexpr size_t PULL_ITEM_BYTES = 8 * PULL_W + 4 * PULL_WORDS + 8;
 
-size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound) {
+static size_t pull_state_bytes(int64_t n, int64_t nnz, int depth_bound, int w) {
   if (n > PULL_ROWS_MAX - PULL_UNIT) return SIZE_MAX;
-  return (size_t)(n + PULL_UNIT) * pull_row_bytes(depth_bound) + (size_t)(nnz / PULL_LIST) * 2 * PULL_ITEM_BYTES;
+  return (size_t)(n + PULL_UNIT) * pull_row_bytes(depth_bound, w) + (size_t)(nnz / PULL_LIST) * 2 * PULL_ITEM_BYTES;
+}
+size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound) { return pull_state_bytes(n, nnz, depth_bound, PULL_W); }
+
+// The most values to a row with which a piece's state fits three quarters of
+// the memory there is (or PULL_ONE_LAUNCH, with all of them), 0 when not even
+// PULL_W_MIN do: of 200 GB, 58 million vertices of ten levels get 256, 180
+// million 32.
+int pull_width(int64_t n, int64_t nnz, int depth_bound, size_t free_bytes) {
+  if (test_memory() == 0 && pull_piece_bytes(n, nnz, depth_bound) <= PULL_ONE_LAUNCH) return PULL_W;
+  for (int w = PULL_W; w >= PULL_W_MIN; w /= 2)
+    if (pull_state_bytes(n, nnz, depth_bound, w) <= free_bytes / 4 * 3) return w;
+  return 0;
 }
 
 template <bool R, bool I, bool F>
 static int pull_launch_t(Ctx &ctx, PullArgs &A) {
+  const auto kernel = A.w < PULL_W ? k_bcreach_pull<R, I, F, true> : k_bcreach_pull<R, I, F, false>;
   int per_sm = 0;
-  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bcreach_pull<R, I, F>, PULL_THREADS, 0));
+  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, PULL_THREADS, 0));
   if (per_sm < 1) {
     set_error("the pull Bc-Reach kernel cannot be resident");
     return BCS_ECUDA;
   }
   per_sm = std::min(per_sm, PULL_CTAS);
   void *args[] = {(void *)&A};
-  BCS_CUDA(cudaLaunchCooperativeKernel((const void *)k_bcreach_pull<R, I, F>, dim3(ctx.num_sms * per_sm),
+  BCS_CUDA(cudaLaunchCooperativeKernel((const void *)kernel, dim3(ctx.num_sms * per_sm),
                                        dim3(PULL_THREADS), args, 0, ctx.stream));
   ctx.launches++;
   return BCS_OK;
@@ -1144,7 +1163,6 @@ static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std
   DBuf<int64_t> d_itemoff;
   DBuf<PullChunk> d_chunks;
   DBuf<PullItem> d_items;
-  const int per_slab = per_batch * (PULL_W / 64);  // sources of a slab
   int64_t items_total = 0, fan = 1, nmax = 1, rows_total = 0, nbatches = 0;
   int depth = 1;
   {
@@ -1185,15 +1203,19 @@ static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std
       BCS_CUDA(cudaGetLastError());
     }
   }
+  size_t free_b = 0;
+  BCS_TRY(device_free_bytes(&free_b));
+  int w = PULL_W;  // the pieces were let in by pull_width
+  for (const PullJob &j : jobs)
+    w = std::min(w, std::max(PULL_W_MIN, pull_width(comps[j.ci].n, comps[j.ci].nnz, j.depth_bound, free_b)));
+  const int per_slab = std::min(per_batch * (PULL_W / 64), w);  // sources of a slab
   // slabs, cut into waves of about the same number of rows
   auto up = [](int64_t x) { return (x + PULL_UNIT - 1) / PULL_UNIT * PULL_UNIT; };
   for (const PullJob &j : jobs) {
     rows_total += (j.nsrc + per_slab - 1) / per_slab * up(comps[j.ci].n);
     nbatches += (j.nsrc + per_batch - 1) / per_batch;
   }
-  size_t free_b = 0;
-  BCS_TRY(device_free_bytes(&free_b));
-  const size_t per_row = pull_row_bytes(depth), budget = std::min<size_t>(free_b / 2, PULL_BYTES);
+  const size_t per_row = pull_row_bytes(depth, w), budget = std::min<size_t>(free_b / 2, PULL_BYTES);
   const int64_t wave_rows = std::max(PULL_ROWS, std::min(PULL_ROWS_TOP, PULL_SLABS * nmax));
   const int64_t nw = (rows_total + wave_rows - 1) / wave_rows;
   const int64_t target = std::max(up(nmax), up((rows_total + nw - 1) / std::max<int64_t>(nw, 1)) + up(nmax) / 2);
@@ -1256,8 +1278,8 @@ static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std
   BCS_TRY(d_slabs.alloc(slabs.size(), s));
   BCS_TRY(d_wave.alloc(wave.size(), s));
   BCS_TRY(d_jobs.alloc(NJ, s));
-  BCS_TRY(S8.alloc((size_t)rows * PULL_W, s));
-  BCS_TRY(S4.alloc((size_t)rows * PULL_W, s));
+  BCS_TRY(S8.alloc((size_t)rows * w, s));
+  BCS_TRY(S4.alloc((size_t)rows * w, s));
   BCS_TRY(M.alloc((size_t)lcap * rows * PULL_WORDS, s));
   BCS_TRY(seen.alloc((size_t)rows * PULL_WORDS, s));
   BCS_TRY(umap.alloc(rows / PULL_UNIT + hmax, s));
@@ -1310,6 +1332,7 @@ static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std
   A.idmax = idmax.p;
   BCS_TRY(recip_table(ctx, &A.recip));
   A.rows = rows;
+  A.w = (uint32_t)w;
   A.slabs_cap = jmax;
   A.lcap = lcap;
   A.bar = GridBarrier{(unsigned int *)barw.p, (unsigned int *)barw.p + 1, d_err, (long long)ctx.max_wait};
@@ -1320,8 +1343,8 @@ static int run_pull_jobs(Ctx &ctx, const std::vector<CompDesc> &comps, const std
   BCS_TRY(BCS_DISPATCH3(pull_launch_t, R, I, fp32, ctx, A));
   ctx.stats.n_wide_batches += nbatches;
   if (tracing) {  // the first waves' pass times (us)
-    std::fprintf(stderr, "[bcs trace] pull: %d pieces, %zu slabs in %d waves of up to %lld rows, %lld items, %d levels at most\n",
-                 NJ, slabs.size(), A.nwaves, (long long)rows, (long long)hmax, lcap);
+    std::fprintf(stderr, "[bcs trace] pull: %d pieces, %zu slabs in %d waves of up to %lld rows, %lld items, %d levels at most, %d values to a row\n",
+                 NJ, slabs.size(), A.nwaves, (long long)rows, (long long)hmax, lcap, w);
     std::vector<unsigned long long> tr(2 * PULL_TRACE_CAP);
     BCS_CUDA(cudaMemcpyAsync(tr.data(), trace.p, tr.size() * 8, cudaMemcpyDeviceToHost, s));
     BCS_CUDA(cudaStreamSynchronize(s));
