@@ -920,12 +920,14 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     for (size_t k = 0; k < small.size(); k++) sorted[off[cls[k]]++] = small[k];
     small.swap(sorted);
   }
-  bool small_coop = false;
+  double coop_cost = 0.0;
   int64_t small_sources = 0;
   for (int32_t ci : small) {
-    small_coop = small_coop || comps[ci].maxdeg > SMALL_COOP_DEG;
-    small_sources += nsrc_of(comps[ci]);
+    const CompDesc &c = comps[ci];
+    if (c.maxdeg > SMALL_COOP_DEG && c.n > SMALL_COOP_N) coop_cost += (double)nsrc_of(c) * (double)(c.nnz + c.n);
+    small_sources += nsrc_of(c);
   }
+  const bool small_coop = coop_cost > 0.875 * total_small_cost;
   auto plan_small = [&](int ng_cap, size_t budget, std::vector<SmallItem> &out, size_t &smem, int &grid) -> int {
     out.clear();
     smem = 0;

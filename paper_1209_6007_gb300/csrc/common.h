@@ -362,10 +362,12 @@ bool small_takes(int64_t n, int64_t nnz, int G);
 int small_max_sources();
 int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, bool coop, size_t smem, int *out);
 size_t small_scratch_words(int64_t ctas, int64_t nmax);  // level offsets and exponents
-// coop: long rows are taken by whole warps; pays when some row is longer than
-// SMALL_COOP_DEG (1,370 vertices, hubs of 90: 0.29 to 0.26 ms; a batch of small
-// graphs with rows up to 60: 0.50 to 0.62)
-constexpr int SMALL_COOP_DEG = 64;
+// coop: long rows are taken by whole warps.  Pays where next to all of the work
+// is in pieces of more than SMALL_COOP_N vertices with rows above SMALL_COOP_DEG,
+// which run a source or two at once (1,370 vertices, hubs of 94: 0.29 to 0.26 ms);
+// with more sources the lanes have work, and it costs (2,000 graphs of up to 600
+// vertices, hubs of 84: 7.1 to 8.0; 8 of up to 1,200: 0.164 to 0.186)
+constexpr int SMALL_COOP_DEG = 64, SMALL_COOP_N = 800;
 int launch_small(Ctx &ctx, bool fp32, bool coop, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
                  const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
                  int *err, unsigned long long *dag);

@@ -1,0 +1,34 @@
+"""Shared-memory pieces with hubs: long rows by whole warps only where a launch
+is all large pieces (needs a CUDA device)."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def small_ms(gpu, call):
+    t = []
+    for _ in range(6):
+        call()
+        t.append(gpu.last_stats()["ms_bcreach_small"])
+    return min(t[1:])
+
+
+def test_a_hub_does_not_slow_its_batch(gpu):
+    """The same graphs with and without one whose hub has 70 entries: the
+    launch is the same but for that graph.  (With all rows by warps 12 to 23 %
+    more on batches of such graphs; 6 % is for the timer and the graph.)"""
+    g, off = gg.batch(500, n_max=300)
+    assert int(g.degrees().max()) <= 64
+    hub = gg.from_edges(120, np.concatenate([np.stack([np.zeros(70, int), np.arange(1, 71)], 1),
+                                             np.stack([np.arange(1, 119), np.arange(2, 120)], 1)]))
+    both = gg.disjoint_union(g, hub)
+    off2 = np.append(off, both.n)
+    base = small_ms(gpu, lambda: gpu.bc_shattered_batch(off, g.row_ptr, g.col))
+    with_hub = small_ms(gpu, lambda: gpu.bc_shattered_batch(off2, both.row_ptr, both.col))
+    got = gpu.bc_shattered_batch(off2, both.row_ptr, both.col)
+    assert float(np.abs(got[off[-1]:] - oracle.bc(hub)).max()) <= 1e-12 * float(oracle.bc(hub).max())
+    assert with_hub <= 1.06 * base
