@@ -476,7 +476,10 @@ static int launch_large_t(Ctx &ctx, int grid, const LargeSrc *work, int64_t nwor
 
 // The small-path work splits the autotuner tries: most sources a CTA runs
 // at once, and the shared-memory budget per CTA (100 KB: 2 CTAs per SM,
-// 72 KB: 3, 54 KB: 4).  The default is the first.
+// 72 KB: 3, 54 KB: 4).  Without it a CTA runs up to 16 with 54 KB (SMALL_BUDGET),
+// which is not among them and the fastest on all that was measured: 5.04 ms on
+// the articulation-vertex workload (these 7.2, 5.7, 5.2, 7.2), 0.52 on 500 graphs of
+// up to 300 vertices (0.71, 0.71, 0.60, 0.78).
 struct Split {
   int ng_cap;
   size_t budget;
@@ -501,9 +504,11 @@ static void remember_split(long long key, int choice) {
 
 // Besides the small-path work split, the autotuner picks, by timing each
 // candidate once per shape bucket and caching the fastest:
-//  * the small/large threshold: the shared memory a piece may need for one
-//    source to take the small path (SMALL_LIMITS); pieces above it take the
-//    large-piece path.  Timed over the pieces that fit the largest limit.
+//  * the small/large threshold: the fixed rule (SMALL_SMEM, and numerous
+//    shallow pieces of many vertices to the pull kernel: MID_SOURCES), or the
+//    shared memory a piece may need for one source to take the small path
+//    (SMALL_LIMITS); pieces above it take the large-piece path.  Timed over the
+//    pieces that fit the largest limit.
 //  * the kernel of each large piece: the pull kernel (where the
 //    piece's depth allows it), 32-source batches (where its depth is below
 //    4 x MS_DEPTH_LIMIT: their cost grows with the levels of a batch), or
@@ -511,7 +516,7 @@ static void remember_split(long long key, int choice) {
 //    fills the GPU for that kernel.
 // Every candidate runs into a scratch accumulator; the call then runs with
 // the choice.  Without the autotuner the fixed limits above decide.
-static const size_t SMALL_LIMITS[] = {SMALL_SMEM, 64 * 1024, 40 * 1024};
+static const size_t SMALL_LIMITS[] = {0, SMALL_SMEM, 64 * 1024, 40 * 1024};  // 0: the fixed rule
 static std::map<long long, int> g_tune_limit, g_tune_large;
 
 static int tuned_in(std::map<long long, int> &m, long long key) {
@@ -672,6 +677,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
                     !po.force_large && !po.per_source_large;
   // the small/large threshold
   size_t small_limit = po.small_limit ? po.small_limit : SMALL_SMEM;
+  bool mid_rule = !po.small_limit && lp_mode == LARGE_PATH_AUTO && !dbg && !po.per_source_large;
   if (tune && !po.small_limit) {
     std::vector<CompDesc> elig;  // pieces that fit the largest limit
     double cost = 0.0, band = 0.0;
@@ -695,6 +701,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
           p2.small_limit = SMALL_LIMITS[k];
           double ms = 0.0;
           BCS_TRY(time_candidate(ctx, elig, in, p2, &ms));
+          if (k == 0) BCS_TRY(time_candidate(ctx, elig, in, p2, &ms));  // the first got the memory pool going
           if (std::getenv("BCS_TRACE"))
             std::fprintf(stderr, "[bcs] tune small/large threshold %zu B: %.3f ms\n", SMALL_LIMITS[k], ms);
           if (ms < best) {
@@ -704,7 +711,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         }
         remember_in(g_tune_limit, key, ch);
       }
-      small_limit = SMALL_LIMITS[ch - 1];
+      mid_rule = SMALL_LIMITS[ch - 1] == 0;
+      small_limit = mid_rule ? SMALL_SMEM : SMALL_LIMITS[ch - 1];
       ctx.stats.tuned |= 1;
     }
   }
@@ -715,7 +723,6 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   int64_t nmax_large = 0, nmax_small = 0;
   double work_se = 0.0, work_sv = 0.0, total_small_cost = 0.0;
   std::vector<int32_t> mids;  // pieces of the small path that the pull kernel may take instead
-  const bool mid_rule = !tune && !po.small_limit && lp_mode == LARGE_PATH_AUTO && !dbg && !po.per_source_large;
   auto small_takes_sources = [&](const CompDesc &c, int g) {
     return small_takes(c.n, c.nnz, g) && small_smem_bytes(c.n, c.nnz, g, R, I) <= SMALL_BUDGET;
   };
