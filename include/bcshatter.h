@@ -193,6 +193,8 @@ typedef struct bcs_stats {
   double ms_mapback;       /* bc accumulation and map back */
   double ms_download;      /* device -> host copy of bc */
   double ms_side;          /* side-vertex marking and the reduced pieces */
+  int64_t n_deep_sources;  /* sources run with a thread per (source, vertex) pair
+                              (deep pieces of small degree) */
 } bcs_stats;
 
 /*

@@ -41,7 +41,7 @@ class Stats(ctypes.Structure):
         "n_wide_batches", "n_rounds", "small_limit", "tuned")] + [(name, c_dbl) for name in (
         "work_nm", "work_sources_entries", "work_sources_vertices", "ms_total", "ms_upload", "ms_validate", "ms_cc", "ms_peel",
         "ms_blocks", "ms_ident", "ms_plan", "ms_bcreach_small", "ms_bcreach_large", "ms_mapback",
-        "ms_download", "ms_side")]
+        "ms_download", "ms_side")] + [("n_deep_sources", c_i64)]
 
 
 class ComponentsView(ctypes.Structure):

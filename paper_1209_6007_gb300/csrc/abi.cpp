@@ -819,6 +819,6 @@ __attribute__((visibility("default"))) int bcs_last_stats(bcs_stats *out) {
 
 __attribute__((visibility("default"))) const char *bcs_last_error(void) { return t_err.c_str(); }
 
-__attribute__((visibility("default"))) int bcs_version(void) { return 100; }
+__attribute__((visibility("default"))) int bcs_version(void) { return 101; }
 
 }  // extern "C"

@@ -1051,6 +1051,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   for (int32_t ci : ps_tuned) ctx.stats.n_large_sources += nsrc_of(comps[ci]);
   for (const PullJob &j : pull) ctx.stats.n_large_sources += j.nsrc;
   for (const DeepJob &j : deep) ctx.stats.n_large_sources += j.nsrc;
+  for (const DeepJob &j : deep) ctx.stats.n_deep_sources += j.nsrc;
   ctx.stats.work_sources_entries = work_se;
   ctx.stats.work_sources_vertices = work_sv;
   if (small.empty() && large.empty() && pull.empty() && deep.empty() && ms_tuned.empty() && ps_tuned.empty()) return BCS_OK;
