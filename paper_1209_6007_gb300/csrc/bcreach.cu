@@ -857,17 +857,21 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       const bool tune_this = tune && c.src_off < 0 && nsrc_of(c) >= 24LL * ctx.num_sms;
       int choice = LARGE_PATH_AUTO;
       if (tune_this) {
-        const long long key = ((long long)(R * 2 + I) << 40) | (bits_of(c.n) << 24) |
+        // what the piece may run on and the precision are part of its shape: a
+        // choice made without them may not be open here, or not the fastest
+        const long long key = ((long long)(((F * 2 + ok) * 2 + deep_ok) * 4 + R * 2 + I) << 40) | (bits_of(c.n) << 24) |
                               (bits_of((double)c.nnz / c.n) << 16) | bits_of(depth);
         choice = tuned_in(g_tune_large, key);
         if (!choice) {
           BCS_TRY(tune_large_piece(ctx, c, in, po, ok, deep_ok, depth, ord, &choice));
           remember_in(g_tune_large, key, choice);
         }
-        ctx.stats.tuned |= 1ll << choice;
         if (choice == LARGE_PATH_BATCHED) ms_tuned.push_back(ci);
         if (choice == LARGE_PATH_PER_SOURCE) ps_tuned.push_back(ci);
-        if (choice != LARGE_PATH_WIDE && choice != LARGE_PATH_DEEP) continue;
+        if (choice != LARGE_PATH_WIDE && choice != LARGE_PATH_DEEP) {
+          ctx.stats.tuned |= 1ll << choice;
+          continue;
+        }
       }
       bool take = ok && lp_mode != LARGE_PATH_DEEP && choice != LARGE_PATH_DEEP && (!apart || force_wide || choice == LARGE_PATH_WIDE);
       if (choice == LARGE_PATH_AUTO && !force_wide && !force_mid) take = take && depth <= PULL_MAX_ECC;
@@ -876,10 +880,11 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
         BCS_TRY(device_free_bytes(&free_b));
         take = pull_width(c.n, c.nnz, bound, free_b) > 0;
       }
-      if (!take && !deep_ok) {
+      if (!take && !deep_ok) {  // (a chosen kernel's memory may be gone)
         rest.push_back(ci);
         continue;
       }
+      if (tune_this) ctx.stats.tuned |= 1ll << (take ? LARGE_PATH_WIDE : LARGE_PATH_DEEP);
       if (po.sources) {  // the caller's sources
         std::vector<int32_t> h(po.nsources);
         for (int64_t i = 0; i < po.nsources; i++) h[i] = (int32_t)po.sources[i];
