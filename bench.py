@@ -240,13 +240,17 @@ def run_reference(args):
 def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
     """Roofline of the call's dominant Bc-Reach kernel.
 
-    Large pieces (the pull kernel): HBM.  Algorithmic bytes per
-    (source, CSR entry) of a piece, with S sources sharing one adjacency
-    read: 8/S (the row) + 2/8 (level bits) + f_DAG * 28 (path count written
-    and read, coefficient, weights, per shortest-path DAG edge) + (n / 2m) *
-    32 (per-vertex state written and read once); f_DAG is the DAG edges the
-    call counted over its (source, entry) pairs.  Per launch: the sum over
-    processed sources of these bytes, over the kernel's CUDA-event time.
+    Large pieces: HBM.  For the pull kernel the DRAM bytes of a whole launch
+    (ncu, committed summary of the same kernel sources), per batch of 64
+    sources, times this call's batches, over the kernel's CUDA-event time.
+    Without such a record, and for the other kernels, a model in its place
+    (`basis` says which): the bytes of a frontier search per (source, CSR
+    entry) of a piece, with S sources sharing one adjacency read: 8/S (the
+    row) + 2/8 (level bits) + f_DAG * 28 (path count written and read,
+    coefficient, weights, per shortest-path DAG edge) + (n / 2m) * 32
+    (per-vertex state written and read once); f_DAG is the DAG edges the call
+    counted over its (source, entry) pairs.  The pull kernel moves less: it
+    shares a row among 256 sources and most of its values take four bytes.
 
     Shared-memory pieces only: the issue rate, the kernel's warp
     instructions per launch (ncu, committed summary of the same command)
@@ -258,19 +262,25 @@ def roofline(st: dict, clk: dict, peaks: dict, n_sm: int) -> dict:
     wse, wsv = float(st["work_sources_entries"]), float(st["work_sources_vertices"])
     sm_mhz = clk.get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))
     if st["ms_bcreach_large"] > st["ms_bcreach_small"]:
-        # sources sharing one batch of the pull kernel (32 or 64)
-        S = 64 if st["n_wide_batches"] and st["n_large_sources"] > 32 * st["n_wide_batches"] else 32
+        ns, deep = int(st["n_large_sources"]), int(st.get("n_deep_sources", 0))
+        pulled = int(st["n_wide_batches"]) > 0 and 2 * deep < ns
+        # sources sharing one adjacency read
+        S = 64 if pulled and ns > 32 * st["n_wide_batches"] else 1 if 2 * deep >= ns > 0 else 32
         f_dag = dag / wse if wse else 0.0
         by = wse * (8.0 / S + 2.0 / 8.0 + f_dag * 28.0) + wsv * 32.0
         ms = st["ms_bcreach_large"]
         peak = float(peaks.get("hbm_gbs", 6800.0))
-        achieved = by / (ms / 1e3) / 1e9
         rec = measured_traffic("wide")
-        traffic = rec["dram_bytes_per_batch"] * st["n_wide_batches"] if rec and st["n_wide_batches"] else None
+        traffic = rec["dram_bytes_per_batch"] * st["n_wide_batches"] if rec and pulled else None
+        achieved = (traffic or by) / (ms / 1e3) / 1e9
+        kernel = ("k_bcreach_pull (whole GPU on one BFS level of many sources)" if pulled else
+                  "k_bcreach_deep (a thread per (source, vertex) pair)" if 2 * deep >= ns > 0 else
+                  "k_bcreach_ms (32 sources per CTA)" if st.get("n_ms_batches") else "k_bcreach_large (one source per CTA)")
         return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": "k_bcreach_pull (whole GPU on one BFS level of many sources)",
+                "basis": "measured DRAM bytes" if traffic else "model of the bytes a frontier search has to move",
+                "traffic": traffic, "kernel": kernel,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
-                "work": {"bytes": by, "f_dag": f_dag, "sources_x_entries": wse, "sources_x_vertices": wsv,
+                "work": {"model_bytes": by, "f_dag": f_dag, "sources_x_entries": wse, "sources_x_vertices": wsv,
                          "batches": int(st["n_wide_batches"]), "ms": ms,
                          "traffic_scaled_from": "ncu DRAM bytes of a full launch per batch (profiles/bcreach_pull_twins.json) "
                                                 "x this call's batches" if traffic else None}}
@@ -369,13 +379,15 @@ def run_ours(args):
 
     # the other dependency precision on the same step, and its difference
     # (shared-memory workloads: one untimed call first, which runs that
-    # precision's autotuner; a large piece's call is too long to repeat)
-    if float(st["ms_bcreach_large"]) < 1000.0:
+    # precision's autotuner; a large piece's call is too long to repeat, and
+    # takes the fixed rules)
+    short = float(st["ms_bcreach_large"]) < 1000.0
+    if short:
         bcs.bc_shattered(rp, col, delta_fp32=not fp32, autotune=True)
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
-    b_other = bcs.bc_shattered(rp, col, delta_fp32=not fp32, autotune=True)
+    b_other = bcs.bc_shattered(rp, col, delta_fp32=not fp32, autotune=short)
     ev1.record(stream)
     ev1.synchronize()
     t_other = ev0.elapsed_time(ev1) / 1e3
