@@ -56,7 +56,7 @@ constexpr int SMALL_LEVELS = 64;  // level offsets kept in shared memory, the re
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// shared memory of a piece's rows (padded to fours), weights and codes, and of its pairs with G sources
+// shared memory of a piece's rows, weights and codes, and of its pairs with G sources
 __host__ __device__ inline size_t small_piece_bytes(int64_t n, int64_t nnz, bool reach, bool ident) {
   return align16((size_t)(n + 1) * 2) + align16((size_t)(nnz + 3) * 2) + (reach ? align16((size_t)n * 8) : 0) +
          (ident ? align16((size_t)n * 4) : 0) + align16((size_t)n * 4);
@@ -65,7 +65,7 @@ size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident) {
   const size_t p = (size_t)n * G;
   return small_piece_bytes(n, nnz, reach, ident) + align16(p * 8) * 2 + align16(p * 4) + align16(p * 2);
 }
-// 16-bit columns, row offsets (in fours) and queue places
+// 16-bit columns, row offsets and queue places
 bool small_takes(int64_t n, int64_t nnz, int G) {
   int gs = 0;
   while ((1 << gs) < G) gs++;
@@ -77,10 +77,13 @@ int small_max_sources() { return SMALL_MAX_G; }
 // entries, the warp takes those together: a hub's row taken by one lane holds
 // up the level.  Where no row is long the ballots and the registers cost more
 // than they give (articulation-vertex workload: 5.0 ms without, 6.2 with).
+// FP32: four CTAs per SM (by itself it takes 56 registers, three: a ring of 500,
+// one source per CTA, 0.62 ms in two rounds, 0.39 in one; 5.42 and 5.48 ms on the
+// articulation-vertex workload).
 // GLOBAL (a piece above shared memory, G = 1): codes and queue in shared
 // memory, the counts and sums in global memory (`state`), the rows the caller's.
 template <bool REACH, bool IDENT, bool FP32, bool COOP, bool GLOBAL>
-__global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, GLOBAL ? 2 : COOP ? 4 : 0) k_bcreach_small(
+__global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, GLOBAL ? 2 : COOP || FP32 ? 4 : 0) k_bcreach_small(
     const SmallItem *__restrict__ items, int nitems, int *item_counter, const CompDesc *__restrict__ comps,
     const int64_t *__restrict__ g_row, const int32_t *__restrict__ g_col, const int32_t *__restrict__ g_reach,
     const int32_t *__restrict__ g_ident, const double *__restrict__ g_init, const int64_t *__restrict__ srcs,
