@@ -72,25 +72,26 @@ constexpr int DEEP_MIN_ECC = 40;
 constexpr int MID_SOURCES = 2;
 constexpr int MID_PIECE_ECC = 8;
 constexpr int64_t MID_MIN_ROWS = 1 << 15;
-// Source lists of at most one round of CTAs (three per SM).  All kernels then
-// wait for the latency of their levels, one source per CTA for the fewest, and
-// the search by one CTA that orders the sources for the others takes about as
+// Source lists of at most FEW_ROUNDS rounds of CTAs (three per SM).  All kernels
+// then wait for the latency of their levels, one source per CTA for the fewest,
+// and the search by one CTA that orders the sources for the others takes about as
 // long as one source.
-// Graphs of up to FEW_MAX_N vertices whose entries and longest row take one
-// source in a CTA of its own less than FEW_US: no search (15,200 vertices in 38
+// Graphs of up to FEW_MAX_N vertices whose entries and longest row take these
+// rounds less than FEW_US: no search (15,200 vertices in 38
 // layers, 32 sources, 0.93 ms, 2.4 on the pull kernel; a ring of 6,000, 1 source,
 // 9.7 ms, 18 on the deep one).  Above it the pull kernel is sooner (20,000
 // vertices of a power law, 300 sources, 1.4 ms and 2.4), if the graph is not
 // deep.  Of mean degree FEW_MEAN_DEG or less it may be a road, where more than
 // FEW_ROAD_SOURCES are worth the order (a square grid of 10,000: 400 sources
-// 1.8 ms on the deep kernel, 2.8; 1 source 1.5 and 1.1).  Above FEW_DENSE_DEG the
+// 1.8 ms on the deep kernel, 2.8; 1 source 1.5 and 1.1; a power-law graph of 3,400
+// with pendants, 100 sources, 0.99 on the pull kernel, 0.64).  Above FEW_DENSE_DEG the
 // pull kernel cuts the rows, and is sooner (800 vertices of degree 100 in a few
 // levels, 1 source 0.48 ms and 0.58; 1,600 in 16 levels 0.86 and 1.02).
 constexpr int32_t FEW_MAX_N = 16384;
 constexpr double FEW_US = 470.0;
-constexpr int64_t FEW_MEAN_DEG = 6, FEW_ROAD_SOURCES = 32, FEW_DENSE_DEG = 64;
+constexpr int64_t FEW_ROUNDS = 2, FEW_MEAN_DEG = 6, FEW_ROAD_SOURCES = 128, FEW_DENSE_DEG = 64;
 static double one_source_us(const CompDesc &c) { return 1.8e-3 * (double)c.nnz + 1.2 * c.maxdeg; }
-// The search is given up after these levels: of any width where a graph is small
+// With one round the search is given up after these levels: of any width where a graph is small
 // and no road, else when they hold few vertices (20,000 in a path, 30 sources: 54
 // ms so, 105 with the order).  Where it ends in a small component of such a graph
 // (and of at most FEW_APART_MAX_N vertices: a CTA's state is cleared for it) the
@@ -789,12 +790,14 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     int64_t total = 0;
     PieceBfsEnd end;
     bool no_search = false;
-    const bool few = po.sources && po.nsources <= 3 * (int64_t)ctx.num_sms && lp_mode == LARGE_PATH_AUTO;
-    if (few) {
+    bool cheap = false;  // one source per CTA is
+    if (po.sources && lp_mode == LARGE_PATH_AUTO) {
       const CompDesc &c = comps[0];
+      const int64_t wave = 3 * (int64_t)ctx.num_sms, rounds = (po.nsources + wave - 1) / wave;
       const bool road = c.nnz <= FEW_MEAN_DEG * c.n, small_n = c.n < FEW_MAX_N && c.nnz <= FEW_DENSE_DEG * c.n;
-      no_search = small_n && one_source_us(c) < FEW_US && (po.nsources <= FEW_ROAD_SOURCES || !road);
-      end = small_n && !road ? FEW_END : FEW_NARROW_END;
+      cheap = rounds <= FEW_ROUNDS && rounds * one_source_us(c) < FEW_US;
+      no_search = small_n && cheap && (po.nsources <= FEW_ROAD_SOURCES || !road);
+      if (rounds <= 1) end = small_n && !road ? FEW_END : FEW_NARROW_END;
     }
     for (int32_t ci : large) {
       const CompDesc &c = comps[ci];
@@ -829,7 +832,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       int depth = cta_depth[k];
       int64_t reached = cta_reached[k];
       bool apart = false;  // a graph of many small components
-      if (reached == -2 || (few && reached >= 0 && reached < c.n / 4 && c.n <= FEW_APART_MAX_N && one_source_us(c) < FEW_US)) {
+      if (reached == -2 || (cheap && reached >= 0 && reached < c.n / 4 && c.n <= FEW_APART_MAX_N)) {
         rest.push_back(ci);
         continue;
       }
