@@ -962,7 +962,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       smem = std::max(smem, small_smem_bytes(c.n, c.nnz, ng, R, I));
     }
     int per_sm = 1;
-    BCS_TRY(small_ctas_per_sm(ctx, R, I, F, small_coop, smem, &per_sm));
+    BCS_TRY(small_ctas_per_sm(ctx, R, I, F, small_variant(ctx, F, small_coop, small_sources, smem), smem, &per_sm));
     grid = ctx.num_sms * per_sm;
     const double target = total_small_cost / (double)((int64_t)grid * 8) + 1.0;
     for (size_t k = 0; k < small.size(); k++) {
@@ -1091,7 +1091,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
       BCS_CUDA(cudaMemsetAsync(d_err.p + 1, 0, sizeof(int), ctx.stream));
       BcInput tin = in;
       tin.bcp = target;
-      return launch_small(ctx, F, small_coop, grid, smem, d_items.p, (int)its.size(), d_err.p + 1, d_comps.p, tin,
+      return launch_small(ctx, F, small_variant(ctx, F, small_coop, small_sources, smem), grid, smem, d_items.p, (int)its.size(), d_err.p + 1, d_comps.p, tin,
                           po.sources ? d_srcs.p : po.srcmap, lvl.p, nmax_small, d_err.p, d_dag.p);
     };
     tr.mark("alloc");

@@ -360,7 +360,11 @@ struct SmallItem {
 size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident);
 bool small_takes(int64_t n, int64_t nnz, int G);
 int small_max_sources();
-int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, bool coop, size_t smem, int *out);
+// the kernel's variants (small.cu) and the one for a launch: `coop` below,
+// sources in all, shared memory of a CTA
+enum { SMALL_PLAIN = 0, SMALL_COOP = 1, SMALL_FOUR = 2 };
+int small_variant(const Ctx &ctx, bool fp32, bool coop, int64_t sources, size_t smem);
+int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, int variant, size_t smem, int *out);
 size_t small_scratch_words(int64_t ctas, int64_t nmax);  // level offsets and exponents
 // coop: long rows are taken by whole warps.  Pays where next to all of the work
 // is in pieces of more than SMALL_COOP_N vertices with rows above SMALL_COOP_DEG,
@@ -368,7 +372,7 @@ size_t small_scratch_words(int64_t ctas, int64_t nmax);  // level offsets and ex
 // with more sources the lanes have work, and it costs (2,000 graphs of up to 600
 // vertices, hubs of 84: 7.1 to 8.0; 8 of up to 1,200: 0.164 to 0.186)
 constexpr int SMALL_COOP_DEG = 64, SMALL_COOP_N = 800;
-int launch_small(Ctx &ctx, bool fp32, bool coop, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
+int launch_small(Ctx &ctx, bool fp32, int variant, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
                  const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
                  int *err, unsigned long long *dag);
 // device address of the reciprocals of the integers below RECIP_TABLE

@@ -73,22 +73,24 @@ bool small_takes(int64_t n, int64_t nnz, int G) {
 }
 int small_max_sources() { return SMALL_MAX_G; }
 
-// COOP: where a warp's pairs have at most SMALL_LONGS rows of more than 32
+// SMALL_COOP: where a warp's pairs have at most SMALL_LONGS rows of more than 32
 // entries, the warp takes those together: a hub's row taken by one lane holds
 // up the level.  Where no row is long the ballots and the registers cost more
 // than they give (articulation-vertex workload: 5.0 ms without, 6.2 with).
-// FP32: four CTAs per SM (by itself it takes 56 registers, three: a ring of 500,
-// one source per CTA, 0.62 ms in two rounds, 0.39 in one; 5.42 and 5.48 ms on the
-// articulation-vertex workload).
+// SMALL_FOUR: four CTAs per SM.  With FP32 dependencies it takes 56 registers by
+// itself, three CTAs, which is the faster where there is work for many rounds
+// (articulation-vertex workload 5.42 ms, 5.48 with four), but not for one or two
+// (a ring of 500, one source per CTA: 0.62 and 0.39).
 // GLOBAL (a piece above shared memory, G = 1): codes and queue in shared
 // memory, the counts and sums in global memory (`state`), the rows the caller's.
-template <bool REACH, bool IDENT, bool FP32, bool COOP, bool GLOBAL>
-__global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, GLOBAL ? 2 : COOP || FP32 ? 4 : 0) k_bcreach_small(
+template <bool REACH, bool IDENT, bool FP32, int VARIANT, bool GLOBAL>
+__global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, GLOBAL ? 2 : VARIANT != SMALL_PLAIN ? 4 : 0) k_bcreach_small(
     const SmallItem *__restrict__ items, int nitems, int *item_counter, const CompDesc *__restrict__ comps,
     const int64_t *__restrict__ g_row, const int32_t *__restrict__ g_col, const int32_t *__restrict__ g_reach,
     const int32_t *__restrict__ g_ident, const double *__restrict__ g_init, const int64_t *__restrict__ srcs,
     const double *__restrict__ recip, double *bcp, size_t bcp_stride, int32_t *lvl_scratch, int lvl_stride, int lvl_G,
     unsigned char *state, size_t state_stride, int *err, unsigned long long *dag_total) {
+  constexpr bool COOP = VARIANT == SMALL_COOP;
   constexpr int NT = GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_max[SMALL_MAX_G];  // largest count of each source on the level, as bits
@@ -469,22 +471,22 @@ __global__ void __launch_bounds__(GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS,
 static std::mutex g_small_mu;
 static std::map<long long, int> g_small_occ;  // (variant, device, smem) -> CTAs per SM
 
-template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
+template <bool R, bool I, bool F, int V, bool GLOBAL>
 static int small_prepare(int device) {
   static std::mutex mu;
   static std::set<int> done;
   std::lock_guard<std::mutex> lk(mu);
   if (!done.count(device)) {
-    BCS_CUDA(cudaFuncSetAttribute(k_bcreach_small<R, I, F, COOP, GLOBAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    BCS_CUDA(cudaFuncSetAttribute(k_bcreach_small<R, I, F, V, GLOBAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)SMALL_SMEM));
     done.insert(device);
   }
   return BCS_OK;
 }
 
-template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
+template <bool R, bool I, bool F, int V, bool GLOBAL>
 static int small_ctas_c(int device, size_t smem, int *out) {
-  const long long key = ((long long)(R * 16 + I * 8 + F * 4 + COOP * 2 + GLOBAL) << 48) | ((long long)device << 32) |
+  const long long key = ((long long)(R * 32 + I * 16 + F * 8 + V * 2 + GLOBAL) << 48) | ((long long)device << 32) |
                         (long long)smem;
   {
     std::lock_guard<std::mutex> lk(g_small_mu);
@@ -494,8 +496,8 @@ static int small_ctas_c(int device, size_t smem, int *out) {
       return BCS_OK;
     }
   }
-  BCS_TRY((small_prepare<R, I, F, COOP, GLOBAL>(device)));
-  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bcreach_small<R, I, F, COOP, GLOBAL>,
+  BCS_TRY((small_prepare<R, I, F, V, GLOBAL>(device)));
+  BCS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bcreach_small<R, I, F, V, GLOBAL>,
                                                          GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, smem));
   if (*out < 1) *out = 1;
   std::lock_guard<std::mutex> lk(g_small_mu);
@@ -504,13 +506,21 @@ static int small_ctas_c(int device, size_t smem, int *out) {
 }
 
 template <bool R, bool I, bool F>
-static int small_ctas_t(int device, bool coop, size_t smem, int *out) {
-  return coop ? small_ctas_c<R, I, F, true, false>(device, smem, out)
-              : small_ctas_c<R, I, F, false, false>(device, smem, out);
+static int small_ctas_t(int device, int variant, size_t smem, int *out) {
+  if (variant == SMALL_COOP) return small_ctas_c<R, I, F, SMALL_COOP, false>(device, smem, out);
+  if constexpr (F)
+    if (variant == SMALL_FOUR) return small_ctas_c<R, I, F, SMALL_FOUR, false>(device, smem, out);
+  return small_ctas_c<R, I, F, SMALL_PLAIN, false>(device, smem, out);
 }
 
-int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, bool coop, size_t smem, int *out) {
-  return BCS_DISPATCH3(small_ctas_t, R, I, F, ctx.device, coop, smem, out);
+int small_ctas_per_sm(Ctx &ctx, bool R, bool I, bool F, int variant, size_t smem, int *out) {
+  return BCS_DISPATCH3(small_ctas_t, R, I, F, ctx.device, variant, smem, out);
+}
+
+int small_variant(const Ctx &ctx, bool fp32, bool coop, int64_t sources, size_t smem) {
+  if (coop) return SMALL_COOP;
+  const bool rounds = sources > 3 * (int64_t)ctx.num_sms && sources <= 16 * (int64_t)ctx.num_sms;
+  return fp32 && rounds && smem <= SMALL_BUDGET ? SMALL_FOUR : SMALL_PLAIN;
 }
 
 size_t small_scratch_words(int64_t ctas, int64_t nmax) { return (size_t)ctas * (SMALL_MAX_G + 1) * (nmax + 2); }
@@ -530,12 +540,12 @@ struct SmallLaunch {
   unsigned long long *dag;
 };
 
-template <bool R, bool I, bool F, bool COOP, bool GLOBAL>
+template <bool R, bool I, bool F, int V, bool GLOBAL>
 static int small_launch_c(Ctx &ctx, int grid, size_t smem, const BcInput &in, const SmallLaunch &a) {
-  BCS_TRY((small_prepare<R, I, F, COOP, GLOBAL>(ctx.device)));
+  BCS_TRY((small_prepare<R, I, F, V, GLOBAL>(ctx.device)));
   const double *recip = nullptr;
   BCS_TRY(recip_table(ctx, &recip));
-  k_bcreach_small<R, I, F, COOP, GLOBAL><<<grid, GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, smem, ctx.stream>>>(
+  k_bcreach_small<R, I, F, V, GLOBAL><<<grid, GLOBAL ? SMALL_GLOBAL_THREADS : SMALL_THREADS, smem, ctx.stream>>>(
       a.items, a.nitems, a.counter, a.comps, in.row, in.col, in.reach, in.ident, in.init, a.srcs, recip,
       in.bcp, a.bcp_stride, a.lvl, a.lvl_stride, a.lvl_G, a.state, a.state_stride, a.err, a.dag);
   ctx.launches++;
@@ -544,17 +554,19 @@ static int small_launch_c(Ctx &ctx, int grid, size_t smem, const BcInput &in, co
 }
 
 template <bool R, bool I, bool F>
-static int small_launch_t(Ctx &ctx, bool coop, int grid, size_t smem, const BcInput &in, const SmallLaunch &a) {
-  return coop ? small_launch_c<R, I, F, true, false>(ctx, grid, smem, in, a)
-              : small_launch_c<R, I, F, false, false>(ctx, grid, smem, in, a);
+static int small_launch_t(Ctx &ctx, int variant, int grid, size_t smem, const BcInput &in, const SmallLaunch &a) {
+  if (variant == SMALL_COOP) return small_launch_c<R, I, F, SMALL_COOP, false>(ctx, grid, smem, in, a);
+  if constexpr (F)
+    if (variant == SMALL_FOUR) return small_launch_c<R, I, F, SMALL_FOUR, false>(ctx, grid, smem, in, a);
+  return small_launch_c<R, I, F, SMALL_PLAIN, false>(ctx, grid, smem, in, a);
 }
 
-int launch_small(Ctx &ctx, bool fp32, bool coop, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
+int launch_small(Ctx &ctx, bool fp32, int variant, int grid, size_t smem, const SmallItem *items, int nitems, int *counter,
                  const CompDesc *comps, const BcInput &in, const int64_t *srcs, int32_t *scratch, int64_t nmax,
                  int *err, unsigned long long *dag) {
   const bool R = in.reach != nullptr || in.init != nullptr, I = in.ident != nullptr;
   const SmallLaunch a{items, nitems, counter, comps, srcs, 0, scratch, (int)nmax + 2, SMALL_MAX_G, nullptr, 0, err, dag};
-  return BCS_DISPATCH3(small_launch_t, R, I, fp32, ctx, coop, grid, smem, in, a);
+  return BCS_DISPATCH3(small_launch_t, R, I, fp32, ctx, variant, grid, smem, in, a);
 }
 
 // ------------------------------------- plain Brandes in a fixed scratch
@@ -594,7 +606,7 @@ static int fixed_launch(Ctx &ctx, const CompDesc &desc, size_t smem, int G, size
   const int64_t n = desc.n;
   const size_t head = FIXED_HEAD + fixed_up256((size_t)n * sizeof(SmallItem));
   int per_sm = 1;
-  BCS_TRY((small_ctas_c<false, false, F, true, GLOBAL>(ctx.device, smem, &per_sm)));
+  BCS_TRY((small_ctas_c<false, false, F, SMALL_COOP, GLOBAL>(ctx.device, smem, &per_sm)));
   const size_t part_bytes = fixed_up256((size_t)FIXED_COPIES * n * 8);
   const int64_t fit = (int64_t)((bytes - head - part_bytes) / (lvl_bytes + state_bytes));
   const int64_t ctas = std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx.num_sms * per_sm, fit));
@@ -620,7 +632,7 @@ static int fixed_launch(Ctx &ctx, const CompDesc &desc, size_t smem, int G, size
                                                                 (SmallItem *)(scratch + FIXED_HEAD), a.nitems, per, G);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
-  BCS_TRY((small_launch_c<false, false, F, true, GLOBAL>(ctx, grid, smem, in, a)));
+  BCS_TRY((small_launch_c<false, false, F, SMALL_COOP, GLOBAL>(ctx, grid, smem, in, a)));
   k_fixed_add<<<(int)((n + 63) / 64), 64, 0, ctx.stream>>>((int)n, part, bc);
   ctx.launches++;
   BCS_CUDA(cudaGetLastError());
