@@ -123,9 +123,14 @@ __global__ void k_bfs_init(int64_t n, const uint8_t *__restrict__ alive, const i
 
 // Rows of more than LONG_ROW entries are walked by the whole warp: one thread
 // on a hub's row holds up the launch (a power-law graph of 194,000 vertices: low
-// and high, unions and rows 6.0 ms with a thread each, 2.6 so).  WARP_STRIDE: a grid-stride loop that whole
-// warps run through together (i may be past n).
+// and high, unions and rows 6.0 ms with a thread each, 2.6 so).  The copies' rows
+// are written entry by entry in order, so there a warp takes only rows of twice
+// the mean and more: in a dense graph all are alike, and its 32 one after
+// the other (200 vertices, all joined: rows 0.10 ms, 0.27 with a warp each).
+// WARP_STRIDE: a grid-stride loop that whole warps run through together (i may be
+// past n).
 constexpr int LONG_ROW = 32;
+static int long_slot_row(const DevGraph &g) { return (int)std::max<int64_t>(LONG_ROW, 2 * g.nnz / std::max<int64_t>(g.n, 1)); }
 #define WARP_STRIDE(i, n)                                                                              \
   for (int64_t i##0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll, i = i##0 + (threadIdx.x & 31); \
        i##0 < (n); i##0 += (int64_t)gridDim.x * blockDim.x, i += (int64_t)gridDim.x * blockDim.x)
@@ -472,15 +477,15 @@ __global__ void k_slot_degrees(int64_t cnt, const int32_t *__restrict__ verts, b
                                const int32_t *__restrict__ col, const uint8_t *__restrict__ alive,
                                const int32_t *__restrict__ parent, const int32_t *__restrict__ level,
                                const int32_t *__restrict__ bid, const int32_t *__restrict__ home_slot,
-                               const int32_t *__restrict__ top_slot, int64_t *sdeg) {
+                               const int32_t *__restrict__ top_slot, int64_t *sdeg, int longer) {
   WARP_STRIDE(i, cnt) {
     const bool valid = i < cnt;
     const int32_t v = valid ? verts[i] : 0;
     const int32_t hs = valid ? home_slot[v] : -1;  // most of v's entries go to its home slot: counted in a register
     int64_t nh = 0;
     const int64_t b = valid ? rp[v] : 0, e = valid ? rp[v + 1] : 0;
-    const unsigned longs = __ballot_sync(0xffffffffu, e - b > LONG_ROW);
-    if (e - b <= LONG_ROW)
+    const unsigned longs = __ballot_sync(0xffffffffu, e - b > longer);
+    if (e - b <= longer)
       for (int64_t k = b; k < e; k++) {
         const int32_t w = col[k];
         if (!alive[w]) continue;
@@ -505,14 +510,14 @@ __global__ void k_slot_fill(int64_t cnt, const int32_t *__restrict__ verts, bool
                             const int32_t *__restrict__ col, const uint8_t *__restrict__ alive,
                             const int32_t *__restrict__ parent, const int32_t *__restrict__ level,
                             const int32_t *__restrict__ bid, const int32_t *__restrict__ home_slot,
-                            const int32_t *__restrict__ top_slot, int64_t *cursor, int32_t *scol) {
+                            const int32_t *__restrict__ top_slot, int64_t *cursor, int32_t *scol, int longer) {
   const int lane = threadIdx.x & 31;
   WARP_STRIDE(i, cnt) {
     const bool valid = i < cnt;
     const int32_t v = valid ? verts[i] : 0;
     const int64_t b = valid ? rp[v] : 0, e = valid ? rp[v + 1] : 0;
-    const unsigned longs = __ballot_sync(0xffffffffu, e - b > LONG_ROW);
-    if (e - b <= LONG_ROW) {
+    const unsigned longs = __ballot_sync(0xffffffffu, e - b > longer);
+    if (e - b <= longer) {
       const int32_t hs = home_slot[v];
       int64_t hpos = valid && hs >= 0 ? cursor[hs] : 0;  // the home slot's cursor stays in a register
       for (int64_t k = b; k < e; k++) {
@@ -765,7 +770,7 @@ int device_pieces(Ctx &ctx, const DevGraph &g, const uint8_t *alive, const int32
   BCS_TRY(out->srow.alloc(S + 1, ctx.stream));
   BCS_CUDA(cudaMemsetAsync(sdeg.p, 0, (S + 1) * sizeof(int64_t), ctx.stream));
   k_slot_degrees<<<gw, B, 0, ctx.stream>>>(nverts, verts, art, g.rp, g.col, alive, parent.p, level.p, bid.p,
-                                           home_slot.p, art ? top_slot.p : nullptr, sdeg.p);
+                                           home_slot.p, art ? top_slot.p : nullptr, sdeg.p, long_slot_row(g));
   ctx.launches++;
   BCS_TRY(launch_exclusive_scan(ctx, sdeg.p, out->srow.p, S + 1, tot.p));
   BCS_CUDA(cudaMemcpyAsync(cursor.p, out->srow.p, (S + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, ctx.stream));
@@ -774,7 +779,7 @@ int device_pieces(Ctx &ctx, const DevGraph &g, const uint8_t *alive, const int32
   out->nentries = E;
   BCS_TRY(out->scol.alloc(E, ctx.stream));
   k_slot_fill<<<gw, B, 0, ctx.stream>>>(nverts, verts, art, g.rp, g.col, alive, parent.p, level.p, bid.p, home_slot.p,
-                                        art ? top_slot.p : nullptr, cursor.p, out->scol.p);
+                                        art ? top_slot.p : nullptr, cursor.p, out->scol.p, long_slot_row(g));
   ctx.launches++;
   tr.mark("rows");
   BCS_TRY(out->piece_maxdeg.alloc(nb, ctx.stream));

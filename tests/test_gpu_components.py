@@ -23,3 +23,18 @@ def test_a_long_path(gpu, seed):
         ms.append(gpu.last_stats()["ms_cc"])
         assert np.array_equal(np.sort(got), want)
     assert min(ms) < 10.0
+
+
+def test_rows_of_a_dense_graph(gpu):
+    """200 vertices, all joined: the pieces' rows are written with a thread to a
+    row, in less than twice the time of the merging stage (1.4; 2.4 with a warp to
+    a row, its 32 rows one after the other)."""
+    g = gg.complete(200)
+    blocks, ident = [], []
+    for _ in range(12):
+        got = gpu.bc_shattered(g.row_ptr, g.col, steps=gpu.STEP_D)
+        st = gpu.last_stats()
+        blocks.append(st["ms_blocks"])
+        ident.append(st["ms_ident"])
+        assert np.array_equal(got, np.zeros(200))
+    assert min(blocks) <= 2.0 * min(ident)
