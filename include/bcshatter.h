@@ -165,9 +165,10 @@ typedef struct bcs_stats {
   int64_t small_ng_cap;    /* most sources one small-path CTA ran at once */
   int64_t small_smem_budget; /* shared-memory budget per small-path CTA (bytes) */
   int64_t n_side;          /* side vertices taken out of the pieces (BCS_STEP_S) */
-  int64_t n_wide_batches;  /* batches of 64 sources run with the whole GPU on one
-                              BFS level of many of them (pieces of small BFS depth
-                              that do not fit shared memory) */
+  int64_t n_wide_batches;  /* sources run with the whole GPU on one BFS level of
+                              many of them (pieces of small BFS depth that do not
+                              fit shared memory), counted in 64s per piece; the
+                              kernel takes up to 256 together */
   int64_t n_rounds;        /* split-and-merge rounds of the preprocessing loop
                               (BCS_STEP_L) */
   int64_t small_limit;     /* shared memory (bytes) a piece may need for one source

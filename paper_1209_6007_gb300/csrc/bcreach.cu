@@ -1142,7 +1142,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   if (!pull.empty()) {
     StageTimer tm(ctx.stream);
     tm.start();
-    int per_batch = 64;
+    int per_batch = 64;  // a quarter of a slab (for tests: an eighth)
     if (const char *e = std::getenv("BCS_WIDE_SOURCES"))
       if (lp_mode != LARGE_PATH_MID) per_batch = std::atoi(e) <= 32 ? 32 : 64;
     BCS_TRY(run_pull(ctx, comps, pull, in, F, pull_order.p, d_comps.p, per_batch, d_err.p, d_dag.p));
@@ -1267,12 +1267,5 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   }
   return BCS_OK;
 }
-
-// ------------------------------------------- fixed-scratch plain Brandes
-// Plain Brandes (reach = ident = 1) over one component of n vertices on the
-// global-memory path, with every piece of device state carved out of a
-// caller-given scratch region instead of allocated.  Used by the
-// allocation-free entry point.
-
 
 }  // namespace bcs

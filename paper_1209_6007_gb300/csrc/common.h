@@ -290,7 +290,8 @@ struct BcInput {
   double *bcp = nullptr;          // accumulation target, indexed by vertex
 };
 
-// WIDE: the pull kernel; MID: the pull kernel on connected pieces of at most 65,536 vertices
+// WIDE: the pull kernel; MID: the same on connected pieces of at most 65,536
+// vertices only (all that is left of a kernel of its own)
 enum { LARGE_PATH_AUTO = 0, LARGE_PATH_WIDE = 1, LARGE_PATH_BATCHED = 2, LARGE_PATH_PER_SOURCE = 3, LARGE_PATH_MID = 4, LARGE_PATH_DEEP = 5 };
 
 struct BcPlanOpts {
@@ -333,7 +334,8 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps, const BcInput &in,
 // Bc-Reach on pieces of small BFS depth, the whole GPU on one level of many
 // sources at a time (pull.cu).  A job: a piece, its sources (local ids at
 // d_order[ord_off ..)) and a bound on their BFS depth (at most
-// pull_depth_limit()).  per_batch: 64 (or 32) sources, four of these to a slab.
+// pull_depth_limit()).  per_batch: 64 (or 32) sources, four of these to a slab
+// where its state fits.
 struct PullJob {
   int32_t ci, nsrc;
   int depth_bound;

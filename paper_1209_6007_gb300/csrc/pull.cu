@@ -46,8 +46,8 @@
 // last to finish adds them up like a list of neighbours and completes the row.
 //
 // What bounds it: the latency of the gathers and the instructions around them
-// (half of the issue slots, a fifth of HBM bandwidth), with FP64 dependencies
-// also the FP64 pipe (half busy).  256 sources to a slab: a neighbour is on a
+// (a third of the issue slots, a fifth of HBM bandwidth with FP64 dependencies
+// and a third with FP32), with FP64 dependencies also the FP64 pipe (half busy).  256 sources to a slab: a neighbour is on a
 // shortest path for 40 of 256 sources where it is for 14 of 64, so walking,
 // listing and ranking cost a third per source; waves of 2^20 rows: waves of
 // 2^18 measured 10-15 % slower (the tail of every pass).  Four CTAs per SM: at
