@@ -46,15 +46,16 @@
 // last to finish adds them up like a list of neighbours and completes the row.
 //
 // What bounds it: the latency of the gathers and the instructions around them
-// (a third of the issue slots, a fifth of HBM bandwidth with FP64 dependencies
-// and a third with FP32), with FP64 dependencies also the FP64 pipe (half busy).  256 sources to a slab: a neighbour is on a
+// (a third of the issue slots with FP64 dependencies, half with FP32; a fifth of
+// HBM bandwidth, a third at 424,000 vertices), with FP64 dependencies also the FP64
+// pipe (half busy).  256 sources to a slab: a neighbour is on a
 // shortest path for 40 of 256 sources where it is for 14 of 64, so walking,
 // listing and ranking cost a third per source; waves of 2^20 rows: waves of
 // 2^18 measured 10-15 % slower (the tail of every pass).  Four CTAs per SM: at
 // 48 registers (five) it spills and the FP64 cases lose what FP32 gains.
 // On one GB300, whole calls: 87,000 vertices, 1.15 M entries, FP32 dependencies,
-// every vertex a source 295 ms (1,340 ms with one 64-source batch on the whole
-// GPU and pushed counts); 13,690 vertices FP64 14.5 ms (80 ms with 32 sources
+// every vertex a source 302 ms (1,340 ms with one 64-source batch on the whole
+// GPU and pushed counts); 13,690 vertices FP64 14.6 ms (80 ms with 32 sources
 // per CTA); 7,009 vertices plain 3.9 ms (21.5 ms with one source per CTA).
 #include <algorithm>
 #include <cstdio>
