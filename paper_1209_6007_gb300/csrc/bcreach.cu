@@ -680,22 +680,29 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   size_t small_limit = po.small_limit ? po.small_limit : SMALL_SMEM;
   bool mid_rule = !po.small_limit && lp_mode == LARGE_PATH_AUTO && !dbg && !po.per_source_large;
   if (tune && !po.small_limit) {
-    std::vector<CompDesc> elig;  // pieces that fit the largest limit
-    double cost = 0.0, band = 0.0;
+    double cost = 0.0, band = 0.0;  // of the pieces that fit the largest limit, and of those above the lowest
     const size_t lowest = SMALL_LIMITS[sizeof(SMALL_LIMITS) / sizeof(SMALL_LIMITS[0]) - 1];
+    auto fits_any = [&](const CompDesc &c, size_t *s1) {
+      if (c.n < 2 || nsrc_of(c) == 0 || !small_takes(c.n, c.nnz, 1)) return false;
+      *s1 = small_smem_bytes(c.n, c.nnz, 1, R, I);
+      return *s1 <= SMALL_SMEM;
+    };
     for (const CompDesc &c : comps) {
-      const int64_t ns = nsrc_of(c);
-      if (c.n < 2 || ns == 0 || c.n > 65535) continue;
-      const size_t s1 = small_smem_bytes(c.n, c.nnz, 1, R, I);
-      if (s1 > SMALL_SMEM || !small_takes(c.n, c.nnz, 1)) continue;
-      elig.push_back(c);
-      cost += (double)ns * (double)(c.nnz + c.n);
-      if (s1 > lowest) band += (double)ns * (double)(c.nnz + c.n);
+      size_t s1 = 0;
+      if (!fits_any(c, &s1)) continue;
+      const double work = (double)nsrc_of(c) * (double)(c.nnz + c.n);
+      cost += work;
+      if (s1 > lowest) band += work;
     }
     if (band > 0.0) {
       const long long key = ((long long)(R * 2 + I) << 40) | (bits_of(cost) << 20) | bits_of(band);
       int ch = tuned_in(g_tune_limit, key);
       if (!ch) {
+        std::vector<CompDesc> elig;
+        for (const CompDesc &c : comps) {
+          size_t s1 = 0;
+          if (fits_any(c, &s1)) elig.push_back(c);
+        }
         double best = 1e300;
         for (int k = 0; k < (int)(sizeof(SMALL_LIMITS) / sizeof(SMALL_LIMITS[0])); k++) {
           BcPlanOpts p2 = po;
@@ -721,6 +728,7 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
   std::vector<SmallItem> items;
   std::vector<LargeSrc> work;
   std::vector<int32_t> large, small;
+  small.reserve(C);
   int64_t nmax_large = 0, nmax_small = 0;
   double work_se = 0.0, work_sv = 0.0, total_small_cost = 0.0;
   std::vector<int32_t> mids;  // pieces of the small path that the pull kernel may take instead

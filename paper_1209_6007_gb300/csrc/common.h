@@ -359,8 +359,20 @@ struct SmallItem {
   int32_t s_end;
   int32_t ngroups;
 };
-size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident);
-bool small_takes(int64_t n, int64_t nnz, int G);
+__host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+// of a piece's rows, weights and codes, and of its pairs with G sources (inline:
+// the planner asks several times for each of tens of thousands of pieces)
+inline size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident) {
+  const size_t p = (size_t)n * G;
+  return align16((size_t)(n + 1) * 2) + align16((size_t)(nnz + 3) * 2) + (reach ? align16((size_t)n * 8) : 0) +
+         (ident ? align16((size_t)n * 4) : 0) + align16((size_t)n * 4) + align16(p * 8) * 2 + align16(p * 4) + align16(p * 2);
+}
+// 16-bit columns, row offsets and queue places
+inline bool small_takes(int64_t n, int64_t nnz, int G) {
+  int gs = 0;
+  while ((1 << gs) < G) gs++;
+  return n < 65536 && nnz < 65536 && (n << gs) <= 65536;
+}
 int small_max_sources();
 // the kernel's variants (small.cu) and the one for a launch: `coop` below,
 // sources in all, shared memory of a CTA

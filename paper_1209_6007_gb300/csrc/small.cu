@@ -54,23 +54,6 @@ __host__ __device__ constexpr int small_flush(bool global) { return global ? 64 
 constexpr int FIXED_COPIES = 32;  // of bc', in the fixed-scratch launch
 constexpr int SMALL_LEVELS = 64;  // level offsets kept in shared memory, the rest in global scratch
 
-__host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-
-// shared memory of a piece's rows, weights and codes, and of its pairs with G sources
-__host__ __device__ inline size_t small_piece_bytes(int64_t n, int64_t nnz, bool reach, bool ident) {
-  return align16((size_t)(n + 1) * 2) + align16((size_t)(nnz + 3) * 2) + (reach ? align16((size_t)n * 8) : 0) +
-         (ident ? align16((size_t)n * 4) : 0) + align16((size_t)n * 4);
-}
-size_t small_smem_bytes(int64_t n, int64_t nnz, int G, bool reach, bool ident) {
-  const size_t p = (size_t)n * G;
-  return small_piece_bytes(n, nnz, reach, ident) + align16(p * 8) * 2 + align16(p * 4) + align16(p * 2);
-}
-// 16-bit columns, row offsets and queue places
-bool small_takes(int64_t n, int64_t nnz, int G) {
-  int gs = 0;
-  while ((1 << gs) < G) gs++;
-  return n < 65536 && nnz < 65536 && (n << gs) <= 65536;
-}
 int small_max_sources() { return SMALL_MAX_G; }
 
 // SMALL_COOP: where a warp's pairs have at most SMALL_LONGS rows of more than 32
