@@ -25,6 +25,19 @@ def test_a_long_path(gpu, seed):
     assert min(ms) < 10.0
 
 
+def test_a_path_of_more_vertices_than_threads(gpu):
+    """As above where a kernel's grid of a fixed size has several vertices to a
+    thread (walking: 164 ms)."""
+    n = 2_000_000
+    g = gg.path(n)
+    ms = []
+    for _ in range(2):
+        got = gpu.bc_shattered(g.row_ptr, g.col, steps=gpu.STEP_D)
+        ms.append(gpu.last_stats()["ms_cc"])
+    assert np.array_equal(got, 2.0 * np.arange(n) * (n - 1 - np.arange(n)))
+    assert min(ms) < 10.0
+
+
 def test_rows_of_a_dense_graph(gpu):
     """200 vertices, all joined: the pieces' rows are written with a thread to a
     row, in less than twice the time of the merging stage (1.4; 2.4 with a warp to
