@@ -28,7 +28,7 @@ def layers(count, width, more, seed=2):
 def best(fn):
     fn()
     t = []
-    for _ in range(5):
+    for _ in range(9):
         t0 = time.perf_counter()
         fn()
         t.append(time.perf_counter() - t0)

@@ -20,7 +20,7 @@ def copies(g, count):
 def best(fn):
     fn()
     t = []
-    for _ in range(4):
+    for _ in range(9):
         t0 = time.perf_counter()
         fn()
         t.append(time.perf_counter() - t0)

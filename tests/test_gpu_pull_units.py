@@ -37,7 +37,7 @@ def test_units_of_every_size(gpu, monkeypatch, k):
 def best(fn):
     fn()
     t = []
-    for _ in range(5):
+    for _ in range(9):
         t0 = time.perf_counter()
         fn()
         t.append(time.perf_counter() - t0)

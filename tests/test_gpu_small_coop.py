@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 def small_ms(gpu, call):
     t = []
-    for _ in range(6):
+    for _ in range(14):
         call()
         t.append(gpu.last_stats()["ms_bcreach_small"])
     return min(t[1:])
