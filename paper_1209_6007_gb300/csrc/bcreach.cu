@@ -82,12 +82,13 @@ constexpr int64_t MID_MIN_ROWS = 1 << 15;
 // 9.7 ms, 18 on the deep one).  Above it the pull kernel is sooner (20,000
 // vertices of a power law, 300 sources, 1.4 ms and 2.4), if the graph is not
 // deep.  Of mean degree FEW_MEAN_DEG or less it may be a road, where more than
-// FEW_ROAD_SOURCES are worth the order (a square grid of 10,000: 400 sources
+// FEW_ROAD_SOURCES, or a graph above FEW_ROAD_MAX_N, are worth the order (24,600
+// vertices of a road, 1 source 2.3 ms, 2.8 without; a square grid of 10,000: 400 sources
 // 1.8 ms on the deep kernel, 2.8; 1 source 1.5 and 1.1; a power-law graph of 3,400
 // with pendants, 100 sources, 0.99 on the pull kernel, 0.64).  Above FEW_DENSE_DEG the
 // pull kernel cuts the rows, and is sooner (800 vertices of degree 100 in a few
 // levels, 1 source 0.48 ms and 0.58; 1,600 in 16 levels 0.86 and 1.02).
-constexpr int32_t FEW_MAX_N = 16384;
+constexpr int32_t FEW_MAX_N = 32768, FEW_ROAD_MAX_N = 16384;
 constexpr double FEW_US = 470.0;
 constexpr int64_t FEW_ROUNDS = 2, FEW_MEAN_DEG = 6, FEW_ROAD_SOURCES = 128, FEW_DENSE_DEG = 64;
 static double one_source_us(const CompDesc &c) { return 1.8e-3 * (double)c.nnz + 1.2 * c.maxdeg; }
@@ -802,10 +803,13 @@ int run_bcreach(Ctx &ctx, const std::vector<CompDesc> &comps_in, const BcInput &
     if (po.sources && lp_mode == LARGE_PATH_AUTO) {
       const CompDesc &c = comps[0];
       const int64_t wave = 3 * (int64_t)ctx.num_sms, rounds = (po.nsources + wave - 1) / wave;
-      const bool road = c.nnz <= FEW_MEAN_DEG * c.n, small_n = c.n < FEW_MAX_N && c.nnz <= FEW_DENSE_DEG * c.n;
+      const bool road = c.nnz <= FEW_MEAN_DEG * c.n;
+      const bool small_n = c.n < (road ? FEW_ROAD_MAX_N : FEW_MAX_N) && c.nnz <= FEW_DENSE_DEG * c.n;
       cheap = rounds <= FEW_ROUNDS && rounds * one_source_us(c) < FEW_US;
       no_search = small_n && cheap && (po.nsources <= FEW_ROAD_SOURCES || !road);
       if (rounds <= 1) end = small_n && !road ? FEW_END : FEW_NARROW_END;
+      // deeper than the pull kernel takes, and a row too long for the deep one
+      if (c.maxdeg > DEEP_MAX_DEG && end.levels > PULL_MAX_ECC + 2) end = PieceBfsEnd{PULL_MAX_ECC + 2, INT32_MAX};
     }
     for (int32_t ci : large) {
       const CompDesc &c = comps[ci];

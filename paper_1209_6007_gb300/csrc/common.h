@@ -408,6 +408,7 @@ size_t pull_piece_bytes(int64_t n, int64_t nnz, int depth_bound);
 int run_deep(Ctx &ctx, const CompDesc &c, const BcInput &in, bool fp32, const int32_t *d_bfs, const int32_t *d_parent,
              const int32_t *d_sources, int32_t nsrc, int depth_bound, int *d_err, unsigned long long *d_dag);
 bool deep_takes(const CompDesc &c, int depth_bound, size_t free_bytes);
+constexpr int DEEP_MAX_DEG = 64;  // a row is one thread's work
 // BFS of each listed piece from its first vertex, one piece per CTA: the
 // vertices in the order reached at order[ord_off[i] ..), their tree parents
 // (-1: the root) at parent[ord_off[i] ..), the deepest level and the number

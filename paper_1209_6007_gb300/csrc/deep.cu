@@ -55,7 +55,6 @@ constexpr int DEEP_THREADS = 512;
 constexpr int DEEP_CTAS = 3;    // per SM
 constexpr int DEEP_MAX_G = 16;  // sources per CTA
 constexpr int DEEP_RING = 1024; // queue places of a level kept in shared memory
-constexpr int DEEP_MAX_DEG = 64;  // a row is one thread's work
 constexpr size_t DEEP_BYTES = (size_t)32 << 30;  // state of all CTAs
 constexpr size_t DEEP_SMEM = 54 * 1024;  // codes in shared memory, per CTA (three to an SM, with L1 left)
 constexpr int DEEP_PER_COPY = 48;  // sources to a copy of bc'

@@ -36,7 +36,8 @@ def best(fn):
 
 
 @pytest.mark.parametrize("g,k", [(layers(38, 400, 5), 32), (layers(38, 150, 5), 300), (gg.cycle(6000), 1),
-                                 (gg.cycle(6000), 32), (gg.path(20000), 30), (gg.grid(100, 100), 1)],
+                                 (gg.cycle(6000), 32), (gg.path(20000), 30), (gg.grid(100, 100), 1),
+                                 (layers(60, 300, 20), 1)],
                          ids=lambda x: getattr(x, "name", str(x)))
 def test_no_slower_than_one_source_per_cta(gpu, monkeypatch, g, k):
     src = np.random.default_rng(k).choice(g.n, k, replace=False)
